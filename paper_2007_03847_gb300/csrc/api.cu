@@ -783,7 +783,7 @@ int fmc_lhs_sample_split(fmc_ctx* ctx, uint64_t seed, int64_t N, int64_t k0, int
     if (mode < 0 || mode > 2) return fail(ctx, FMC_EINVAL, "mode %d", mode);
     if (!hi_dev) return fail(ctx, FMC_EINVAL, "hi output is NULL");
     cudaStream_t st = (cudaStream_t)stream;
-    FMC_CUDA(ctx, launch_lhs_split(seed, N, k0, count, d, K, mode, hi_dev, lo_dev, ctx->sms, st), "lhs kernel");
+    FMC_CUDA(ctx, launch_lhs_split(seed, N, k0, count, d, K, mode, nullptr, hi_dev, lo_dev, ctx->sms, st), "lhs kernel");
     return FMC_OK;
 }
 
@@ -843,7 +843,7 @@ int fmc_lhs_decorrelate(fmc_ctx* ctx, uint64_t seed, int64_t N, int32_t M, int32
     int rc = run_decorrelate(ctx, ctx->ws, seed, N, M, st);
     if (rc) return rc;
     const uint32_t* strata = (const uint32_t*)ctx->ws.ic_strata.ptr;
-    if (zeta_dev) FMC_CUDA(ctx, launch_ic_values(seed, N, 0, N, M, mode, strata, zeta_dev, ctx->sms, st), "values");
+    if (zeta_dev) FMC_CUDA(ctx, launch_strata_values(seed, N, 0, N, M, mode, strata, zeta_dev, ctx->sms, st), "values");
     if (strata_dev)
         FMC_CUDA(ctx, cudaMemcpyAsync(strata_dev, strata, (size_t)N * M * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st),
                  "copy");
@@ -1420,7 +1420,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             prof_begin(ctx, PH_LHS, st, &pr);
             FMC_CUDA(ctx,
                      s->correlation == FMC_CORR_RANK
-                         ? launch_ic_values(s->seed, N, k0, count, M, s->sampling, (const uint32_t*)ws.ic_strata.ptr,
+                         ? launch_strata_values(s->seed, N, k0, count, M, s->sampling, (const uint32_t*)ws.ic_strata.ptr,
                                             (float*)ws.zeta32.ptr, ctx->sms, st)
                          : launch_lhs_f32(s->seed, N, k0, count, M, s->sampling, (float*)ws.zeta32.ptr, nullptr,
                                           ctx->sms, st),
@@ -1479,17 +1479,14 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             const size_t rb = (size_t)per * d * Ks * 2;  // bytes of one design (BF16 rows of d Ks)
             for (int k = 0; k < R; ++k)
                 FMC_CUDA(ctx,
-                         launch_lhs_split(seeds[k], per, 0, per, d, K, s->sampling, (char*)ws.zeta_hi.ptr + k * rb,
+                         launch_lhs_split(seeds[k], per, 0, per, d, K, s->sampling, nullptr, (char*)ws.zeta_hi.ptr + k * rb,
                                           split ? (char*)ws.zeta_lo.ptr + k * rb : nullptr, ctx->sms, st),
                          "lhs kernel");
         } else {
             FMC_CUDA(ctx,
-                     s->correlation == FMC_CORR_RANK
-                         ? launch_ic_split(s->seed, N, k0, count, d, K, s->sampling,
-                                           (const uint32_t*)ws.ic_strata.ptr, ws.zeta_hi.ptr,
-                                           split ? ws.zeta_lo.ptr : nullptr, ctx->sms, st)
-                         : launch_lhs_split(s->seed, N, k0, count, d, K, s->sampling, ws.zeta_hi.ptr,
-                                            split ? ws.zeta_lo.ptr : nullptr, ctx->sms, st),
+                     launch_lhs_split(s->seed, N, k0, count, d, K, s->sampling,
+                                      s->correlation == FMC_CORR_RANK ? (const uint32_t*)ws.ic_strata.ptr : nullptr,
+                                      ws.zeta_hi.ptr, split ? ws.zeta_lo.ptr : nullptr, ctx->sms, st),
                      "lhs kernel");
         }
         prof_end(pr, st);

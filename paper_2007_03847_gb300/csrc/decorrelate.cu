@@ -13,13 +13,10 @@
 // Cholesky factorisation and triangular inverse in FP32 (T is within O(1/sqrt N)
 // of the identity), R* by the FP32 GEMM, the per-column ranks by a segmented
 // radix sort (CUB), and the design values from the new strata.
-#include <cuda_bf16.h>
-
 #include <cub/device/device_segmented_radix_sort.cuh>
 
 #include "fmc_common.cuh"
 #include "kernels.cuh"
-#include "lhs_feistel.cuh"
 
 namespace fmc {
 
@@ -66,20 +63,6 @@ __global__ void ic_score_moments_kernel(uint32_t N, const double* __restrict__ a
     if (threadIdx.x == 0) {
         out[0] = mean;
         out[1] = red[0];
-    }
-}
-
-// R[k][i] = a(pi_i(k)) - mean, FP32, row-major [N][M]
-__global__ void ic_scores_kernel(uint32_t k0s, uint32_t k1s, uint32_t N, int M, int h, uint32_t mask,
-                                 const double* __restrict__ a, const double* __restrict__ mom, float* __restrict__ R)
-{
-    const int64_t total = (int64_t)N * M;
-    const double mean = mom[0];
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = t / M;
-        const int i = (int)(t - k * M);
-        const uint32_t s = stratum((uint32_t)k, (uint32_t)i, N, h, mask, k0s, k1s);
-        R[t] = (float)(a[s] - mean);
     }
 }
 
@@ -235,57 +218,6 @@ __global__ void ic_segments_kernel(int M, int64_t N, int* __restrict__ off)
     if (i <= M) off[i] = (int)((int64_t)i * N);
 }
 
-// The design values of given strata [M][N]: zeta = Phi^-1((s + u) / N) with the
-// sample's own uniform u (LHS) or u = 1/2 (midpoint), as the plain design does.
-__device__ __forceinline__ float ic_value(uint32_t k, uint32_t i, uint32_t s, uint32_t N, int mode, uint32_t k0s,
-                                          uint32_t k1s)
-{
-    uint64_t num2;
-    if (mode == FMC_LHS_MIDPOINT) {
-        num2 = ((uint64_t)s << 33) + (1ull << 32);
-    } else {
-        const uint32_t r = philox4x32_10(U4{k, i, 0u, 0u}, k0s, k1s).x;
-        num2 = ((uint64_t)s << 33) + 2ull * r + 1ull;
-    }
-    return normal_from_fraction(num2, N);
-}
-
-// rows k0 .. k0+count-1: zeta [count][M] FP32
-__global__ void ic_values_kernel(uint32_t k0s, uint32_t k1s, uint32_t N, int64_t k0, int64_t count, int M, int mode,
-                                 const uint32_t* __restrict__ strata, float* __restrict__ zeta)
-{
-    const int64_t total = count * M;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = t / M;
-        const int i = (int)(t - j * M);
-        const int64_t k = k0 + j;
-        zeta[t] = ic_value((uint32_t)k, (uint32_t)i, strata[(int64_t)i * N + k], N, mode, k0s, k1s);
-    }
-}
-
-// rows k0 .. k0+count-1 in the split-BF16 layout [count][d][Ks] of the fused path
-__global__ void ic_split_kernel(uint32_t k0s, uint32_t k1s, uint32_t N, int64_t k0, int64_t count, int d, int K, int Ks,
-                                int mode, const uint32_t* __restrict__ strata, __nv_bfloat16* __restrict__ hi,
-                                __nv_bfloat16* __restrict__ lo)
-{
-    const int64_t row = (int64_t)d * Ks;
-    const int64_t total = count * row;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = t / row;
-        const int rem = (int)(t - j * row);
-        const int w = rem / Ks, kk = rem - w * Ks;
-        float z = 0.f;
-        if (kk < K) {
-            const uint32_t i = (uint32_t)(w * K + kk);
-            const int64_t k = k0 + j;
-            z = ic_value((uint32_t)k, i, strata[(int64_t)i * N + k], N, mode, k0s, k1s);
-        }
-        const __nv_bfloat16 zh = __float2bfloat16_rn(z);
-        hi[t] = zh;
-        if (lo) lo[t] = __float2bfloat16_rn(z - __bfloat162float(zh));
-    }
-}
-
 static int ic_grid(int64_t total, int block, int sms)
 {
     int64_t g = (total + block - 1) / block;
@@ -306,14 +238,12 @@ cudaError_t launch_ic_strata(uint64_t seed, int64_t N, int M, const IcWork& w, u
                              cudaStream_t st)
 {
     if (M > IC_MAX_M || N < 2 || N > 2147483647LL || (int64_t)N * M > 2147483647LL) return cudaErrorInvalidValue;
-    const FeistelShape f = feistel_shape(N);
-    const uint32_t k0s = (uint32_t)seed, k1s = (uint32_t)(seed >> 32);
     const int64_t NM = N * (int64_t)M;
     cudaError_t e;
     ic_score_table_kernel<<<ic_grid(N, 256, sms), 256, 0, st>>>((uint32_t)N, w.a);
     ic_score_moments_kernel<<<1, 1024, 0, st>>>((uint32_t)N, w.a, w.mom);
-    ic_scores_kernel<<<ic_grid(NM, 256, sms), 256, 0, st>>>(k0s, k1s, (uint32_t)N, M, f.h, f.mask, w.a, w.mom, w.R);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_design_scores(seed, N, M, w.a, w.mom, w.R, sms, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(w.G, 0, sizeof(double) * (size_t)M * M, st)) != cudaSuccess) return e;
     const int tiles = (M + IC_GT - 1) / IC_GT;
     const int64_t slices = (N + IC_GRAM_ROWS - 1) / IC_GRAM_ROWS;
@@ -335,26 +265,6 @@ cudaError_t launch_ic_strata(uint64_t seed, int64_t N, int M, const IcWork& w, u
                                                       w.off, w.off + 1, 0, 32, st)) != cudaSuccess)
         return e;
     ic_ranks_kernel<<<ic_grid(NM, 256, sms), 256, 0, st>>>(N, M, w.vals_out, strata);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ic_values(uint64_t seed, int64_t N, int64_t k0, int64_t count, int M, int mode,
-                             const uint32_t* strata, float* zeta, int sms, cudaStream_t st)
-{
-    if (count == 0) return cudaSuccess;
-    ic_values_kernel<<<ic_grid(count * M, 256, sms), 256, 0, st>>>((uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)N,
-                                                                   k0, count, M, mode, strata, zeta);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ic_split(uint64_t seed, int64_t N, int64_t k0, int64_t count, int d, int K, int mode,
-                            const uint32_t* strata, void* hi, void* lo, int sms, cudaStream_t st)
-{
-    if (count == 0) return cudaSuccess;
-    const int Ks = round_up(K, 8);
-    ic_split_kernel<<<ic_grid(count * d * Ks, 256, sms), 256, 0, st>>>(
-        (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)N, k0, count, d, K, Ks, mode, strata,
-        (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
     return cudaGetLastError();
 }
 

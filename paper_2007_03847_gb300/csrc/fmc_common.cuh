@@ -49,22 +49,27 @@ __host__ __device__ __forceinline__ U4 philox4x32_10(U4 c, uint32_t k0, uint32_t
 // differences so that it carries FP32 relative accuracy in both tails and at
 // the centre:  Phi^-1(p) = -sqrt2 erfcinv(2p) = sqrt2 erfinv(2p - 1)
 //            = sqrt2 erfcinv(2(1-p)).
-__device__ __forceinline__ float normal_from_fraction(uint64_t num2, uint32_t N)
+// A warp's lanes fall on both sides of the branch between the two functions, so
+// everything else (the 64-bit conversion, the division) is done once before it.
+// rcp: 2^-32 / N where N is a power of two (the product is then the exact
+// quotient, scaled), else 0.
+__device__ __forceinline__ float normal_from_fraction(uint64_t num2, uint32_t N, float rcp)
 {
     const uint64_t half = (uint64_t)N << 32;   // den/2
     const float fhalf = (float)N * 4294967296.0f;
     const float SQRT2 = 1.41421356237309515f;
-    if (num2 <= (half >> 1)) {                  // p <= 1/4
-        float twop = (float)num2 / fhalf;
-        return -SQRT2 * erfcinvf(twop);
+    const uint64_t den = half << 1;
+    const bool low = num2 <= (half >> 1);           // p <= 1/4
+    const bool high = num2 >= den - (half >> 1);    // p >= 3/4
+    const bool neg = num2 < half;
+    const uint64_t v = low ? num2 : (high ? den - num2 : (neg ? half - num2 : num2 - half));
+    const float f = (float)v;
+    const float x = rcp != 0.f ? f * rcp : f / fhalf;
+    if (low || high) {
+        const float z = SQRT2 * erfcinvf(x);
+        return low ? -z : z;
     }
-    uint64_t den = half << 1;
-    if (num2 >= den - (half >> 1)) {            // p >= 3/4
-        float twoq = (float)(den - num2) / fhalf;
-        return SQRT2 * erfcinvf(twoq);
-    }
-    int64_t c = (int64_t)(num2 - half);         // 2p - 1 = c / half
-    return SQRT2 * erfinvf((float)c / fhalf);
+    return SQRT2 * erfinvf(neg ? -x : x);  // 2p - 1 = (num2 - half) / half
 }
 
 // The normal of (sample k, disturbance w, step n) of the per-step-normal Monte
@@ -76,7 +81,7 @@ __device__ __forceinline__ float em_normal(uint32_t k, int w, int n, uint32_t k0
 {
     const U4 o = philox4x32_10(U4{k, (uint32_t)n, EM_TAG, (uint32_t)(w >> 2)}, k0, k1);
     const uint32_t r = (w & 3) == 0 ? o.x : ((w & 3) == 1 ? o.y : ((w & 3) == 2 ? o.z : o.w));
-    return normal_from_fraction(2ull * r + 1ull, 1u);
+    return normal_from_fraction(2ull * r + 1ull, 1u, 0x1p-32f);
 }
 
 // Packed FP32 (two lanes per register pair) fused multiply-add of sm_100+:

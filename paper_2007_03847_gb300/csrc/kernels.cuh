@@ -32,8 +32,14 @@ struct EmSpec {
 
 cudaError_t launch_lhs_f32(uint64_t seed, int64_t N, int64_t k0, int64_t count, int M, int mode, float* zeta,
                            uint32_t* strata, int sms, cudaStream_t st);
-cudaError_t launch_lhs_split(uint64_t seed, int64_t N, int64_t k0, int64_t count, int d, int K, int mode, void* hi,
-                             void* lo, int sms, cudaStream_t st);
+// strata: null, or the strata [d K][N] to take instead of the design's own
+cudaError_t launch_lhs_split(uint64_t seed, int64_t N, int64_t k0, int64_t count, int d, int K, int mode,
+                             const uint32_t* strata, void* hi, void* lo, int sms, cudaStream_t st);
+// values [count][M] of given strata [M][N], and the scores R[k][i] = score[pi_i(k)] - *mean [N][M]
+cudaError_t launch_strata_values(uint64_t seed, int64_t N, int64_t k0, int64_t count, int M, int mode,
+                                 const uint32_t* strata, float* zeta, int sms, cudaStream_t st);
+cudaError_t launch_design_scores(uint64_t seed, int64_t N, int M, const double* score, const double* mean, float* R,
+                                 int sms, cudaStream_t st);
 cudaError_t launch_em_increments(uint64_t seed, int64_t k0, int64_t count, int d, int Nt, double dt, float* dW,
                                  int sms, cudaStream_t st);
 cudaError_t launch_basis_f32(int K, int Nt, double T, int basis, float* phi, int sms, cudaStream_t st);
@@ -156,12 +162,6 @@ size_t ic_sort_bytes(int64_t N, int M);
 // strata [M][N] of the decorrelated design (M <= 4096, N*M < 2^31)
 cudaError_t launch_ic_strata(uint64_t seed, int64_t N, int M, const IcWork& w, uint32_t* strata, int sms,
                              cudaStream_t st);
-// design values of rows k0..k0+count-1 from strata [M][N]: zeta [count][M] FP32,
-// or the split-BF16 layout [count][d][round_up(K, 8)]
-cudaError_t launch_ic_values(uint64_t seed, int64_t N, int64_t k0, int64_t count, int M, int mode,
-                             const uint32_t* strata, float* zeta, int sms, cudaStream_t st);
-cudaError_t launch_ic_split(uint64_t seed, int64_t N, int64_t k0, int64_t count, int d, int K, int mode,
-                            const uint32_t* strata, void* hi, void* lo, int sms, cudaStream_t st);
 
 // The Appendix's identification: the objective L' of a record xi [n] (FP64)
 // for the coefficients q (kind 1: sigma polynomial; kind 2: sigma^2

@@ -1,7 +1,7 @@
 // Algorithm 1 step 1 / Section IV-B: Latin hypercube sampling of the M = d*K
-// KL coefficients on the GPU.  One thread per (sample, dimension); the design is
-// stateless (a keyed Feistel permutation per dimension), so any sub-range of the
-// N rows is produced bit-identically without sorting or communication.
+// KL coefficients on the GPU.  The design is stateless (a keyed Feistel
+// permutation per dimension), so any sub-range of the N rows is produced
+// bit-identically without sorting or communication.
 #include <cuda_bf16.h>
 
 #include "fmc_common.cuh"
@@ -10,64 +10,274 @@
 
 namespace fmc {
 
-__device__ __forceinline__ float lhs_value(uint32_t k, uint32_t dim, uint32_t N, int mode, int h, uint32_t mask,
-                                           uint32_t k0, uint32_t k1, uint32_t* s_out)
+constexpr int DESIGN_SMEM_MAX = 224 * 1024;
+
+// ---------------------------------------------------------------------------
+// design_kernel: the design's values of a tile of positions x samples.
+//
+// What bounds it: integer issue.  Computed from its definition, an entry costs
+// seven Philox calls (six Feistel rounds and the uniform), and a domain 4^h above
+// N repeats the six until the value falls below N (cycle walking).  But a round
+// function takes its argument from h bits only, so per dimension it has 2^h
+// values: a CTA tabulates the 6 x 2^h of its dimensions in shared memory (the
+// masked Philox words, so the permutation is the same bit for bit) and a round
+// becomes one lookup.  Tables pay from about 2^h rows per CTA on; the tile takes
+// up to 16 x 2^h.
+//
+// Layout: a thread keeps one position (column) and steps over rows, with DB
+// neighbouring positions in neighbouring lanes, so that a row's outputs go out as
+// whole 32-byte sectors and no index division is left in the loop.  Strata go
+// through a short per-thread list in shared memory: walking lanes take their next
+// row as soon as their value is found instead of waiting for the warp's longest
+// walk, and the list is read transposed where strata themselves are stored or
+// loaded (their rows run along the samples).
+//
+// Measured (GB300): 65536 x 600 values and strata 735 -> 355 us (entries computed
+// one by one from the definition before; 0.9 TB/s of output, the uniform's Philox
+// call and the two branches of the inverse CDF now take the issue slots); the
+// split-BF16 rows of 19001 x 2400 (domain 4^8, 3.4 walks per entry) 6.99 -> 0.70 ms.
+// ---------------------------------------------------------------------------
+enum { PERM_NONE = 0, PERM_DIRECT, PERM_TAB8, PERM_TAB16, PERM_GIVEN };
+enum { OUT_F32 = 0, OUT_SPLIT, OUT_SCORE };
+
+template <int PERM>
+struct DesignTile {
+    static constexpr int THREADS = PERM == PERM_TAB16 ? 512 : 256;
+    static constexpr int DB = PERM == PERM_TAB16 ? 8 : 16;   // positions per CTA
+    static constexpr int RPI = THREADS / DB;                 // rows per pass of the CTA
+    static constexpr int LCAP = PERM == PERM_TAB16 ? 4 : 16; // list entries per thread
+    static constexpr int SUB = RPI * LCAP;                   // rows per list filling
+    static constexpr int LIST_BYTES = SUB * (DB + 1) * 4;
+};
+
+struct DesignArgs {
+    uint32_t k0s, k1s, N;
+    int64_t k0, count;
+    int cols;          // positions per row: M, or d Ks with K..Ks-1 of every group zero
+    int K, Ks;         // OUT_SPLIT
+    int mode, h;
+    uint32_t mask;
+    float rcp;         // see normal_from_fraction
+    int walk;          // N < 4^h
+    int npos;          // position blocks
+    int64_t rows;      // rows per CTA
+    float* zeta;       // OUT_F32 / OUT_SCORE [count][cols], may be null (strata only)
+    __nv_bfloat16 *hi, *lo;
+    uint32_t* strata;            // [M][count] out, or null
+    const uint32_t* strata_in;   // PERM_GIVEN: [M][N]
+    const double *score, *mean;  // OUT_SCORE: a(s) and its mean
+};
+
+template <int PERM>
+__device__ __forceinline__ uint32_t feistel_round(const void* tab, uint32_t R, int r, const DesignArgs& a, uint32_t dim)
 {
-    if (mode == FMC_SRS) {
-        uint32_t r = philox4x32_10(U4{k, dim, 0u, 0u}, k0, k1).x;
-        *s_out = k;
-        return normal_from_fraction(2ull * r + 1ull, 1u);
-    }
-    uint32_t s = stratum(k, dim, N, h, mask, k0, k1);
-    *s_out = s;
-    uint64_t num2;
-    if (mode == FMC_LHS_MIDPOINT) {
-        num2 = ((uint64_t)s << 33) + (1ull << 32);
-    } else {
-        uint32_t r = philox4x32_10(U4{k, dim, 0u, 0u}, k0, k1).x;
-        num2 = ((uint64_t)s << 33) + 2ull * r + 1ull;
-    }
-    return normal_from_fraction(num2, N);
+    if constexpr (PERM == PERM_TAB8)
+        return static_cast<const uint8_t*>(tab)[((uint32_t)r << a.h) + R];
+    else if constexpr (PERM == PERM_TAB16)
+        return static_cast<const uint16_t*>(tab)[((uint32_t)r << a.h) + R];
+    else
+        return philox4x32_10(U4{R, dim, 1u + (uint32_t)r, 0u}, a.k0s, a.k1s).x & a.mask;
 }
 
-__global__ void lhs_f32_kernel(uint32_t k0s, uint32_t k1s, uint32_t N, int64_t k0, int64_t count, int M, int mode,
-                               int h, uint32_t mask, float* __restrict__ zeta, uint32_t* __restrict__ strata)
+// One application of the Feistel network (feistel() of lhs_feistel.cuh).
+template <int PERM>
+__device__ __forceinline__ uint32_t permute(const void* tab, uint32_t x, const DesignArgs& a, uint32_t dim)
 {
-    int64_t total = count * (int64_t)M;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t j = t / M;
-        int i = (int)(t - j * M);
-        uint32_t s;
-        float z = lhs_value((uint32_t)(k0 + j), (uint32_t)i, N, mode, h, mask, k0s, k1s, &s);
-        if (zeta) zeta[t] = z;
-        if (strata) strata[(int64_t)i * count + j] = s;
+    uint32_t L = (x >> a.h) & a.mask, R = x & a.mask;
+#pragma unroll
+    for (int r = 0; r < kFeistelRounds; ++r) {
+        const uint32_t n = L ^ feistel_round<PERM>(tab, R, r, a, dim);
+        L = R;
+        R = n;
     }
+    return (L << a.h) | R;
 }
 
-// Split-BF16 layout for the tensor-core contraction: [count][d][Ks] with zeros
-// in the K..Ks-1 padding of every group.
-__global__ void lhs_split_kernel(uint32_t k0s, uint32_t k1s, uint32_t N, int64_t k0, int64_t count, int d, int K,
-                                 int Ks, int mode, int h, uint32_t mask, __nv_bfloat16* __restrict__ hi,
-                                 __nv_bfloat16* __restrict__ lo)
+template <int PERM, int OUT>
+__global__ void __launch_bounds__(DesignTile<PERM>::THREADS) design_kernel(const DesignArgs a)
 {
-    int64_t row = (int64_t)d * Ks;
-    int64_t total = count * row;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t j = t / row;
-        int rem = (int)(t - j * row);
-        int w = rem / Ks;
-        int kk = rem - w * Ks;
-        float z = 0.f;
-        if (kk < K) {
-            uint32_t s;
-            z = lhs_value((uint32_t)(k0 + j), (uint32_t)(w * K + kk), N, mode, h, mask, k0s, k1s, &s);
+    using T = DesignTile<PERM>;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    uint32_t* list = reinterpret_cast<uint32_t*>(dsm);
+    unsigned char* tabs = dsm + T::LIST_BYTES;
+    const int tid = threadIdx.x;
+    const int dc = tid % T::DB, q = tid / T::DB;
+    const int pb = (int)(blockIdx.x % (unsigned)a.npos);
+    const int64_t j0 = (int64_t)(blockIdx.x / (unsigned)a.npos) * a.rows;
+    const int64_t j1 = j0 + a.rows < a.count ? j0 + a.rows : a.count;
+    const int pos = pb * T::DB + dc;
+    // the dimension of this thread's position (split rows: groups of Ks, K of them real)
+    uint32_t dim = (uint32_t)pos;
+    bool real = pos < a.cols;
+    if (OUT == OUT_SPLIT) {
+        const int w = pos / a.Ks, kk = pos - w * a.Ks;
+        dim = (uint32_t)(w * a.K + kk);
+        real = real && kk < a.K;
+    }
+    const void* tab = nullptr;
+    if constexpr (PERM == PERM_TAB8 || PERM == PERM_TAB16) {
+        // the CTA's tables: [DB][6][2^h]
+        constexpr int EB = PERM == PERM_TAB8 ? 1 : 2;
+        const int per = kFeistelRounds << a.h;
+        for (int e = q; e < per; e += T::RPI) {
+            uint32_t v = 0;
+            if (real)
+                v = philox4x32_10(U4{(uint32_t)e & a.mask, dim, 1u + ((uint32_t)e >> a.h), 0u}, a.k0s, a.k1s).x & a.mask;
+            if (EB == 1)
+                tabs[dc * per + e] = (uint8_t)v;
+            else
+                reinterpret_cast<uint16_t*>(tabs)[dc * per + e] = (uint16_t)v;
         }
-        __nv_bfloat16 zh = __float2bfloat16_rn(z);
-        hi[t] = zh;
-        if (lo) lo[t] = __float2bfloat16_rn(z - __bfloat162float(zh));
+        __syncthreads();
+        tab = tabs + (size_t)dc * per * EB;
     }
+    for (int64_t jb = j0; jb < j1; jb += T::SUB) {
+        const int nrow = j1 - jb < T::SUB ? (int)(j1 - jb) : T::SUB;  // rows of this filling
+        const int mine = q < nrow ? (nrow - q + T::RPI - 1) / T::RPI : 0;
+        uint32_t* my = list + q * (T::DB + 1) + dc;  // entry i at my[i * RPI * (DB + 1)]
+        constexpr int LS = T::RPI * (T::DB + 1);
+        const uint32_t kb = (uint32_t)(a.k0 + jb) + (uint32_t)q;
+        if constexpr (PERM == PERM_GIVEN) {
+            // strata_in rows run along the samples: read them so, transposed into the list
+            __syncthreads();
+            for (int e = tid; e < T::DB * T::SUB; e += T::THREADS) {
+                const int c = e / T::SUB, row = e % T::SUB;
+                const int p2 = pb * T::DB + c;
+                uint32_t dim2 = (uint32_t)p2;
+                bool real2 = p2 < a.cols;
+                if (OUT == OUT_SPLIT) {
+                    const int w = p2 / a.Ks, kk = p2 - w * a.Ks;
+                    dim2 = (uint32_t)(w * a.K + kk);
+                    real2 = real2 && kk < a.K;
+                }
+                if (real2 && row < nrow)
+                    list[row * (T::DB + 1) + c] = a.strata_in[(int64_t)dim2 * a.N + a.k0 + jb + row];
+            }
+            __syncthreads();
+        } else if constexpr (PERM != PERM_NONE) {
+            if (a.walk) {
+                int i = 0;
+                uint32_t y = kb;
+                while (real && i < mine) {
+                    y = permute<PERM>(tab, y, a, dim);
+                    if (y < a.N) {
+                        my[i * LS] = y;
+                        ++i;
+                        y = kb + (uint32_t)(i * T::RPI);
+                    }
+                }
+            } else if (real) {
+#pragma unroll 2
+                for (int i = 0; i < mine; ++i) my[i * LS] = permute<PERM>(tab, kb + (uint32_t)(i * T::RPI), a, dim);
+            }
+        } else if (a.strata) {
+            for (int i = 0; i < mine; ++i) my[i * LS] = kb + (uint32_t)(i * T::RPI);  // (no permutation: s = k)
+        }
+        if (pos < a.cols && (OUT != OUT_F32 || a.zeta)) {
+#pragma unroll 2
+            for (int i = 0; i < mine; ++i) {
+                const uint32_t k = kb + (uint32_t)(i * T::RPI);
+                const int64_t o = (jb + q + i * T::RPI) * a.cols + pos;
+                if constexpr (OUT == OUT_SCORE) {
+                    a.zeta[o] = (float)(a.score[my[i * LS]] - *a.mean);
+                } else {
+                    float z = 0.f;
+                    if (real) {
+                        if (PERM == PERM_NONE) {
+                            const uint32_t r = philox4x32_10(U4{k, dim, 0u, 0u}, a.k0s, a.k1s).x;
+                            z = normal_from_fraction(2ull * r + 1ull, 1u, 0x1p-32f);
+                        } else {
+                            const uint32_t s = my[i * LS];
+                            uint64_t num2 = ((uint64_t)s << 33) + (1ull << 32);
+                            if (a.mode != FMC_LHS_MIDPOINT) {
+                                const uint32_t r = philox4x32_10(U4{k, dim, 0u, 0u}, a.k0s, a.k1s).x;
+                                num2 = ((uint64_t)s << 33) + 2ull * r + 1ull;
+                            }
+                            z = normal_from_fraction(num2, a.N, a.rcp);
+                        }
+                    }
+                    if constexpr (OUT == OUT_F32) {
+                        a.zeta[o] = z;
+                    } else {
+                        const __nv_bfloat16 zh = __float2bfloat16_rn(z);
+                        a.hi[o] = zh;
+                        if (a.lo) a.lo[o] = __float2bfloat16_rn(z - __bfloat162float(zh));
+                    }
+                }
+            }
+        }
+        if (OUT == OUT_F32 && a.strata) {
+            __syncthreads();
+            for (int e = tid; e < T::DB * T::SUB; e += T::THREADS) {
+                const int c = e / T::SUB, row = e % T::SUB;
+                const int p2 = pb * T::DB + c;
+                if (p2 < a.cols && row < nrow) a.strata[(int64_t)p2 * a.count + jb + row] = list[row * (T::DB + 1) + c];
+            }
+            __syncthreads();
+        }
+    }
+}
+
+template <int PERM, int OUT>
+static cudaError_t launch_design_t(DesignArgs& a, int sms, cudaStream_t st)
+{
+    using T = DesignTile<PERM>;
+    constexpr bool TAB = PERM == PERM_TAB8 || PERM == PERM_TAB16;
+    a.npos = (a.cols + T::DB - 1) / T::DB;
+    // rows per CTA: four CTAs per SM in all, but 2 .. 16 rows per table entry where
+    // there are tables (their filling is at most three Philox calls per entry, at
+    // most 3/8 for large designs), and whole list fillings (whole passes below one)
+    int64_t rows = (a.count * a.npos + 4 * sms - 1) / (4 * (int64_t)sms);
+    const int64_t lo = TAB ? (int64_t)2 << a.h : 1, hi = TAB ? (int64_t)16 << a.h : (int64_t)1 << 14;
+    rows = rows < lo ? lo : (rows > hi ? hi : rows);
+    const int64_t unit = rows < T::SUB ? T::RPI : T::SUB;
+    rows = (rows + unit - 1) / unit * unit;
+    while ((a.count + rows - 1) / rows * a.npos > 2147483647LL) rows *= 2;
+    a.rows = rows;
+    const int smem = T::LIST_BYTES + (TAB ? T::DB * (kFeistelRounds << a.h) * (PERM == PERM_TAB8 ? 1 : 2) : 0);
+    auto kern = design_kernel<PERM, OUT>;
+    if (smem > 48 * 1024) {
+        // process-wide attribute: always the same bound (launches may race on it)
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DESIGN_SMEM_MAX);
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t grid = (a.count + rows - 1) / rows * a.npos;
+    kern<<<(unsigned)grid, T::THREADS, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+// The rule: tables while they fit (uint8 up to h = 8, 24 KB; uint16 up to h = 11,
+// 192 KB) and a block of rows at least 2^(h+1) long repays them; the rounds from
+// their definition above (more than 2^22 samples) and for short blocks of a large
+// design; no permutation for simple random sampling.
+template <int OUT>
+static cudaError_t launch_design(DesignArgs& a, int sms, cudaStream_t st)
+{
+    if (a.count == 0) return cudaSuccess;
+    a.walk = a.h < 16 && ((uint64_t)1 << (2 * a.h)) > a.N;
+    if (a.strata_in) return launch_design_t<PERM_GIVEN, OUT>(a, sms, st);
+    if (a.mode == FMC_SRS) return launch_design_t<PERM_NONE, OUT>(a, sms, st);
+    const bool rows_enough = a.count >= ((int64_t)2 << a.h);
+    if (a.h <= 8 && rows_enough) return launch_design_t<PERM_TAB8, OUT>(a, sms, st);
+    if (a.h <= 11 && rows_enough) return launch_design_t<PERM_TAB16, OUT>(a, sms, st);
+    return launch_design_t<PERM_DIRECT, OUT>(a, sms, st);
+}
+
+static DesignArgs design_args(uint64_t seed, int64_t N, int64_t k0, int64_t count, int cols, int mode)
+{
+    const FeistelShape f = feistel_shape(N);
+    DesignArgs a{};
+    a.k0s = (uint32_t)seed;
+    a.k1s = (uint32_t)(seed >> 32);
+    a.N = (uint32_t)N;
+    a.k0 = k0;
+    a.count = count;
+    a.cols = cols;
+    a.mode = mode;
+    a.h = f.h;
+    a.mask = f.mask;
+    a.rcp = (N & (N - 1)) == 0 ? 0x1p-32f / (float)N : 0.f;
+    return a;
 }
 
 // The paper's traditional Monte Carlo (Section V-B, Eq. distito): increments
@@ -98,25 +308,42 @@ static int grid_for(int64_t total, int block, int sms)
 cudaError_t launch_lhs_f32(uint64_t seed, int64_t N, int64_t k0, int64_t count, int M, int mode, float* zeta,
                            uint32_t* strata, int sms, cudaStream_t st)
 {
-    if (count == 0) return cudaSuccess;
-    FeistelShape f = feistel_shape(N);
-    int64_t total = count * (int64_t)M;
-    lhs_f32_kernel<<<grid_for(total, 256, sms), 256, 0, st>>>((uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)N,
-                                                              k0, count, M, mode, f.h, f.mask, zeta, strata);
-    return cudaGetLastError();
+    DesignArgs a = design_args(seed, N, k0, count, M, mode);
+    a.zeta = zeta;
+    a.strata = strata;
+    return launch_design<OUT_F32>(a, sms, st);
 }
 
 cudaError_t launch_lhs_split(uint64_t seed, int64_t N, int64_t k0, int64_t count, int d, int K, int mode,
-                             void* hi, void* lo, int sms, cudaStream_t st)
+                             const uint32_t* strata, void* hi, void* lo, int sms, cudaStream_t st)
 {
-    if (count == 0) return cudaSuccess;
-    FeistelShape f = feistel_shape(N);
-    int Ks = round_up(K, 8);
-    int64_t total = count * (int64_t)d * Ks;
-    lhs_split_kernel<<<grid_for(total, 256, sms), 256, 0, st>>>(
-        (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)N, k0, count, d, K, Ks, mode, f.h, f.mask,
-        (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
-    return cudaGetLastError();
+    const int Ks = round_up(K, 8);
+    DesignArgs a = design_args(seed, N, k0, count, d * Ks, mode);
+    a.K = K;
+    a.Ks = Ks;
+    a.hi = static_cast<__nv_bfloat16*>(hi);
+    a.lo = static_cast<__nv_bfloat16*>(lo);
+    a.strata_in = strata;
+    return launch_design<OUT_SPLIT>(a, sms, st);
+}
+
+cudaError_t launch_strata_values(uint64_t seed, int64_t N, int64_t k0, int64_t count, int M, int mode,
+                                 const uint32_t* strata, float* zeta, int sms, cudaStream_t st)
+{
+    DesignArgs a = design_args(seed, N, k0, count, M, mode);
+    a.zeta = zeta;
+    a.strata_in = strata;
+    return launch_design<OUT_F32>(a, sms, st);
+}
+
+cudaError_t launch_design_scores(uint64_t seed, int64_t N, int M, const double* score, const double* mean, float* R,
+                                 int sms, cudaStream_t st)
+{
+    DesignArgs a = design_args(seed, N, 0, N, M, FMC_LHS);
+    a.zeta = R;
+    a.score = score;
+    a.mean = mean;
+    return launch_design<OUT_SCORE>(a, sms, st);
 }
 
 cudaError_t launch_em_increments(uint64_t seed, int64_t k0, int64_t count, int d, int Nt, double dt, float* dW,

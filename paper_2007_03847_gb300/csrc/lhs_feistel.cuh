@@ -11,36 +11,10 @@ namespace fmc {
 
 constexpr int kFeistelRounds = 6;
 
-// Balanced Feistel network on 2h bits; round function = Philox word 0 of the
-// counter (R, dim, 1 + round, 0) masked to h bits.
-__device__ __forceinline__ uint32_t feistel(uint32_t x, uint32_t dim, int h, uint32_t mask, uint32_t k0,
-                                            uint32_t k1)
-{
-    uint32_t L = (x >> h) & mask;
-    uint32_t R = x & mask;
-#pragma unroll
-    for (int r = 0; r < kFeistelRounds; ++r) {
-        U4 o = philox4x32_10(U4{R, dim, 1u + (uint32_t)r, 0u}, k0, k1);
-        uint32_t nL = R;
-        R = L ^ (o.x & mask);
-        L = nL;
-    }
-    return (L << h) | R;
-}
-
-// pi_dim(k): cycle walking restricts the permutation of [0, 2^(2h)) to [0, N);
-// it ends because the cycle through k < N returns to [0, N) within 2^(2h) - N + 1
-// applications.
-__device__ __forceinline__ uint32_t stratum(uint32_t k, uint32_t dim, uint32_t N, int h, uint32_t mask,
-                                            uint32_t k0, uint32_t k1)
-{
-    uint32_t y = k;
-    do {
-        y = feistel(y, dim, h, mask, k0, k1);
-    } while (y >= N);
-    return y;
-}
-
+// Balanced Feistel network on 2h bits: six rounds (L, R) -> (R, L ^ f_r(R)) with
+// f_r(R) = Philox word 0 of the counter (R, dim, 1 + r, 0), masked to h bits;
+// pi_dim(k) is the first iterate of it from k that falls in [0, N) (cycle walking
+// ends: the cycle through k < N returns to [0, N) within 4^h - N + 1 applications).
 struct FeistelShape {
     int h;
     uint32_t mask;
