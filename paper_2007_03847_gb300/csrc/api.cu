@@ -987,7 +987,7 @@ int fmc_kle_reconstruct(fmc_ctx* ctx, const float* zeta_dev, int64_t count, int3
         rc = ensure(ctx, ctx->phi32, (size_t)K * Nt * sizeof(float));
         if (rc) return rc;
         FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, FMC_BASIS_SINE, (float*)ctx->phi32.ptr, ctx->sms, st), "basis kernel");
-        FMC_CUDA(ctx, launch_sgemm_nn(count * d, Nt, K, zeta_dev, (const float*)ctx->phi32.ptr, dW_dev, st),
+        FMC_CUDA(ctx, launch_sgemm_nn(count * d, Nt, K, zeta_dev, (const float*)ctx->phi32.ptr, dW_dev, false, st),
                  "sgemm kernel");
         return FMC_OK;
     }
@@ -1067,7 +1067,7 @@ int fmc_kle_reconstruct_noalloc(fmc_ctx* ctx, const float* zeta_dev, int64_t cou
     if (precision == FMC_PREC_F32) {
         float* phi32 = reinterpret_cast<float*>(base + o_phi32);
         FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, FMC_BASIS_SINE, phi32, ctx->sms, st), "basis kernel");
-        FMC_CUDA(ctx, launch_sgemm_nn(count * d, Nt, K, zeta_dev, phi32, dW_dev, st), "sgemm kernel");
+        FMC_CUDA(ctx, launch_sgemm_nn(count * d, Nt, K, zeta_dev, phi32, dW_dev, false, st), "sgemm kernel");
         return FMC_OK;
     }
     const int split = (precision == FMC_PREC_BF16X3);
@@ -1440,7 +1440,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             prof_begin(ctx, PH_CONTRACT, st, &pr);
             FMC_CUDA(ctx,
                      launch_sgemm_nn(count * d, cols, K, (const float*)ws.zeta32.ptr, (const float*)ws.phi32.ptr,
-                                     (float*)ws.dW.ptr, st),
+                                     (float*)ws.dW.ptr, false, st),
                      "sgemm kernel");
             prof_end(pr, st);
         }

@@ -32,7 +32,7 @@ constexpr int DESIGN_SMEM_MAX = 224 * 1024;
 // walk, and the list is read transposed where strata themselves are stored or
 // loaded (their rows run along the samples).
 //
-// Measured (GB300): 65536 x 600 values and strata 735 -> 355 us (entries computed
+// Measured (GB300): 65536 x 600 values and strata 735 -> 361 us (entries computed
 // one by one from the definition before; 0.9 TB/s of output, the uniform's Philox
 // call and the two branches of the inverse CDF now take the issue slots); the
 // split-BF16 rows of 19001 x 2400 (domain 4^8, 3.4 walks per entry) 6.99 -> 0.70 ms.
