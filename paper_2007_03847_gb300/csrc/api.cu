@@ -46,6 +46,7 @@ struct ProfRec {
 // status word; the plain path's FP32 design, increments and trajectories.
 struct Workspace {
     DevBuf zeta_hi, zeta_lo, phi_hi, phi_lo, phi32, dW, traj, part, eq, scen, status, zeta32;
+    DevBuf trig;    // cosines of the basis by residue (launch_basis_*)
     DevBuf wconst;  // constant block of the large-system kernel
     DevBuf rrf;     // [4] FP64: sums of the response function and its square, a zero shift
     DevBuf ic, ic_strata;  // the correlation-reducing permutation: working memory, new strata [M][N]
@@ -159,6 +160,23 @@ static int ensure(fmc_ctx* ctx, DevBuf& b, size_t bytes)
     b.bytes = want;
     ctx->used += want;
     return FMC_OK;
+}
+
+// The basis kernels' table of cosines (basis_table_doubles), grown if need be; null
+// where a memory budget has no room for it: the kernels then do without.
+static double* trig_table(fmc_ctx* ctx, Workspace& ws, int K, int Nt, int basis, int forcing)
+{
+    const size_t bytes = (size_t)basis_table_doubles(K, Nt, basis, forcing) * sizeof(double);
+    if (ctx->budget && ws.trig.bytes < bytes) return nullptr;
+    if (ensure(ctx, ws.trig, bytes) != FMC_OK) return nullptr;
+    return (double*)ws.trig.ptr;
+}
+
+// The table as reserve() left it (no allocation), or null.
+static double* trig_if_ready(const Workspace& ws, int K, int Nt, int basis, int forcing)
+{
+    return ws.trig.bytes >= (size_t)basis_table_doubles(K, Nt, basis, forcing) * sizeof(double) ? (double*)ws.trig.ptr
+                                                                                             : nullptr;
 }
 
 // ---- profiling --------------------------------------------------------------
@@ -735,7 +753,7 @@ int fmc_destroy(fmc_ctx* ctx)
     DevBuf* bufs[] = {&ctx->zeta_hi, &ctx->zeta_lo, &ctx->phi_hi, &ctx->phi_lo, &ctx->phi32,  &ctx->dW,
                       &ctx->traj,    &ctx->part,    &ctx->eq,     &ctx->scen,   &ctx->status, &ctx->zeta32,
                       &ctx->wconst,  &ctx->rrfbuf, &ctx->ws.ic, &ctx->ws.ic_strata,
-                      &ctx->ws.ident};
+                      &ctx->ws.ident, &ctx->ws.trig};
     for (DevBuf* b : bufs)
         if (b->ptr) cudaFree(b->ptr);
     delete ctx;
@@ -969,7 +987,7 @@ int fmc_kl_basis(fmc_ctx* ctx, int32_t K, double T, int32_t Nt, int32_t basis, f
     if (basis != FMC_BASIS_SINE && basis != FMC_BASIS_COSINE) return fail(ctx, FMC_EINVAL, "basis %d", basis);
     if (K < 1 || Nt < 1 || !(T > 0.0)) return fail(ctx, FMC_EINVAL, "K = %d, Nt = %d, T = %g", K, Nt, T);
     if (!phi_dev) return fail(ctx, FMC_EINVAL, "phi is NULL");
-    FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, basis, phi_dev, ctx->sms, (cudaStream_t)stream), "basis kernel");
+    FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, basis, nullptr, phi_dev, ctx->sms, (cudaStream_t)stream), "basis kernel");
     return FMC_OK;
 }
 
@@ -986,7 +1004,9 @@ int fmc_kle_reconstruct(fmc_ctx* ctx, const float* zeta_dev, int64_t count, int3
     if (precision == FMC_PREC_F32) {
         rc = ensure(ctx, ctx->phi32, (size_t)K * Nt * sizeof(float));
         if (rc) return rc;
-        FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, FMC_BASIS_SINE, (float*)ctx->phi32.ptr, ctx->sms, st), "basis kernel");
+        double* trig = trig_table(ctx, ctx->ws, K, Nt, FMC_BASIS_SINE, 0);
+        FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, FMC_BASIS_SINE, trig, (float*)ctx->phi32.ptr, ctx->sms, st),
+                 "basis kernel");
         FMC_CUDA(ctx, launch_sgemm_nn(count * d, Nt, K, zeta_dev, (const float*)ctx->phi32.ptr, dW_dev, false, st),
                  "sgemm kernel");
         return FMC_OK;
@@ -998,7 +1018,7 @@ int fmc_kle_reconstruct(fmc_ctx* ctx, const float* zeta_dev, int64_t count, int3
     const int Ks = round_up(K, 8);
     const int Kpad = round_up(K, TC_BK);
     const int nkb = (Ks + TC_BK - 1) / TC_BK;
-    const int TN = 64;
+    const int TN = 128;
     // split zeta [count][d*K] FP32 -> [count][d][Ks] BF16 hi/lo via a tiny conversion on the device
     size_t zbytes = (size_t)count * d * Ks * 2;
     if ((rc = ensure(ctx, ctx->zeta_hi, zbytes))) return rc;
@@ -1007,7 +1027,10 @@ int fmc_kle_reconstruct(fmc_ctx* ctx, const float* zeta_dev, int64_t count, int3
     if ((rc = ensure(ctx, ctx->phi_lo, (size_t)Nt * Kpad * 2))) return rc;
     if ((rc = ensure(ctx, ctx->status, 64))) return rc;
     FMC_CUDA(ctx, launch_split_rows(zeta_dev, count, d, K, Ks, ctx->zeta_hi.ptr, ctx->zeta_lo.ptr, st), "split");
-    FMC_CUDA(ctx, launch_basis_split(K, Nt, T, FMC_BASIS_SINE, Kpad, ctx->phi_hi.ptr, ctx->phi_lo.ptr, ctx->sms, st), "basis");
+    FMC_CUDA(ctx,
+             launch_basis_split(K, Nt, T, FMC_BASIS_SINE, Kpad, trig_table(ctx, ctx->ws, K, Nt, FMC_BASIS_SINE, 0),
+                                ctx->phi_hi.ptr, ctx->phi_lo.ptr, ctx->sms, st),
+             "basis");
     CUtensorMap maps[4];
     if ((rc = make_contract_maps(ctx, maps, count, d, Ks, Nt, Kpad, TN, split))) return rc;
     FMC_CUDA(ctx, cudaMemsetAsync(ctx->status.ptr, 0, 64, st), "memset");
@@ -1066,19 +1089,19 @@ int fmc_kle_reconstruct_noalloc(fmc_ctx* ctx, const float* zeta_dev, int64_t cou
     FMC_CUDA(ctx, cudaMemsetAsync(status, 0, NOALLOC_STATUS_BYTES, st), "memset");
     if (precision == FMC_PREC_F32) {
         float* phi32 = reinterpret_cast<float*>(base + o_phi32);
-        FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, FMC_BASIS_SINE, phi32, ctx->sms, st), "basis kernel");
+        FMC_CUDA(ctx, launch_basis_f32(K, Nt, T, FMC_BASIS_SINE, nullptr, phi32, ctx->sms, st), "basis kernel");
         FMC_CUDA(ctx, launch_sgemm_nn(count * d, Nt, K, zeta_dev, phi32, dW_dev, false, st), "sgemm kernel");
         return FMC_OK;
     }
     const int split = (precision == FMC_PREC_BF16X3);
     const int nkb = (Ks + TC_BK - 1) / TC_BK;
-    const int TN = 64;
+    const int TN = 128;
     void* zhi = base + o_zhi;
     void* zlo = base + o_zlo;
     void* phi_hi = base + o_phi_hi;
     void* phi_lo = base + o_phi_lo;
     FMC_CUDA(ctx, launch_split_rows(zeta_dev, count, d, K, Ks, zhi, zlo, st), "split");
-    FMC_CUDA(ctx, launch_basis_split(K, Nt, T, FMC_BASIS_SINE, Kpad, phi_hi, phi_lo, ctx->sms, st), "basis");
+    FMC_CUDA(ctx, launch_basis_split(K, Nt, T, FMC_BASIS_SINE, Kpad, nullptr, phi_hi, phi_lo, ctx->sms, st), "basis");
     CUtensorMap maps[4];
     if ((rc = make_contract_maps_at(ctx, maps, zhi, zlo, phi_hi, phi_lo, count, d, Ks, Nt, Kpad, TN, split)))
         return rc;
@@ -1357,6 +1380,7 @@ static int reserve(fmc_ctx* ctx, Workspace& ws, const Prepared& P, bool want_tra
     const int S = 2 * n;
     int rc;
     const bool em = (P.s.sampling == FMC_SRS_EM);
+    if (!em) trig_table(ctx, ws, K, Nt, P.s.basis, P.s.forcing == FMC_FORCING_SMOOTH);
     if (P.path == FMC_PATH_PLAIN) {
         const int M = d * K;
         // the smooth form takes the forcing at the 2 Nt + 1 half-step times
@@ -1406,6 +1430,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
     ProfRec* pr;
 
     const bool em = (s->sampling == FMC_SRS_EM);
+    double* trig = trig_if_ready(ws, K, Nt, s->basis, s->forcing == FMC_FORCING_SMOOTH);
     EmSpec ems{em ? 1 : 0, (uint32_t)s->seed, (uint32_t)(s->seed >> 32), k0, (float)std::sqrt(s->dt)};
 
     if (P.path == FMC_PATH_PLAIN) {
@@ -1431,10 +1456,10 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             const int cols = smooth ? 2 * Nt + 1 : Nt;
             prof_begin(ctx, PH_BASIS, st, &pr);
             if (smooth)
-                FMC_CUDA(ctx, launch_forcing_f32(K, Nt, s->T, s->basis, (float*)ws.phi32.ptr, ctx->sms, st),
+                FMC_CUDA(ctx, launch_forcing_f32(K, Nt, s->T, s->basis, trig, (float*)ws.phi32.ptr, ctx->sms, st),
                          "forcing basis kernel");
             else
-                FMC_CUDA(ctx, launch_basis_f32(K, Nt, s->T, s->basis, (float*)ws.phi32.ptr, ctx->sms, st),
+                FMC_CUDA(ctx, launch_basis_f32(K, Nt, s->T, s->basis, trig, (float*)ws.phi32.ptr, ctx->sms, st),
                          "basis kernel");
             prof_end(pr, st);
             prof_begin(ctx, PH_CONTRACT, st, &pr);
@@ -1491,11 +1516,10 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
         }
         prof_end(pr, st);
         prof_begin(ctx, PH_BASIS, st, &pr);
+        void* plo = split ? ws.phi_lo.ptr : nullptr;
         FMC_CUDA(ctx,
-                 smooth ? launch_forcing_split(K, Nt, s->T, s->basis, Kpad, ws.phi_hi.ptr, split ? ws.phi_lo.ptr : nullptr,
-                                               ctx->sms, st)
-                        : launch_basis_split(K, Nt, s->T, s->basis, Kpad, ws.phi_hi.ptr, split ? ws.phi_lo.ptr : nullptr,
-                                             ctx->sms, st),
+                 smooth ? launch_forcing_split(K, Nt, s->T, s->basis, Kpad, trig, ws.phi_hi.ptr, plo, ctx->sms, st)
+                        : launch_basis_split(K, Nt, s->T, s->basis, Kpad, trig, ws.phi_hi.ptr, plo, ctx->sms, st),
                  "basis kernel");
         prof_end(pr, st);
         if ((rc = make_contract_maps_at(ctx, maps, ws.zeta_hi.ptr, ws.zeta_lo.ptr, ws.phi_hi.ptr, ws.phi_lo.ptr, count, d,
@@ -1665,7 +1689,7 @@ int fmc::release_workspace(fmc_ctx* ctx, cudaStream_t st)
     // the buffers that scale with the samples or the horizon; the small ones stay
     DevBuf* big[] = {&ctx->ws.zeta_hi, &ctx->ws.zeta_lo, &ctx->ws.phi_hi, &ctx->ws.phi_lo, &ctx->ws.phi32,
                      &ctx->ws.dW,      &ctx->ws.traj,    &ctx->ws.part,   &ctx->ws.zeta32,
-                     &ctx->ws.ic,      &ctx->ws.ic_strata};
+                     &ctx->ws.ic,      &ctx->ws.ic_strata, &ctx->ws.trig};
     for (DevBuf* b : big) {
         if (!b->ptr) continue;
         if (ctx->stream_ordered)
@@ -1804,7 +1828,7 @@ static void batch_free(fmc_batch* b)
     for (Workspace* w : b->ws) {
         DevBuf* bufs[] = {&w->zeta_hi, &w->zeta_lo, &w->phi_hi, &w->phi_lo, &w->phi32,  &w->dW,
                           &w->traj,    &w->part,    &w->eq,     &w->scen,   &w->status, &w->zeta32,
-                          &w->wconst,  &w->rrf,    &w->ic,     &w->ic_strata};
+                          &w->wconst,  &w->rrf,    &w->ic,     &w->ic_strata, &w->trig};
         for (DevBuf* d : bufs)
             if (d->ptr) {
                 cudaFree(d->ptr);

@@ -21,47 +21,173 @@
 
 namespace fmc {
 
-__device__ __forceinline__ double basis_value(int k, int n, int Nt, double T, int basis)
+// An entry is (amplitude of k) x cos(pi m / P) x (sine of k) with an integer residue m:
+// only P' distinct cosines for K Nt entries.  FP64 arithmetic is the bound (two FMA
+// per SM and clock on this part), so the cosines of all residues are tabulated once
+// per call (trig_table_kernel) and an entry costs two FP64 products, the residue kept
+// by additions modulo the period along a thread's times.  Without room for the table
+// (the allocation-free reconstruction) a thread evaluates the cosine itself.  The
+// operations per entry are the same either way, in the same order.
+// Measured (GB300), split form: K = 200, Nt = 4000 148 -> 11 us; K = 100, Nt = 1000
+// 32 -> 8 us.
+struct BasisArgs {
+    int K, Nt, basis;
+    double T;
+    int forcing;           // the smooth form's forcing (below) instead of the increments
+    const double* table;   // cosines by residue (by odd residue for the sine increments), then amplitude and
+                           // sine of every k; or null
+    int64_t cosines;       // entries of the table before the rows'
+};
+
+// The period of the cosine's argument in units of pi / den: den = period / 2.
+__host__ __device__ inline int64_t basis_period(int Nt, int basis)
+{
+    return basis == FMC_BASIS_COSINE ? 4LL * Nt : 8LL * Nt;
+}
+
+// Entries of the table: all residues, or the odd ones (the sine increments' products
+// of odd numbers).
+static int64_t basis_table_entries(int Nt, int basis, int forcing)
+{
+    return (basis == FMC_BASIS_SINE && !forcing) ? 4LL * Nt : basis_period(Nt, basis);
+}
+
+int64_t basis_table_doubles(int K, int Nt, int basis, int forcing)
+{
+    return basis_table_entries(Nt, basis, forcing) + 2 * (int64_t)K;
+}
+
+__device__ __forceinline__ double basis_cos(int64_t m, int Nt, int basis)
+{
+    return cospi((double)m / (basis == FMC_BASIS_COSINE ? 2.0 * Nt : 4.0 * Nt));
+}
+
+// What an entry of row k needs besides its cosine: value = (amp cos) sine (increments)
+// or amp cos (forcing); the constant mode of the cosine basis has no cosine.
+struct BasisRow {
+    double amp, sine;
+    bool flat;       // value = amp
+    uint32_t odd;    // 2k+1 or k: the residue of time index j is odd * (2j+1) (increments) or odd * j
+};
+
+__device__ __forceinline__ BasisRow basis_row(const BasisArgs& a, int k)
 {
     const double PI = 3.141592653589793238462643;
-    if (basis == FMC_BASIS_COSINE) {
-        if (k == 0) return sqrt(T) / (double)Nt;
-        int64_t m = ((int64_t)k * (int64_t)(2 * n + 1)) % (4LL * Nt);
-        double c = sqrt(2.0 * T) / ((double)k * PI);
-        return 2.0 * c * cospi((double)m / (2.0 * Nt)) * sinpi((double)k / (2.0 * Nt));
+    BasisRow r;
+    const bool cosine = a.basis == FMC_BASIS_COSINE;
+    r.flat = cosine && k == 0;
+    r.odd = cosine ? (uint32_t)k : 2u * (uint32_t)k + 1u;
+    r.sine = 1.0;
+    if (a.forcing) {
+        r.amp = r.flat ? 1.0 / sqrt(a.T) : sqrt(2.0 / a.T);
+        return r;
     }
-    int64_t m = ((int64_t)(2 * k + 1) * (int64_t)(2 * n + 1)) % (8LL * Nt);
-    double c = 2.0 * sqrt(2.0 * T) / ((double)(2 * k + 1) * PI);
-    return 2.0 * c * cospi((double)m / (4.0 * Nt)) * sinpi((double)(2 * k + 1) / (4.0 * Nt));
+    if (r.flat) {
+        r.amp = sqrt(a.T) / (double)a.Nt;
+    } else if (cosine) {
+        const double c = sqrt(2.0 * a.T) / ((double)k * PI);
+        r.amp = 2.0 * c;
+        r.sine = sinpi((double)k / (2.0 * a.Nt));
+    } else {
+        const double c = 2.0 * sqrt(2.0 * a.T) / ((double)(2 * k + 1) * PI);
+        r.amp = 2.0 * c;
+        r.sine = sinpi((double)(2 * k + 1) / (4.0 * a.Nt));
+    }
+    return r;
 }
 
-// phi32 [K][Nt] FP32
-__global__ void basis_f32_kernel(int K, int Nt, double T, int basis, float* __restrict__ phi)
+// The table: the cosines, then (amplitude, sine) of every row.
+__global__ void trig_table_kernel(BasisArgs a, int odd, double* __restrict__ table)
 {
-    int64_t total = (int64_t)K * Nt;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int k = (int)(t / Nt);
-        int n = (int)(t - (int64_t)k * Nt);
-        phi[t] = (float)basis_value(k, n, Nt, T, basis);
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e < a.cosines) {
+        table[e] = basis_cos(odd ? 2 * e + 1 : e, a.Nt, a.basis);
+    } else if (e - a.cosines < a.K) {
+        const BasisRow r = basis_row(a, (int)(e - a.cosines));
+        table[a.cosines + 2 * (e - a.cosines)] = r.amp;
+        table[a.cosines + 2 * (e - a.cosines) + 1] = r.sine;
     }
 }
 
-// Time-major split BF16 for the tensor-core B operand: hi/lo [Nt][Kpad],
-// zeros for k >= K.
-__global__ void basis_split_kernel(int K, int Nt, double T, int basis, int Kpad, __nv_bfloat16* __restrict__ hi,
-                                   __nv_bfloat16* __restrict__ lo)
+// Row k with its FP64 constants from the table, where there is one.
+__device__ __forceinline__ BasisRow basis_row_of(const BasisArgs& a, int k)
 {
-    int64_t total = (int64_t)Nt * Kpad;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int n = (int)(t / Kpad);
-        int k = (int)(t - (int64_t)n * Kpad);
-        float v = 0.f;
-        if (k < K) v = (float)basis_value(k, n, Nt, T, basis);
-        __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[t] = h;
-        if (lo) lo[t] = __float2bfloat16_rn(v - __bfloat162float(h));
+    if (!a.table) return basis_row(a, k);
+    BasisRow r;
+    r.flat = a.basis == FMC_BASIS_COSINE && k == 0;
+    r.odd = a.basis == FMC_BASIS_COSINE ? (uint32_t)k : 2u * (uint32_t)k + 1u;
+    r.amp = __ldg(a.table + a.cosines + 2 * (int64_t)k);
+    r.sine = __ldg(a.table + a.cosines + 2 * (int64_t)k + 1);
+    return r;
+}
+
+// x y mod P (32-bit arithmetic where the product allows it).
+__device__ __forceinline__ int64_t mod_product(int64_t x, int64_t y, int64_t P)
+{
+    const int64_t m = x * y;
+    if (m >> 32 == 0 && P >> 32 == 0) return (uint32_t)m % (uint32_t)P;
+    return m % P;
+}
+
+__device__ __forceinline__ float basis_entry(const BasisArgs& a, const BasisRow& r, int64_t m)
+{
+    if (r.flat) return (float)r.amp;
+    const double c = a.table ? __ldg(a.table + ((a.basis == FMC_BASIS_SINE && !a.forcing) ? m >> 1 : m))
+                             : basis_cos(m, a.Nt, a.basis);
+    return a.forcing ? (float)(r.amp * c) : (float)(r.amp * c * r.sine);
+}
+
+// The residue of row r at time index j, and the advance per `step` time indices.
+__device__ __forceinline__ int64_t basis_residue(const BasisArgs& a, const BasisRow& r, int64_t j)
+{
+    return mod_product(r.odd, a.forcing ? j : 2 * j + 1, basis_period(a.Nt, a.basis));
+}
+__device__ __forceinline__ int64_t basis_advance(const BasisArgs& a, const BasisRow& r, int64_t step)
+{
+    return mod_product(r.odd, a.forcing ? step : 2 * step, basis_period(a.Nt, a.basis));
+}
+
+// FP32 [K][J] (J times; J contiguous): a CTA takes row k = blockIdx.y.
+__global__ void __launch_bounds__(256) basis_f32_kernel(BasisArgs a, int J, float* __restrict__ phi)
+{
+    const int64_t P = basis_period(a.Nt, a.basis);
+    const int64_t step = (int64_t)gridDim.x * 256;
+    for (int k = blockIdx.y; k < a.K; k += gridDim.y) {
+        const BasisRow r = basis_row_of(a, k);
+        int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x;
+        int64_t m = basis_residue(a, r, j);
+        const int64_t dm = basis_advance(a, r, step);
+        for (; j < J; j += step) {
+            phi[(int64_t)k * J + j] = basis_entry(a, r, m);
+            m += dm;
+            if (m >= P) m -= P;
+        }
+    }
+}
+
+// Time-major split BF16 for the tensor-core B operand: hi/lo [J][Kpad], zeros for
+// k >= K.  A thread keeps its k and steps over times.
+constexpr int BASIS_TIMES = 8;  // times per CTA of 8 x 32 threads and pass
+
+__global__ void __launch_bounds__(256) basis_split_kernel(BasisArgs a, int J, int Kpad, __nv_bfloat16* __restrict__ hi,
+                                                          __nv_bfloat16* __restrict__ lo)
+{
+    const int64_t P = basis_period(a.Nt, a.basis);
+    const int64_t step = (int64_t)gridDim.x * BASIS_TIMES;
+    for (int k = blockIdx.y * 32 + threadIdx.x % 32; k < Kpad; k += gridDim.y * 32) {
+        const bool real = k < a.K;
+        const BasisRow r = basis_row_of(a, real ? k : 0);
+        int64_t j = blockIdx.x * (int64_t)BASIS_TIMES + threadIdx.x / 32;
+        int64_t m = basis_residue(a, r, j);
+        const int64_t dm = basis_advance(a, r, step);
+        for (; j < J; j += step) {
+            const float v = real ? basis_entry(a, r, m) : 0.f;
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            hi[j * Kpad + k] = h;
+            if (lo) lo[j * Kpad + k] = __float2bfloat16_rn(v - __bfloat162float(h));
+            m += dm;
+            if (m >= P) m -= P;
+        }
     }
 }
 
@@ -70,83 +196,68 @@ __global__ void basis_split_kernel(int K, int Nt, double T, int basis, int Kpad,
 // j = 0..2 Nt.  Brownian eigenbasis: sqrt(2/T) cos((k+1/2) pi t / T) =
 // sqrt(2/T) cospi((2k+1) j / (4 Nt)), the argument reduced modulo 8 Nt; the
 // paper's basis: 1/sqrt(T) (k = 0), sqrt(2/T) cospi(k j / (2 Nt)) (mod 4 Nt).
-__device__ __forceinline__ double forcing_value(int k, int j, int Nt, double T, int basis)
+static cudaError_t basis_prepare(BasisArgs& a, double* table, cudaStream_t st)
 {
-    if (basis == FMC_BASIS_COSINE) {
-        if (k == 0) return 1.0 / sqrt(T);
-        int64_t m = ((int64_t)k * (int64_t)j) % (4LL * Nt);
-        return sqrt(2.0 / T) * cospi((double)m / (2.0 * Nt));
-    }
-    int64_t m = ((int64_t)(2 * k + 1) * (int64_t)j) % (8LL * Nt);
-    return sqrt(2.0 / T) * cospi((double)m / (4.0 * Nt));
-}
-
-// mdot [K][2 Nt + 1] FP32
-__global__ void forcing_f32_kernel(int K, int Nt, double T, int basis, float* __restrict__ mdot)
-{
-    const int J = 2 * Nt + 1;
-    int64_t total = (int64_t)K * J;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int k = (int)(t / J);
-        int j = (int)(t - (int64_t)k * J);
-        mdot[t] = (float)forcing_value(k, j, Nt, T, basis);
-    }
-}
-
-// The forcing basis in the split-BF16 layout of the fused path: time-major
-// [2 Nt + 1][Kpad], the K contiguous (the tensor cores' K-major B operand).
-__global__ void forcing_split_kernel(int K, int Nt, double T, int basis, int Kpad, __nv_bfloat16* __restrict__ hi,
-                                     __nv_bfloat16* __restrict__ lo)
-{
-    const int64_t total = (2 * (int64_t)Nt + 1) * Kpad;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / Kpad);
-        const int k = (int)(t - (int64_t)j * Kpad);
-        const float v = k < K ? (float)forcing_value(k, j, Nt, T, basis) : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[t] = h;
-        if (lo) lo[t] = __float2bfloat16_rn(v - __bfloat162float(h));
-    }
-}
-
-cudaError_t launch_forcing_split(int K, int Nt, double T, int basis, int Kpad, void* hi, void* lo, int sms,
-                                 cudaStream_t st)
-{
-    int64_t total = (2 * (int64_t)Nt + 1) * Kpad;
-    int64_t g = (total + 255) / 256;
-    if (g > sms * 16) g = sms * 16;
-    forcing_split_kernel<<<(int)g, 256, 0, st>>>(K, Nt, T, basis, Kpad, (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
+    a.table = nullptr;
+    if (!table) return cudaSuccess;
+    a.cosines = basis_table_entries(a.Nt, a.basis, a.forcing);
+    const int odd = a.basis == FMC_BASIS_SINE && !a.forcing;
+    trig_table_kernel<<<(unsigned)((a.cosines + a.K + 63) / 64), 64, 0, st>>>(a, odd, table);
+    a.table = table;
     return cudaGetLastError();
 }
 
-cudaError_t launch_forcing_f32(int K, int Nt, double T, int basis, float* mdot, int sms, cudaStream_t st)
+static cudaError_t launch_f32(BasisArgs a, double* table, float* phi, int sms, cudaStream_t st)
 {
-    int64_t total = (int64_t)K * (2 * (int64_t)Nt + 1);
-    int64_t g = (total + 255) / 256;
-    if (g > sms * 16) g = sms * 16;
-    forcing_f32_kernel<<<(int)g, 256, 0, st>>>(K, Nt, T, basis, mdot);
+    cudaError_t e = basis_prepare(a, table, st);
+    if (e != cudaSuccess) return e;
+    const int64_t J = a.forcing ? 2 * (int64_t)a.Nt + 1 : a.Nt;
+    if (J > 2147483647LL) return cudaErrorInvalidValue;
+    const int gy = a.K < 65535 ? a.K : 65535;
+    // eight entries or more per thread: its row and residue cost a few entries' work
+    int64_t gx = (J + 256 * 8 - 1) / (256 * 8);
+    const int64_t cap = ((int64_t)sms * 16 + gy - 1) / gy;
+    if (gx > cap) gx = cap;
+    basis_f32_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(a, (int)J, phi);
     return cudaGetLastError();
 }
 
-cudaError_t launch_basis_f32(int K, int Nt, double T, int basis, float* phi, int sms, cudaStream_t st)
+static cudaError_t launch_split(BasisArgs a, double* table, int Kpad, void* hi, void* lo, int sms, cudaStream_t st)
 {
-    int64_t total = (int64_t)K * Nt;
-    int64_t g = (total + 255) / 256;
-    if (g > sms * 16) g = sms * 16;
-    basis_f32_kernel<<<(int)g, 256, 0, st>>>(K, Nt, T, basis, phi);
+    cudaError_t e = basis_prepare(a, table, st);
+    if (e != cudaSuccess) return e;
+    const int64_t J = a.forcing ? 2 * (int64_t)a.Nt + 1 : a.Nt;
+    if (J > 2147483647LL) return cudaErrorInvalidValue;
+    const int ky = Kpad / 32;
+    const int gy = ky < 65535 ? ky : 65535;
+    int64_t gx = (J + BASIS_TIMES * 8 - 1) / (BASIS_TIMES * 8);
+    const int64_t cap = ((int64_t)sms * 16 + gy - 1) / gy;
+    if (gx > cap) gx = cap;
+    basis_split_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(a, (int)J, Kpad, (__nv_bfloat16*)hi,
+                                                                         (__nv_bfloat16*)lo);
     return cudaGetLastError();
 }
 
-cudaError_t launch_basis_split(int K, int Nt, double T, int basis, int Kpad, void* hi, void* lo, int sms,
-                               cudaStream_t st)
+cudaError_t launch_forcing_split(int K, int Nt, double T, int basis, int Kpad, double* table, void* hi, void* lo,
+                                 int sms, cudaStream_t st)
 {
-    int64_t total = (int64_t)Nt * Kpad;
-    int64_t g = (total + 255) / 256;
-    if (g > sms * 16) g = sms * 16;
-    basis_split_kernel<<<(int)g, 256, 0, st>>>(K, Nt, T, basis, Kpad, (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
-    return cudaGetLastError();
+    return launch_split(BasisArgs{K, Nt, basis, T, 1, nullptr, 0}, table, Kpad, hi, lo, sms, st);
+}
+
+cudaError_t launch_forcing_f32(int K, int Nt, double T, int basis, double* table, float* phi, int sms, cudaStream_t st)
+{
+    return launch_f32(BasisArgs{K, Nt, basis, T, 1, nullptr, 0}, table, phi, sms, st);
+}
+
+cudaError_t launch_basis_f32(int K, int Nt, double T, int basis, double* table, float* phi, int sms, cudaStream_t st)
+{
+    return launch_f32(BasisArgs{K, Nt, basis, T, 0, nullptr, 0}, table, phi, sms, st);
+}
+
+cudaError_t launch_basis_split(int K, int Nt, double T, int basis, int Kpad, double* table, void* hi, void* lo,
+                               int sms, cudaStream_t st)
+{
+    return launch_split(BasisArgs{K, Nt, basis, T, 0, nullptr, 0}, table, Kpad, hi, lo, sms, st);
 }
 
 }  // namespace fmc

@@ -17,10 +17,12 @@ namespace fmc {
 struct ContractArgs {
     int64_t count;
     int d, Ks, nkb, Nt, TN;
-    int split;
+    int split, ns;
     float* dW;
     int* err;
 };
+
+constexpr int CT_LD = 33;  // floats per row of a warp's 32 x 32 transpose
 
 __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant__ CUtensorMap mAh,
                                                           const __grid_constant__ CUtensorMap mAl,
@@ -32,7 +34,7 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
     // integer round trip), so that every access through these pointers stays a
     // shared-memory access rather than a generic one
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    __shared__ uint64_t bars[5];  // full[2], freed[2], done
+    __shared__ uint64_t bars[2 * TC_MAX_STAGES + 1];  // full[ns], freed[ns], done
     __shared__ uint32_t tmem_base;
     __shared__ int ok_flag;
 
@@ -47,18 +49,15 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
     r.b_bytes = a.TN * 64;
     r.split = a.split;
     r.base = smem;
-    r.ns = 2;
+    r.ns = (uint32_t)a.ns;
     r.full = &bars[0];
-    r.freed = &bars[2];
+    r.freed = &bars[TC_MAX_STAGES];
+    uint64_t* done = &bars[2 * TC_MAX_STAGES];
 
     if (threadIdx.x == 0) {
         prefetch_tmap(&mAh);
         prefetch_tmap(&mBh);
-        mbar_init(&bars[0], 1);
-        mbar_init(&bars[1], 1);
-        mbar_init(&bars[2], 1);
-        mbar_init(&bars[3], 1);
-        mbar_init(&bars[4], 1);
+        for (int b = 0; b < 2 * TC_MAX_STAGES + 1; ++b) mbar_init(&bars[b], 1);
         fence_mbar_init();
         ok_flag = 1;
     }
@@ -72,14 +71,19 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
         const uint32_t idesc = umma_idesc_bf16(TC_M, a.TN);
         bool ok = true;
         const int ax0 = w * a.Ks;
-        ok = ring_load(r, 0, &mAh, &mAl, &mBh, &mBl, ax0, (int)row0, 0, n0);
+        int issued = 0;
+        auto load = [&](int kb) {
+            return ring_load(r, (uint32_t)kb, &mAh, &mAl, &mBh, &mBl, ax0 + kb * TC_BK, (int)row0, kb * TC_BK, n0);
+        };
+        for (; issued < a.nkb && issued + 1 < a.ns && ok; ++issued) ok = load(issued);
         for (int kb = 0; kb < a.nkb && ok; ++kb) {
-            if (kb + 1 < a.nkb)
-                ok = ring_load(r, kb + 1, &mAh, &mAl, &mBh, &mBl, ax0 + (kb + 1) * TC_BK, (int)row0,
-                               (kb + 1) * TC_BK, n0);
-            if (ok) ok = ring_mma(r, kb, tmem, idesc, kb == 0);
+            if (issued < a.nkb) {
+                ok = load(issued);
+                ++issued;
+            }
+            if (ok) ok = ring_mma(r, (uint32_t)kb, tmem, idesc, kb == 0);
         }
-        if (ok) umma_commit(&bars[4]);
+        if (ok) umma_commit(done);
         if (!ok) {
             ok_flag = 0;
             atomicExch(a.err, DEV_TIMEOUT_TMA);
@@ -87,26 +91,35 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
     }
     __syncthreads();
     bool ok = ok_flag != 0;
-    if (ok && !mbar_wait(&bars[4], 0)) {
+    if (ok && !mbar_wait(done, 0)) {
         ok = false;
         if (lane == 0) atomicExch(a.err, DEV_TIMEOUT_MMA);
     }
-    // warps agree on ok (tcgen05.ld is warp-collective)
-    ok = __all_sync(0xffffffffu, ok);
+    // all warps agree on ok (tcgen05.ld is warp-collective, and the transposes below
+    // take the ring's place: every MMA has read its operands)
+    ok = __syncthreads_and(ok);
     tc_fence_after();
     if (ok) {
-        const int64_t srow = row0 + warp * 32 + lane;
         const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-        for (int c = 0; c < a.TN; c += 4) {
-            float v[4];
-            tmem_ld4(lane_addr + c, v);
-            tmem_ld_wait();
-            if (srow < a.count) {
-                float* out = a.dW + (srow * a.d + w) * (int64_t)a.Nt + n0 + c;
+        float* tr = reinterpret_cast<float*>(smem) + warp * 32 * CT_LD;
+        const int64_t left = a.count - row0 - warp * 32;  // samples of this warp
+        const int rows = left <= 0 ? 0 : (left >= 32 ? 32 : (int)left);
+        float* out = a.dW + ((row0 + warp * 32) * a.d + w) * (int64_t)a.Nt + n0;
+        const int64_t rs = (int64_t)a.d * a.Nt;
+        // a lane holds a sample's row: 32 steps at a time are turned in shared memory, so
+        // that a warp stores 128 consecutive bytes of one row
+        for (int c = 0; c < a.TN && n0 + c < a.Nt; c += 32) {
+            float v[32];
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (n0 + c + e < a.Nt) out[e] = v[e];
-            }
+            for (int e = 0; e < 32; e += 8) tmem_ld8(lane_addr + c + e, reinterpret_cast<float(&)[8]>(v[e]));
+            tmem_ld_wait();
+            __syncwarp();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) tr[lane * CT_LD + e] = v[e];
+            __syncwarp();
+            if (n0 + c + lane < a.Nt)
+#pragma unroll 8
+                for (int s = 0; s < rows; ++s) __stcs(out + s * rs + c + lane, tr[s * CT_LD + lane]);
         }
     }
     tc_fence_before();
@@ -115,39 +128,49 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
 }
 
 // zeta [count][d*K] FP32 -> hi/lo [count][d][Ks] BF16 with zero padding.
-__global__ void split_rows_kernel(const float* __restrict__ z, int64_t count, int d, int K, int Ks,
-                                  __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo)
+// A CTA takes 128 consecutive positions of the padded row and steps over samples, so
+// no index division is left per entry.
+__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ z, int64_t count, int d, int K,
+                                                         int Ks, __nv_bfloat16* __restrict__ hi,
+                                                         __nv_bfloat16* __restrict__ lo)
 {
-    int64_t row = (int64_t)d * Ks;
-    int64_t total = count * row;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t j = t / row;
-        int rem = (int)(t - j * row);
-        int w = rem / Ks, kk = rem - w * Ks;
-        float v = (kk < K) ? z[j * (int64_t)d * K + (int64_t)w * K + kk] : 0.f;
-        __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[t] = h;
-        lo[t] = __float2bfloat16_rn(v - __bfloat162float(h));
+    const int64_t cols = (int64_t)d * Ks;
+    for (int64_t pos = blockIdx.y * (int64_t)128 + threadIdx.x % 128; pos < cols; pos += (int64_t)gridDim.y * 128) {
+        const int64_t w = pos / Ks, kk = pos - w * Ks;
+        const bool real = kk < K;
+        const float* zc = z + w * K + kk;
+        for (int64_t j = blockIdx.x * (int64_t)2 + threadIdx.x / 128; j < count; j += (int64_t)gridDim.x * 2) {
+            const float v = real ? zc[j * d * K] : 0.f;
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            hi[j * cols + pos] = h;
+            lo[j * cols + pos] = __float2bfloat16_rn(v - __bfloat162float(h));
+        }
     }
 }
 
 cudaError_t launch_split_rows(const float* z, int64_t count, int d, int K, int Ks, void* hi, void* lo, cudaStream_t st)
 {
-    int64_t total = count * (int64_t)d * Ks;
-    int64_t g = (total + 255) / 256;
-    if (g > 65536) g = 65536;
-    split_rows_kernel<<<(unsigned)g, 256, 0, st>>>(z, count, d, K, Ks, (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
+    int64_t gy = ((int64_t)d * Ks + 127) / 128;
+    if (gy > 65535) gy = 65535;
+    int64_t gx = (count + 15) / 16;  // eight samples per thread
+    if (gx > 65536) gx = 65536;
+    split_rows_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(z, count, d, K, Ks, (__nv_bfloat16*)hi,
+                                                                       (__nv_bfloat16*)lo);
     return cudaGetLastError();
 }
 
 cudaError_t launch_contract_tc(const CUtensorMap* maps, int64_t count, int d, int Ks, int nkb, int Nt, int TN,
                                int split, float* dW, int* err, cudaStream_t st)
 {
-    ContractArgs a{count, d, Ks, nkb, Nt, TN, split, dW, err};
+    // three CTAs per SM with two 32 KB stages (four with three 16 KB stages in plain
+    // BF16): one CTA's stores run beside the others' loads and MMAs
     const int stage_bytes = (TC_M * 64 + TN * 64) * (split ? 2 : 1);
+    const int ns = split ? 2 : 3;
+    ContractArgs a{count, d, Ks, nkb, Nt, TN, split, ns, dW, err};
     // at least 47 KB so that no more than four CTAs (4 x 128 TMEM columns) share an SM
-    int smem = 2 * stage_bytes + 1024;
+    int smem = ns * stage_bytes + 1024;
+    const int trans = 4 * 32 * CT_LD * 4 + 1024;
+    if (smem < trans) smem = trans;
     if (smem < 233472 / 5 - 1024 + 64) smem = 233472 / 5 - 1024 + 64;
     static bool attr_done = false;
     if (!attr_done) {

@@ -42,14 +42,17 @@ cudaError_t launch_design_scores(uint64_t seed, int64_t N, int M, const double* 
                                  int sms, cudaStream_t st);
 cudaError_t launch_em_increments(uint64_t seed, int64_t k0, int64_t count, int d, int Nt, double dt, float* dW,
                                  int sms, cudaStream_t st);
-cudaError_t launch_basis_f32(int K, int Nt, double T, int basis, float* phi, int sms, cudaStream_t st);
-// the smooth form's forcing basis mdot [K][2 Nt + 1] (half-step times), FP32
-cudaError_t launch_forcing_f32(int K, int Nt, double T, int basis, float* mdot, int sms, cudaStream_t st);
-cudaError_t launch_basis_split(int K, int Nt, double T, int basis, int Kpad, void* hi, void* lo, int sms,
+// The increment basis (and the smooth form's forcing at the 2 Nt + 1 half-step times):
+// FP32 [K][Nt] ([K][2 Nt + 1]), or split BF16, time-major [Nt][Kpad] ([2 Nt + 1][Kpad]).
+// table: basis_table_doubles(..) doubles of working memory, or null (slower)
+int64_t basis_table_doubles(int K, int Nt, int basis, int forcing);
+cudaError_t launch_basis_f32(int K, int Nt, double T, int basis, double* table, float* phi, int sms, cudaStream_t st);
+cudaError_t launch_forcing_f32(int K, int Nt, double T, int basis, double* table, float* mdot, int sms,
                                cudaStream_t st);
-// the smooth form's forcing basis in split BF16, time-major [2 Nt + 1][Kpad]
-cudaError_t launch_forcing_split(int K, int Nt, double T, int basis, int Kpad, void* hi, void* lo, int sms,
-                                 cudaStream_t st);
+cudaError_t launch_basis_split(int K, int Nt, double T, int basis, int Kpad, double* table, void* hi, void* lo,
+                               int sms, cudaStream_t st);
+cudaError_t launch_forcing_split(int K, int Nt, double T, int basis, int Kpad, double* table, void* hi, void* lo,
+                                 int sms, cudaStream_t st);
 // C [R][Ncols] = A [R][K] B [K][Ncols]; upper: B is upper triangular (k <= column)
 cudaError_t launch_sgemm_nn(int64_t R, int Ncols, int K, const float* A, const float* B, float* C, bool upper,
                             cudaStream_t st);
