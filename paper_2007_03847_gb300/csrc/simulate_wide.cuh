@@ -26,6 +26,8 @@
 // equilibrium, diagonal excluded).
 #pragma once
 
+#include <type_traits>
+
 #include "fmc_common.cuh"
 #include "kernels.cuh"
 #include "swing.cuh"
@@ -89,6 +91,7 @@ template <int NMT, int TIER, int CST, int H>
 __device__ __forceinline__ void publish_tier(uint32_t hi, uint32_t lo, const float (&x)[NMT], float csh,
                                              const float* cst_s, int h, int n, int nb, float bcm, float bsn)
 {
+    constexpr int KREAL = (wide_tc_min_n(NMT, H) - H) / H + 1;  // slots that hold a machine in every such layout
     float pg = 0.f, pe = 0.f;
 #pragma unroll
     for (int k = 0; k < NMT; ++k) {
@@ -97,8 +100,9 @@ __device__ __forceinline__ void publish_tier(uint32_t hi, uint32_t lo, const flo
         float sn, cm1;
         deviation_trig1<TIER>(x[k] - csh, &sn, &cm1);
         const bool bus = k == NMT - 1 && i == nb;  // (the bus holds a warp's last slot)
-        const float gx = i < n ? fmaf(csn.x, cm1, -csn.y * sn) : (bus ? bcm : 0.f);
-        const float ex = i < n ? fmaf(csn.y, cm1, csn.x * sn) : (bus ? -bsn : 0.f);
+        const bool real = k < KREAL || i < n;
+        const float gx = real ? fmaf(csn.x, cm1, -csn.y * sn) : (bus ? bcm : 0.f);
+        const float ex = real ? fmaf(csn.y, cm1, csn.x * sn) : (bus ? -bsn : 0.f);
         if (k & 1)
             net_store4(hi, lo, 2 * (k - 1), pg, pe, gx, ex);
         else if (k == NMT - 1)
@@ -117,10 +121,11 @@ __device__ __forceinline__ void publish_angles(uint32_t hi, uint32_t lo, const f
 {
     float bcm = 0.f, bsn = 0.f;
     if (nb >= 0 && nb % H == h) bus_deviation(csh, &bcm, &bsn);
+    constexpr int KREAL = (wide_tc_min_n(NMT, H) - H) / H + 1;
     float m = 0.f;
 #pragma unroll
     for (int k = 0; k < NMT; ++k)
-        if (h + H * k < n) m = fmaxf(m, fabsf(x[k] - csh));
+        if (k < KREAL || h + H * k < n) m = fmaxf(m, fabsf(x[k] - csh));
     const uint32_t mm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
     if (mm <= __float_as_uint(0.05f))
         publish_tier<NMT, 0, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
@@ -130,6 +135,71 @@ __device__ __forceinline__ void publish_angles(uint32_t hi, uint32_t lo, const f
         publish_tier<NMT, 2, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
     else
         publish_tier<NMT, 3, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
+}
+
+// The (gamma, eta) of the next stage input (one A buffer: wide_tc_stash) into the
+// thread's row of shared memory, 2 k and 2 k + 1 for slot k.  pub (a stage's input):
+// the series of each machine's own tier (wide_gamma_eta_tier); else (a step's) that of
+// all of the warp's machines, as publish_angles takes it.  Both ask first whether the
+// shortest series will do for all.
+template <int NMT, int CST, int H>
+__device__ __forceinline__ void stash_angles(float* row, const float (&x)[NMT], float csh, const float* cst_s, int h,
+                                             int n, int nb, bool pub)
+{
+    constexpr int KREAL = (wide_tc_min_n(NMT, H) - H) / H + 1;
+    float bcm = 0.f, bsn = 0.f;
+    if (nb >= 0 && nb % H == h) bus_deviation(csh, &bcm, &bsn);
+    uint32_t mu = 0;  // (magnitudes compare as their bit patterns, a NaN above all)
+    float mf = 0.f;
+#pragma unroll
+    for (int k = 0; k < NMT; ++k)
+        if (k < KREAL || h + H * k < n) {
+            mu = max(mu, __float_as_uint(fabsf(x[k] - csh)));
+            if (!pub) mf = fmaxf(mf, fabsf(x[k] - csh));
+        }
+    const uint32_t mm = __reduce_max_sync(0xffffffffu, pub ? mu : __float_as_uint(mf));
+    auto put = [&](int k, float sn, float cm1) {
+        const int i = h + H * k;
+        const bool real = k < KREAL || i < n;
+        const float2 csn = *reinterpret_cast<const float2*>(cst_s + i * CST);
+        const bool bus = k == NMT - 1 && i == nb;
+        row[2 * k] = real ? fmaf(csn.x, cm1, -csn.y * sn) : (bus ? bcm : 0.f);
+        row[2 * k + 1] = real ? fmaf(csn.y, cm1, csn.x * sn) : (bus ? -bsn : 0.f);
+    };
+    if (mm <= __float_as_uint(0.05f)) {
+#pragma unroll
+        for (int k = 0; k < NMT; ++k) {
+            float sn, cm1;
+            sin_cosm1_tiny(x[k] - csh, &sn, &cm1);
+            put(k, sn, cm1);
+        }
+        return;
+    }
+#pragma unroll 1
+    for (int k = 0; k < NMT; ++k) {
+        // (the slot's angle by selects: a run-time index would put x in memory)
+        float xk = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < NMT; ++kk)
+            if (kk == k) xk = x[kk];
+        const float y = xk - csh;
+        uint32_t t = mm;
+        if (pub) t = __reduce_max_sync(0xffffffffu, h + H * k < n ? __float_as_uint(fabsf(y)) : 0u);
+        float sn, cm1;
+        if (t <= __float_as_uint(0.05f))
+            sin_cosm1_tiny(y, &sn, &cm1);
+        else if (t <= __float_as_uint(0.25f))
+            sin_cosm1_mid(y, &sn, &cm1);
+        else if (t <= __float_as_uint(0.8f))
+            sin_cosm1_small(y, &sn, &cm1);
+        else
+            sin_cosm1_any(y, &sn, &cm1);
+        const int i = h + H * k;
+        const bool real = i < n, bus = k == NMT - 1 && i == nb;
+        const float2 csn = *reinterpret_cast<const float2*>(cst_s + i * CST);
+        row[2 * k] = real ? fmaf(csn.x, cm1, -csn.y * sn) : (bus ? bcm : 0.f);
+        row[2 * k + 1] = real ? fmaf(csn.y, cm1, csn.x * sn) : (bus ? -bsn : 0.f);
+    }
 }
 
 // TCN: the network sums on the tensor cores (wide_tc.cuh) instead of the FP32
@@ -237,6 +307,8 @@ __global__ void __launch_bounds__(H * 128, 4 / H)
     const bool em = a.em.on != 0;
     uint64_t* netbar = &bars[2 * TC_MAX_STAGES + 1];
     uint64_t* netld = &bars[2 * TC_MAX_STAGES + 2];
+    // slots below KREAL hold a machine in every layout of this bucket
+    constexpr int KREAL = TCN ? (wide_tc_min_n(NMT, H) - H) / H + 1 : 0;
     if (tid == 0) {
         if (!em) {
             prefetch_tmap(&mAh);
@@ -262,6 +334,8 @@ __global__ void __launch_bounds__(H * 128, 4 / H)
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     // TCN: this warp's columns of A_hi, A_lo (buffer 0; AB2: buffer 1 at +3 NN) and D
     constexpr bool AB2 = TCN && wide_tc_abuf2(NMT, H);
+    constexpr bool STASH = TCN && wide_tc_stash(NMT, H);
+    constexpr bool EARLY = AB2 || STASH;  // the next input is formed beside the product
     const uint32_t a_hi = lane_addr + net0 + (uint32_t)(h * wide_kh(NMT));
     const uint32_t a_lo = a_hi + NN, a_d = a_hi + 2 * NN;
     int bad = 0;          // TCN: a bounded wait of this thread gave up
@@ -461,7 +535,7 @@ if constexpr (TCN) {
                 const bool pub = (st + 1 < nst);
                 float pg = 0.f, pe = 0.f;  // (gamma, eta) of the pair's first machine
                 float ps = 0.f;            // sum of the next input's deviations
-                if constexpr (AB2) {
+                if constexpr (EARLY) {
                     // the angle half while the product runs: delta' depends on omega
                     // alone, so the next stage's angle input (after the last stage:
                     // the step's new angles, the next step's first input) and its
@@ -472,14 +546,31 @@ if constexpr (TCN) {
                         const float kd = a.omega_s * (yw[k] - w0);
                         ad[k] = fmaf(b, kd, ad[k]);
                         yn[k] = pub ? fmaf(cn, kd, del[k]) : fmaf(hh, ad[k], del[k]);
-                        ps += h + H * k < n ? yn[k] : 0.f;
+                        ps += (k < KREAL || h + H * k < n) ? yn[k] : 0.f;
                     }
-                    publish_angles<NMT, CST, H>(a_hi + an, a_lo + an, yn, csh, cst_s, h, n, nb);
+                    if constexpr (AB2) {
+                        publish_angles<NMT, CST, H>(a_hi + an, a_lo + an, yn, csh, cst_s, h, n, nb);
+                    } else {
+                        stash_angles<NMT, CST, H>(wbuf + lane * WROW, yn, csh, cst_s, h, n, nb, pub);
+                    }
                     cpart[(gb ^ 1) * (H * 128) + h * 128 + r] = ps;
                 }
                 float xs[ND];
 #pragma unroll
                 for (int e = 0; e < ND; ++e) xs[e] = fmaf(xw, x1[e] - x0[e], x0[e]);
+                // the next input's angles need no network sums, and neither does the question
+                // whether all of them are in the shortest series' range: asked here, once for
+                // the warp's machines, it leaves the loop below free of votes and branches
+                bool tiny = false;
+                if (!EARLY && pub) {
+                    uint32_t mu = 0;  // (magnitudes compare as their bit patterns, a NaN above all)
+#pragma unroll
+                    for (int k = 0; k < NMT; ++k) {
+                        const float yd = fmaf(cn, a.omega_s * (yw[k] - w0), del[k]);
+                        if (k < KREAL || h + H * k < n) mu = max(mu, __float_as_uint(fabsf(yd - csh)));
+                    }
+                    tiny = __reduce_max_sync(0xffffffffu, mu) <= __float_as_uint(0.05f);
+                }
                 if (!net_wait(netbar, nph)) {
                     bad = 1;
                     atomicExch(a.err, DEV_TIMEOUT_MMA);
@@ -490,66 +581,95 @@ if constexpr (TCN) {
                 // (2 RP columns; 2 from 7 slots on, where registers are scarcest),
                 // so that few values are live at once; with one A buffer the next
                 // stage's input goes out in pairs of machines as soon as they are
-                // computed
-                constexpr int RP = NMT >= 7 ? 2 : 4;
-                float dd[2 * RP], ah[2 * RP], al[2 * RP];
+                // computed.  TINY: every machine's series is the shortest (see above).
                 // (one A buffer: the infinite bus's slot of the next input, from csh)
                 float bcm = 0.f, bsn = 0.f;
-                if (!AB2 && pub && nb >= 0 && nb % H == h) bus_deviation(csh, &bcm, &bsn);
+                if (!EARLY && pub && nb >= 0 && nb % H == h) bus_deviation(csh, &bcm, &bsn);
+                auto machines = [&](auto tiny_c) {
+                    constexpr bool TINY = decltype(tiny_c)::value;
+                    constexpr int RP = NMT >= 7 ? 2 : 4;
+                    float dd[2 * RP], ah[2 * RP], al[2 * RP];
 #pragma unroll
-                for (int k = 0; k < NMT; ++k) {
-                    if (k % RP == 0) {
-                        // columns of a last, partial piece
-                        constexpr int WT = NMT % RP == 0 ? 2 * RP : (2 * (NMT % RP) + 3) & ~3;
-                        if (NMT - k >= RP)
-                            net_read<2 * RP>(a_d, a_hi + ab, a_lo + ab, 2 * k, dd, ah, al);
-                        else
-                            net_read<WT>(a_d, a_hi + ab, a_lo + ab, 2 * k, reinterpret_cast<float(&)[WT]>(dd),
-                                         reinterpret_cast<float(&)[WT]>(ah), reinterpret_cast<float(&)[WT]>(al));
-                    }
-                    const int i = h + H * k;
-                    const int c = 2 * (k % RP);
-                    const float du = dd[c], dv = dd[c + 1];
-                    const float gi = ah[c] + al[c], ei = ah[c + 1] + al[c + 1];
-                    const float4 ca = *reinterpret_cast<const float4*>(cst_s + i * CST);
-                    const float cs = ca.x, ss = ca.y;
-                    float dpe = fmaf(cs, du, ss * dv);
-                    dpe = fmaf(gi, ca.z + du, dpe);
-                    dpe = fmaf(ei, ca.w + dv, dpe);
-                    float f = 0.f;
-#pragma unroll
-                    for (int e4 = 0; e4 < ND; e4 += 4) {
-                        // rows past the slots in use are zero
-                        const float4 cj = *reinterpret_cast<const float4*>(cst_s + i * CST + 8 + e4);
-                        const float cjv[4] = {cj.x, cj.y, cj.z, cj.w};
-#pragma unroll
-                        for (int e = e4; e < ND && e < e4 + 4; ++e) f = fmaf(cjv[e - e4], xs[e], f);
-                    }
-                    const float2 cb = *reinterpret_cast<const float2*>(cst_s + i * CST + 5);
-                    const float kw = (f - dpe - cb.y * yw[k]) * cb.x;
-                    if constexpr (!AB2) {
-                        const float kd = a.omega_s * (yw[k] - w0);
-                        ad[k] = fmaf(b, kd, ad[k]);
-                        const float yd = fmaf(cn, kd, del[k]);
-                        if (pub) {
-                            // the next stage's input of machine i (its columns were read above)
-                            const float2 g = wide_gamma_eta_tier(yd - csh, cs, ss, i < n);
-                            const bool bus = k == NMT - 1 && i == nb;
-                            const float gx = i < n ? g.x : (bus ? bcm : 0.f);
-                            const float ex = i < n ? g.y : (bus ? -bsn : 0.f);
-                            ps += i < n ? yd : 0.f;
-                            if (k & 1)
-                                net_store4(a_hi, a_lo, 2 * (k - 1), pg, pe, gx, ex);
-                            else if (k == NMT - 1)
-                                net_store4(a_hi, a_lo, 2 * k, gx, ex, 0.f, 0.f);
-                            pg = gx;
-                            pe = ex;
+                    for (int k = 0; k < NMT; ++k) {
+                        if (k % RP == 0) {
+                            // columns of a last, partial piece
+                            constexpr int WT = NMT % RP == 0 ? 2 * RP : (2 * (NMT % RP) + 3) & ~3;
+                            if (NMT - k >= RP)
+                                net_read<2 * RP>(a_d, a_hi + ab, a_lo + ab, 2 * k, dd, ah, al);
+                            else
+                                net_read<WT>(a_d, a_hi + ab, a_lo + ab, 2 * k, reinterpret_cast<float(&)[WT]>(dd),
+                                             reinterpret_cast<float(&)[WT]>(ah), reinterpret_cast<float(&)[WT]>(al));
                         }
+                        const int i = h + H * k;
+                        const bool real = k < KREAL || i < n;
+                        const int c = 2 * (k % RP);
+                        const float du = dd[c], dv = dd[c + 1];
+                        const float gi = ah[c] + al[c], ei = ah[c + 1] + al[c + 1];
+                        const float4 ca = *reinterpret_cast<const float4*>(cst_s + i * CST);
+                        const float cs = ca.x, ss = ca.y;
+                        float dpe = fmaf(cs, du, ss * dv);
+                        dpe = fmaf(gi, ca.z + du, dpe);
+                        dpe = fmaf(ei, ca.w + dv, dpe);
+                        float f = 0.f;
+#pragma unroll
+                        for (int e4 = 0; e4 < ND; e4 += 4) {
+                            // rows past the slots in use are zero
+                            const float4 cj = *reinterpret_cast<const float4*>(cst_s + i * CST + 8 + e4);
+                            const float cjv[4] = {cj.x, cj.y, cj.z, cj.w};
+#pragma unroll
+                            for (int e = e4; e < ND && e < e4 + 4; ++e) f = fmaf(cjv[e - e4], xs[e], f);
+                        }
+                        // delta*, 1/(2H), D, H / sum H
+                        const float4 cb = *reinterpret_cast<const float4*>(cst_s + i * CST + 4);
+                        const float kw = (f - dpe - cb.z * yw[k]) * cb.y;
+                        if constexpr (!EARLY) {
+                            const float kd = a.omega_s * (yw[k] - w0);
+                            ad[k] = fmaf(b, kd, ad[k]);
+                            const float yd = fmaf(cn, kd, del[k]);
+                            if (pub) {
+                                // the next stage's input of machine i (its columns were read above)
+                                float2 g;
+                                if constexpr (TINY) {
+                                    float sn, cm1;
+                                    sin_cosm1_tiny(yd - csh, &sn, &cm1);
+                                    g = make_float2(fmaf(cs, cm1, -ss * sn), fmaf(ss, cm1, cs * sn));
+                                } else {
+                                    g = wide_gamma_eta_tier(yd - csh, cs, ss, real);
+                                }
+                                const bool bus = k == NMT - 1 && i == nb;
+                                const float gx = real ? g.x : (bus ? bcm : 0.f);
+                                const float ex = real ? g.y : (bus ? -bsn : 0.f);
+                                ps += real ? yd : 0.f;
+                                if (k & 1)
+                                    net_store4(a_hi, a_lo, 2 * (k - 1), pg, pe, gx, ex);
+                                else if (k == NMT - 1)
+                                    net_store4(a_hi, a_lo, 2 * k, gx, ex, 0.f, 0.f);
+                                pg = gx;
+                                pe = ex;
+                            }
+                        }
+                        aw[k] = fmaf(b, kw, aw[k]);
+                        yw[k] = fmaf(cn, kw, w[k]);
                     }
-                    aw[k] = fmaf(b, kw, aw[k]);
-                    yw[k] = fmaf(cn, kw, w[k]);
+                };
+                if constexpr (EARLY) {
+                    machines(std::false_type{});
+                } else {
+                    if (tiny)
+                        machines(std::true_type{});
+                    else
+                        machines(std::false_type{});
                 }
-                if (!AB2 && pub) {
+                if constexpr (STASH) {
+                    // the product has read the input: the next one takes its place
+                    const float* sw = wbuf + lane * WROW;
+#pragma unroll
+                    for (int k = 0; k < NMT; k += 2)
+                        net_store4(a_hi, a_lo, 2 * k, sw[2 * k], sw[2 * k + 1], k + 1 < NMT ? sw[2 * k + 2] : 0.f,
+                                   k + 1 < NMT ? sw[2 * k + 3] : 0.f);
+                    tmem_st_wait();
+                }
+                if (!EARLY && pub) {
                     tmem_st_wait();
                     cpart[(gb ^ 1) * (H * 128) + h * 128 + r] = ps;
                 }
@@ -699,14 +819,14 @@ if constexpr (TCN) {
             theta = fmaf(hh, ath, theta);
 #pragma unroll
             for (int e = 0; e < ND; ++e) x0[e] = x1[e];
-            // stage-0 input of the next step (AB2: already published by the last stage)
-            if constexpr (AB2) {
+            // stage-0 input of the next step (EARLY: already published by the last stage)
+            if constexpr (EARLY) {
                 if (h == 0) w0buf[(gb ^ 1) * 128 + r] = w[0];
                 gb ^= 1;
             } else if constexpr (TCN) {
                 float ps = 0.f;
 #pragma unroll
-                for (int k = 0; k < NMT; ++k) ps += h + H * k < n ? del[k] : 0.f;
+                for (int k = 0; k < NMT; ++k) ps += (k < KREAL || h + H * k < n) ? del[k] : 0.f;
                 publish_angles<NMT, CST, H>(a_hi, a_lo, del, csh, cst_s, h, n, nb);
                 cpart[(gb ^ 1) * (H * 128) + h * 128 + r] = ps;
                 if (h == 0) w0buf[(gb ^ 1) * 128 + r] = w[0];

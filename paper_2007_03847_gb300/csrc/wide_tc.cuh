@@ -56,6 +56,20 @@ __host__ __device__ constexpr int wide_tc_net_bytes(int nmt, int H = 4)
     return 2 * wide_nn(nmt, H) * wide_nn(nmt, H) * 4;
 }
 
+// With more slots than that (and four warps per sample) one A buffer is all TMEM
+// holds: the next input is then formed in the same place, beside the product, but
+// waits in shared memory (the transpose rows of the moments, idle during the stages)
+// until the product has read the current one.
+__host__ __device__ constexpr bool wide_tc_stash(int nmt, int H = 4) { return H == 4 && !wide_tc_abuf2(nmt, H); }
+
+// The smallest machine count that takes the layout of nmt slots and H warps per sample
+// (wide_nmt_for and the two-warp buckets): slots below it need no test for padding.
+__host__ __device__ constexpr int wide_tc_min_n(int nmt, int H)
+{
+    return H == 2 ? (nmt == 9 ? 17 : 2 * nmt - 1)
+                  : (nmt == 4 ? 13 : nmt == 5 ? 17 : nmt == 7 ? 21 : nmt == 10 ? 29 : nmt == 13 ? 41 : 1);
+}
+
 // Instruction descriptor of tcgen05.mma kind::tf32: D FP32, A and B TF32 (FP32
 // bit patterns), both K-major, shape M x N.
 __host__ __device__ constexpr uint32_t umma_idesc_tf32(int M, int N)
@@ -81,12 +95,19 @@ __device__ __forceinline__ void umma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, u
         : "memory");
 }
 
-// FP32 rounded to TF32 (nearest, ties away from zero), as an FP32 bit pattern.
+// FP32 rounded to TF32 (nearest, ties away from zero), as an FP32 bit pattern: what
+// cvt.rna.tf32.f32 gives, on the integer pipe.  A NaN stays one (the carry would turn
+// its pattern into a zero; 0 x NaN keeps it), everything finite is unchanged by the FMA.
 __device__ __forceinline__ uint32_t tf32_rna(float x)
 {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
+    const uint32_t h = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    return __float_as_uint(fmaf(0.f, x, __uint_as_float(h)));
+}
+// The same where x is the remainder of such a rounding (its NaN is already in the
+// other part).
+__device__ __forceinline__ uint32_t tf32_rna_rest(float x)
+{
+    return (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
 }
 
 // Warp-collective: four consecutive 32-bit columns of the warp's 32 lanes.
@@ -147,7 +168,7 @@ __device__ __forceinline__ void net_store4(uint32_t hi_addr, uint32_t lo_addr, i
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         hv[c] = tf32_rna(v[c]);
-        lv[c] = tf32_rna(v[c] - __uint_as_float(hv[c]));
+        lv[c] = tf32_rna_rest(v[c] - __uint_as_float(hv[c]));
     }
     tmem_st4(hi_addr + (uint32_t)col, hv[0], hv[1], hv[2], hv[3]);
     tmem_st4(lo_addr + (uint32_t)col, lv[0], lv[1], lv[2], lv[3]);
