@@ -82,6 +82,7 @@ struct fmc_ctx {
     size_t prof_cap = 0;
     int last_fused_ctas_per_sm = 0;
     int kernel_policy = FMC_KERNEL_AUTO;
+    bool team = true;  // the team kernel may be taken (the server: where its partials were charged)
     std::vector<fmc_launch_rule> rules;  // measured launch shapes (fmc_set_launch_rules)
     // Contexts used on one stream only (the server's) grow their workspace in
     // stream order on that stream (cudaFreeAsync / cudaMallocAsync) instead of
@@ -1142,6 +1143,7 @@ struct Prepared {
     int H = 4;         // its warps per sample (2: two CTAs per SM, nmt slots of 2)
     bool bus = false;  // ... for a system with an infinite bus (its own instantiations)
     bool exclusive = true;  // the launch has the GPU to itself (see fused_shape)
+    bool team = false;      // few samples: the team kernel (see team_wanted)
     int64_t k0 = 0, count = 0;
     std::vector<unsigned char> params;
 };
@@ -1241,6 +1243,37 @@ static int choose_kernel(fmc_ctx* ctx, const std::vector<fmc_launch_rule>* rules
     return FMC_OK;
 }
 
+// Bytes of the team kernel's partials (groups of 32 samples).
+static size_t team_part_bytes(int n, int Nt, int64_t count)
+{
+    return (size_t)((count + TEAM_GROUP - 1) / TEAM_GROUP) * ((size_t)Nt + 1) * 6 * (size_t)n * sizeof(float);
+}
+
+// Whether a fused launch that would take the per-sample kernel takes the team kernel
+// (the same results; simulate_team.cuh): while its groups of 32 samples get an SM each
+// (count <= 32 SMs).  Measured (GB300, 10 machines, 3 disturbances, 1000 steps, the
+// whole call, per-sample -> team): 1000 samples 3.44 -> 2.14 ms, 4864 3.72 -> 2.20,
+// 9728 3.68 -> 4.17; 4000 samples of 1 machine 0.99 -> 0.75, 4 machines 1.36 -> 1.20,
+// 8 machines 2.10 -> 1.68, 12 machines 3.47 -> 2.03.  The same line where other launches
+// share the GPU (four arms of 10007 samples at once: 10.6 ms, by teams 19.5).  Its
+// partials are four times the per-sample kernel's: not past 512 MiB, and not in a
+// context with a memory budget.
+static constexpr size_t TEAM_PART_MAX = (size_t)512 << 20;
+
+static bool team_fits(int sms, int nm, int nmt, int32_t path, int n, int Nt, int64_t count)
+{
+    if (path != FMC_PATH_FUSED || nmt > 0 || nm < 0 || nm > TEAM_MAX_NM) return false;
+    return count <= (int64_t)sms * TEAM_GROUP && team_part_bytes(n, Nt, count) <= TEAM_PART_MAX;
+}
+
+static bool team_wanted(const fmc_ctx* ctx, int nm, int nmt, int32_t path, int n, int Nt, int64_t count,
+                        bool exclusive)
+{
+    if (ctx->budget != 0 || !ctx->team) return false;
+    if (exclusive && ctx->kernel_policy != FMC_KERNEL_AUTO) return false;  // (the per-sample kernel by request)
+    return team_fits(ctx->sms, nm, nmt, path, n, Nt, count);
+}
+
 static int prepare(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s, int64_t k0, int64_t count, int32_t path,
                    cudaStream_t st, Prepared& P, bool exclusive = true)
 {
@@ -1274,6 +1307,7 @@ static int prepare(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s, int64_t k
     P.path = path;
     P.k0 = k0;
     P.count = count;
+    P.team = team_wanted(ctx, P.nm, P.nmt, path, n, Nt, count, exclusive);
     // FP64 Newton on the GPU; its angles come back to the host (one stream
     // synchronisation) to form the integrator's constants in the parameter block
     if ((rc = run_equilibrium_ws(ctx, ws, s, st))) return rc;
@@ -1336,6 +1370,16 @@ static FusedShape fused_shape(const fmc_ctx* ctx, const Prepared& P)
     const bool wide = P.nmt > 0;
     const int64_t full = (P.count + TC_M - 1) / TC_M;
     FusedShape f{TC_M, 4, 32, 0};
+    if (P.team) {
+        // 128 TMEM columns per CTA (256 where 16 steps need them); the chunk only has to
+        // outlast the next one's contraction, which runs beside it
+        const int per = (P.s.forcing == FMC_FORCING_SMOOTH ? 2 : 1) * d;
+        f.rows = TEAM_GROUP;
+        f.TC = (128 / per) & ~15;
+        f.TC = f.TC < 16 ? 16 : (f.TC > 64 ? 64 : f.TC);
+        f.ctas = (P.count + f.rows - 1) / f.rows;
+        return f;
+    }
     if (P.exclusive) {
         const int64_t need = (full + sms - 1) / sms;
         f.max_ctas = wide ? 1 : (need >= 3 ? 4 : (int)(need < 1 ? 1 : need));
@@ -1404,7 +1448,8 @@ static int reserve(fmc_ctx* ctx, Workspace& ws, const Prepared& P, bool want_tra
         if ((rc = ensure(ctx, ws.phi_hi, brows * Kpad * 2))) return rc;
         if (split && (rc = ensure(ctx, ws.phi_lo, brows * Kpad * 2))) return rc;
     }
-    if (per_tile_partials && (rc = ensure(ctx, ws.part, (size_t)ntiles * Nt1 * 3 * S * sizeof(float)))) return rc;
+    if ((per_tile_partials || P.team) && (rc = ensure(ctx, ws.part, (size_t)ntiles * Nt1 * 3 * S * sizeof(float))))
+        return rc;
     return FMC_OK;
 }
 
@@ -1527,7 +1572,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             return rc;
     }
     FMC_CUDA(ctx, cudaMemsetAsync((char*)ws.status.ptr + 4, 0, 4, st), "memset");
-    if (!per_tile_partials) {
+    if (!per_tile_partials && !P.team) {
         FMC_CUDA(ctx, cudaMemsetAsync(S1, 0, Nt1 * S * sizeof(double), st), "memset");
         FMC_CUDA(ctx, cudaMemsetAsync(S2, 0, Nt1 * S * sizeof(double), st), "memset");
     }
@@ -1578,6 +1623,9 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
         } else {
             e = launch_simulate_wide(P.nmt, P.nd, maps, wa, st, &occ);
         }
+    } else if (P.team) {
+        e = launch_simulate_team(P.nm, P.nd, P.params.data(), maps, count, Nt, TC, d, Ks, nkb, split, tmem_cols,
+                                 (float*)ws.part.ptr, traj_dev, (int*)ws.status.ptr + 1, ems, rrf, smooth ? 1 : 0, st);
     } else {
         // a launch that has the GPU to itself keeps as many design tiles in L2 as
         // 60 % of it holds: every chunk re-reads each tile, and the whole design
@@ -1599,7 +1647,16 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
                     tmem_cols);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fused simulation kernel");
     prof_end(pr, st);
-    if (per_tile_partials) {
+    if (P.team) {
+        prof_begin(ctx, PH_REDUCE, st, &pr);
+        const size_t per = (size_t)(count / R + TEAM_GROUP - 1) / TEAM_GROUP * Nt1 * 3 * S;  // floats per design
+        for (int k = 0; k < R; ++k)
+            FMC_CUDA(ctx,
+                     launch_group_sums((const float*)ws.part.ptr + (size_t)k * per, Nt1, S, count / R,
+                                       per_tile_partials, S1 + (size_t)k * Nt1 * S, S2 + (size_t)k * Nt1 * S, st),
+                     "moment sums");
+        prof_end(pr, st);
+    } else if (per_tile_partials) {
         prof_begin(ctx, PH_REDUCE, st, &pr);
         if (R > 1) {
             const int64_t tiles = ntiles / R;
@@ -1678,6 +1735,18 @@ int fmc::simulate_moments_replicates(fmc_ctx* ctx, const fmc_scenario* s, int32_
     return FMC_OK;
 }
 
+size_t fmc::team_bytes(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count)
+{
+    const int Nt = (int)std::llround(s->T / s->dt);
+    const int nm = nm_bucket_for(s->n);
+    return team_fits(ctx->sms, nm, 0, path, s->n, Nt, count) ? team_part_bytes(s->n, Nt, count) : 0;
+}
+
+void fmc::set_team(fmc_ctx* ctx, bool on)
+{
+    if (ctx) ctx->team = on;
+}
+
 void fmc::set_stream_ordered(fmc_ctx* ctx, bool on)
 {
     if (ctx) ctx->stream_ordered = on;
@@ -1721,6 +1790,7 @@ int fmc::reserve_workspace(fmc_ctx* ctx, const fmc_scenario* s, int32_t path, in
     P.exclusive = false;
     P.k0 = 0;
     P.count = count;
+    P.team = team_wanted(ctx, P.nm, P.nmt, path, s->n, Nt, count, false);
     return reserve(ctx, ctx->ws, P, false, path == FMC_PATH_PLAIN);
 }
 

@@ -68,6 +68,12 @@ int release_workspace(fmc_ctx* ctx, cudaStream_t st);
 // (without solving anything), on stream st when the context is stream-ordered.
 int reserve_workspace(fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count, cudaStream_t st);
 
+// Bytes of per-group partials that simulate_moments of `count` samples of s holds
+// beyond the design and basis (the team kernel's), 0 where it takes another kernel;
+// and whether ctx may take that kernel.
+size_t team_bytes(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count);
+void set_team(fmc_ctx* ctx, bool on);
+
 // fmc_simulate with a choice of how the fused kernel combines its per-time sums:
 // per_tile_partials = true writes FP32 partials per 128-sample tile and adds them
 // in a fixed order (deterministic); false adds them with FP64 atomics (no

@@ -83,10 +83,22 @@ cudaError_t launch_simulate_fused(int nm_bucket, int nd_bucket, const void* para
                                   int rows, int max_ctas, const double* eq, float* part, double* S1, double* S2,
                                   float* traj, int* err, const EmSpec& em, double* rrf, const L2Keep& keep,
                                   int smooth, cudaStream_t st, int* max_ctas_per_sm);
+// Few samples of up to 12 machines: the team kernel (simulate_team.cuh), 32 samples
+// per CTA; part [groups of 32][Nt+1][3][2n]; maps as above with design boxes of 32 rows
+constexpr int TEAM_GROUP = 32, TEAM_MAX_NM = 12;
+cudaError_t launch_simulate_team(int nm_bucket, int nd_bucket, const void* params, const CUtensorMap* maps,
+                                 int64_t count, int Nt, int TC, int d, int Ks, int nkb, int split, uint32_t tmem_cols,
+                                 float* part, float* traj, int* err, const EmSpec& em, double* rrf, int smooth,
+                                 cudaStream_t st);
 cudaError_t launch_moments(const float* x, int64_t N, int64_t C, double* mean, double* var, int sms, cudaStream_t st);
 cudaError_t launch_traj_sums(const float* x, int64_t N, int64_t C, const double* shift, int S, double* S1, double* S2,
                              int sms, cudaStream_t st);
 cudaError_t launch_fused_sums(const float* part, int nblk, int64_t Nt1, int S, int64_t count, int rows, double* S1,
+                              double* S2, cudaStream_t st);
+// the same from the partials of groups of 32 samples (four to a tile); merge: tiles
+// merged in FP32 as launch_fused_sums does, else added one by one in FP64 (what the
+// per-sample kernel's atomics add)
+cudaError_t launch_group_sums(const float* part, int64_t Nt1, int S, int64_t count, bool merge, double* S1,
                               double* S2, cudaStream_t st);
 cudaError_t launch_finalize(const double* S1, const double* S2, const double* shift, int64_t N, int64_t Nt1, int S,
                             double* mean, double* var, cudaStream_t st);

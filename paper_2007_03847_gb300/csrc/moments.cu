@@ -152,8 +152,31 @@ cudaError_t launch_traj_sums(const float* x, int64_t N, int64_t C, const double*
 // One thread per (t, j); a CTA owns 32 consecutive pairs, its 8 warps stride
 // over the groups (warp g takes groups g, g+8, ...), and the 8 partial sums are
 // added in warp order, so the result does not depend on scheduling.
+// GROUPED: the partials are of groups of 32 samples; four are first combined into
+// their tile's triple (combine_groups, as the per-sample kernel's flush does).
+// MERGE false: every tile enters FP64 on its own (with GROUPED; what the per-sample
+// kernel's FP64 atomics add up).
 constexpr int FS_COLS = 32, FS_GROUPS = 8, FS_G = 8;
 
+struct SumTriple {
+    float c, dv, m2;
+};
+
+template <bool GROUPED>
+__device__ __forceinline__ SumTriple sum_triple(const float* p, int64_t blk, int S, int b, int64_t count)
+{
+    if constexpr (GROUPED) {
+        const float* g = p + 4 * (int64_t)b * blk;
+        SumTriple t;
+        combine_groups(g, g + S, g + 2 * S, (int)blk, count - 128 * (int64_t)b, 4, &t.c, &t.dv, &t.m2);
+        return t;
+    } else {
+        const float* q = p + (int64_t)b * blk;
+        return SumTriple{q[0], q[S], q[2 * S]};
+    }
+}
+
+template <bool GROUPED, bool MERGE>
 __global__ void __launch_bounds__(FS_COLS * FS_GROUPS) fused_sums_kernel(const float* __restrict__ part, int nblk,
                                                                          int64_t Nt1, int S, int64_t count, int rows,
                                                                          double* __restrict__ S1o,
@@ -162,7 +185,7 @@ __global__ void __launch_bounds__(FS_COLS * FS_GROUPS) fused_sums_kernel(const f
     __shared__ double red1[FS_GROUPS][FS_COLS], red2[FS_GROUPS][FS_COLS];
     const int cx = threadIdx.x % FS_COLS, g = threadIdx.x / FS_COLS;
     const int64_t total = Nt1 * S;        // (t, j) pairs
-    const int64_t blk = Nt1 * 3 * S;      // floats per block
+    const int64_t blk = Nt1 * 3 * S;      // floats per block (group)
     const int64_t q = (int64_t)blockIdx.x * FS_COLS + cx;
     double a1 = 0.0, a2 = 0.0;
     if (q < total) {
@@ -170,19 +193,20 @@ __global__ void __launch_bounds__(FS_COLS * FS_GROUPS) fused_sums_kernel(const f
         const int j = (int)(q - t * S);
         const float* p = part + t * 3 * S + j;  // c at p[0], dv at p[S], m2 at p[2 S] of block 0
         const int64_t last_n = count - (int64_t)(nblk - 1) * rows;
-        const int nfull = last_n == rows ? nblk : nblk - 1;  // blocks of `rows` samples
+        const int nfull = MERGE ? (last_n == rows ? nblk : nblk - 1) : 0;  // blocks of `rows` samples, merged
         const float fn = (float)rows, inv_n = 1.f / (float)rows;
         for (int g0 = g * FS_G; g0 < nfull; g0 += FS_GROUPS * FS_G) {
             const int gc = nfull - g0 < FS_G ? nfull - g0 : FS_G;
-            const float cg = p[(int64_t)g0 * blk];
+            float cg = 0.f;
             float dl[FS_G], hi = 0.f, lo = 0.f, mt = 0.f;
 #pragma unroll
             for (int k = 0; k < FS_G; ++k) {
                 dl[k] = 0.f;
                 if (k < gc) {
-                    const float* pb = p + (int64_t)(g0 + k) * blk;
-                    dl[k] = fmaf(fn, pb[0] - cg, pb[S]);
-                    mt += pb[2 * S];
+                    const SumTriple b = sum_triple<GROUPED>(p, blk, S, g0 + k, count);
+                    if (k == 0) cg = b.c;
+                    dl[k] = fmaf(fn, b.c - cg, b.dv);
+                    mt += b.m2;
                     // two-sum: hi + lo carries the exact sum of the dl
                     const float tt = hi + dl[k];
                     const float z = tt - hi;
@@ -203,13 +227,17 @@ __global__ void __launch_bounds__(FS_COLS * FS_GROUPS) fused_sums_kernel(const f
             a1 += s1;
             a2 += (double)fmaf(dd, inv_n, mt) + s1 * s1 / ng;
         }
-        // the partial last block, by the warp whose turn it would be
-        if (nfull < nblk && g == (nfull / FS_G) % FS_GROUPS) {
-            const float* pb = p + (int64_t)(nblk - 1) * blk;
-            const double s1 = fma((double)last_n, (double)pb[0], (double)pb[S]);
-            a1 += s1;
-            a2 += (double)pb[2 * S] + s1 * s1 / (double)last_n;
-        }
+        // the partial last block, by the warp whose turn it would be (without MERGE:
+        // every block in turn)
+        const int first = MERGE ? nfull : g, stride = MERGE ? nblk : FS_GROUPS;
+        if (!MERGE || g == (nfull / FS_G) % FS_GROUPS)
+            for (int bb = first; bb < nblk; bb += stride) {
+                const SumTriple b = sum_triple<GROUPED>(p, blk, S, bb, count);
+                const double nb = (double)(bb < nblk - 1 ? rows : last_n);
+                const double s1 = fma(nb, (double)b.c, (double)b.dv);
+                a1 += s1;
+                a2 += (double)b.m2 + s1 * s1 / nb;
+            }
     }
     red1[g][cx] = a1;
     red2[g][cx] = a2;
@@ -230,8 +258,21 @@ cudaError_t launch_fused_sums(const float* part, int nblk, int64_t Nt1, int S, i
                               double* S2, cudaStream_t st)
 {
     const int64_t total = Nt1 * S;
-    fused_sums_kernel<<<(unsigned)((total + FS_COLS - 1) / FS_COLS), FS_COLS * FS_GROUPS, 0, st>>>(
+    fused_sums_kernel<false, true><<<(unsigned)((total + FS_COLS - 1) / FS_COLS), FS_COLS * FS_GROUPS, 0, st>>>(
         part, nblk, Nt1, S, count, rows, S1, S2);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_group_sums(const float* part, int64_t Nt1, int S, int64_t count, bool merge, double* S1,
+                              double* S2, cudaStream_t st)
+{
+    const int64_t total = Nt1 * S;
+    const int tiles = (int)((count + 127) / 128);
+    // (the combine indexes a tile's groups with 32-bit offsets)
+    if (Nt1 * 3 * S * 4 > 2147483647LL) return cudaErrorInvalidValue;
+    auto kern = merge ? fused_sums_kernel<true, true> : fused_sums_kernel<true, false>;
+    kern<<<(unsigned)((total + FS_COLS - 1) / FS_COLS), FS_COLS * FS_GROUPS, 0, st>>>(part, tiles, Nt1, S, count, 128,
+                                                                                      S1, S2);
     return cudaGetLastError();
 }
 

@@ -32,6 +32,7 @@ struct Request {
     double* mean = nullptr;
     double* var = nullptr;
     size_t bytes = 0;  // device memory charged against the budget
+    bool team = true;  // the team kernel's partials are part of the charge
     int status = FMC_NOT_READY;
     bool started = false;
     std::string error;
@@ -263,7 +264,9 @@ static void worker_loop(fmc_server* srv, int slot)
             r->started = true;
             r->t_start = Clock::now();
         }
-        // moments summed with FP64 atomics: no per-tile partial buffers to hold
+        // moments summed with FP64 atomics (no per-tile partial buffers to hold), or
+        // by the team kernel where its partials were charged
+        for (int k = 0; k < kReplicates; ++k) fmc::set_team(rctx[k], r->team);
         int rc;
         if (r->tol_E > 0 || r->tol_Var > 0) {
             rc = run_target(rctx, rst, r);
@@ -386,6 +389,18 @@ static int submit_request(fmc_server* srv, const fmc_scenario* scen, int32_t pat
     }
     r->bytes = request_bytes(largest, path) * (target ? (size_t)kReplicates : 1u) +
                (n_mm > 0 ? (size_t)merged_part_bytes(*scen, kReplicates * n_mm) : 0u);
+    // small designs take the team kernel, whose partials are charged for the largest
+    // round that takes it; a request they alone would put past the budget does without
+    size_t team = 0;
+    for (int64_t n = scen->N; n <= largest.N; n *= 4) {
+        const size_t t = !target     ? fmc::team_bytes(srv->ctxs[0], scen, path, n)
+                         : n <= n_mm ? fmc::team_bytes(srv->ctxs[0], scen, path, kReplicates * n)
+                                     : kReplicates * fmc::team_bytes(srv->ctxs[0], scen, path, n);
+        team = t > team ? t : team;
+        if (!target) break;
+    }
+    r->team = r->bytes + team <= srv->budget;
+    if (r->team) r->bytes += team;
     r->t_submit = Clock::now();
     std::lock_guard<std::mutex> lk(srv->mu);
     if (srv->stopping) return FMC_ECANCELLED;
