@@ -126,6 +126,7 @@ struct WideArgs {
     double* rrf;          // [2]: sums of the response function and its square, or nullptr
     ItoParams<8> ito;     // general disturbances (ito.on == 0: all OU)
 };
+    const float* rows;    // host copy of its per-machine rows (tensor-core form; read by the launcher)
 
 __host__ __device__ constexpr int wide_nmtp(int nmt) { return (nmt + 3) & ~3; }
 

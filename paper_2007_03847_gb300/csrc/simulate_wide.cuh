@@ -83,20 +83,46 @@ __device__ __forceinline__ float2 wide_gamma_eta_tier(float x, float cs, float s
 // the hot loops keep their registers).
 static __device__ __noinline__ void bus_deviation(float c, float* cm1, float* sn) { sin_cosm1_any(c, sn, cm1); }
 
+// The tensor-core form's per-machine constants: slot k of the warps h as (cos D*, sin D*,
+// u*, v*), (delta*, 1/(2H), D, H / sum H), then the injection row.  With four warps per
+// sample they are constant-bank reads of the kernel's parameter block (50 machines 26.6
+// -> 23.8 ms: from shared memory a 16-byte broadcast takes four passes of the SM's one
+// load pipe); with two they come from shared memory all the same (20 machines 23.8 ms
+// against 24.6, 27 machines 17.0 against 21.0: the constant loads' latency shows).
+template <int NMT, int ND, bool TCN, int H>
+struct WideConsts {
+    static constexpr bool PARAM = TCN && H == 4;
+    static constexpr int C4 = 2 + (ND + 3) / 4;
+    float4 c[PARAM ? H : 1][PARAM ? NMT : 1][PARAM ? C4 : 1];
+};
+template <class WC>
+struct WideConstsRef {
+    const WC& wc;
+    const float4* s;  // [machine][C4] in shared memory
+    int h, H;
+    __device__ __forceinline__ float4 get(int k, int v) const
+    {
+        if constexpr (WC::PARAM)
+            return wc.c[h][k][v];
+        else
+            return s[(h + H * k) * WC::C4 + v];
+    }
+};
+
 // Warp-collective (tensor-core network sum): (gamma, eta) of the deviations
 // x[k] - csh of the warp's machines by the series of tier TIER, split and stored
 // pairwise to the warp's A_hi, A_lo columns; waits for the stores.  Slot nb (an
 // infinite bus, or -1) takes the bus's (bcm, -bsn) = (cos csh - 1, -sin csh).
-template <int NMT, int TIER, int CST, int H>
+template <int NMT, int TIER, int H, class WC>
 __device__ __forceinline__ void publish_tier(uint32_t hi, uint32_t lo, const float (&x)[NMT], float csh,
-                                             const float* cst_s, int h, int n, int nb, float bcm, float bsn)
+                                             const WC& wc, int h, int n, int nb, float bcm, float bsn)
 {
     constexpr int KREAL = (wide_tc_min_n(NMT, H) - H) / H + 1;  // slots that hold a machine in every such layout
     float pg = 0.f, pe = 0.f;
 #pragma unroll
     for (int k = 0; k < NMT; ++k) {
         const int i = h + H * k;
-        const float2 csn = *reinterpret_cast<const float2*>(cst_s + i * CST);
+        const float4 csn = wc.get(k, 0);
         float sn, cm1;
         deviation_trig1<TIER>(x[k] - csh, &sn, &cm1);
         const bool bus = k == NMT - 1 && i == nb;  // (the bus holds a warp's last slot)
@@ -115,9 +141,9 @@ __device__ __forceinline__ void publish_tier(uint32_t hi, uint32_t lo, const flo
 
 // The same with one tier for all of the warp's machines, from their largest
 // shifted deviation (the tiers of wide_gamma_eta_tier).
-template <int NMT, int CST, int H>
+template <int NMT, int H, class WC>
 __device__ __forceinline__ void publish_angles(uint32_t hi, uint32_t lo, const float (&x)[NMT], float csh,
-                                               const float* cst_s, int h, int n, int nb)
+                                               const WC& wc, int h, int n, int nb)
 {
     float bcm = 0.f, bsn = 0.f;
     if (nb >= 0 && nb % H == h) bus_deviation(csh, &bcm, &bsn);
@@ -128,13 +154,13 @@ __device__ __forceinline__ void publish_angles(uint32_t hi, uint32_t lo, const f
         if (k < KREAL || h + H * k < n) m = fmaxf(m, fabsf(x[k] - csh));
     const uint32_t mm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
     if (mm <= __float_as_uint(0.05f))
-        publish_tier<NMT, 0, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
+        publish_tier<NMT, 0, H>(hi, lo, x, csh, wc, h, n, nb, bcm, bsn);
     else if (mm <= __float_as_uint(0.25f))
-        publish_tier<NMT, 1, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
+        publish_tier<NMT, 1, H>(hi, lo, x, csh, wc, h, n, nb, bcm, bsn);
     else if (mm <= __float_as_uint(0.8f))
-        publish_tier<NMT, 2, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
+        publish_tier<NMT, 2, H>(hi, lo, x, csh, wc, h, n, nb, bcm, bsn);
     else
-        publish_tier<NMT, 3, CST, H>(hi, lo, x, csh, cst_s, h, n, nb, bcm, bsn);
+        publish_tier<NMT, 3, H>(hi, lo, x, csh, wc, h, n, nb, bcm, bsn);
 }
 
 // The (gamma, eta) of the next stage input (one A buffer: wide_tc_stash) into the
@@ -142,8 +168,8 @@ __device__ __forceinline__ void publish_angles(uint32_t hi, uint32_t lo, const f
 // the series of each machine's own tier (wide_gamma_eta_tier); else (a step's) that of
 // all of the warp's machines, as publish_angles takes it.  Both ask first whether the
 // shortest series will do for all.
-template <int NMT, int CST, int H>
-__device__ __forceinline__ void stash_angles(float* row, const float (&x)[NMT], float csh, const float* cst_s, int h,
+template <int NMT, int H, class WC>
+__device__ __forceinline__ void stash_angles(float* row, const float (&x)[NMT], float csh, const WC& wc, int h,
                                              int n, int nb, bool pub)
 {
     constexpr int KREAL = (wide_tc_min_n(NMT, H) - H) / H + 1;
@@ -161,7 +187,7 @@ __device__ __forceinline__ void stash_angles(float* row, const float (&x)[NMT], 
     auto put = [&](int k, float sn, float cm1) {
         const int i = h + H * k;
         const bool real = k < KREAL || i < n;
-        const float2 csn = *reinterpret_cast<const float2*>(cst_s + i * CST);
+        const float4 csn = wc.get(k, 0);
         const bool bus = k == NMT - 1 && i == nb;
         row[2 * k] = real ? fmaf(csn.x, cm1, -csn.y * sn) : (bus ? bcm : 0.f);
         row[2 * k + 1] = real ? fmaf(csn.y, cm1, csn.x * sn) : (bus ? -bsn : 0.f);
@@ -196,7 +222,7 @@ __device__ __forceinline__ void stash_angles(float* row, const float (&x)[NMT], 
             sin_cosm1_any(y, &sn, &cm1);
         const int i = h + H * k;
         const bool real = i < n, bus = k == NMT - 1 && i == nb;
-        const float2 csn = *reinterpret_cast<const float2*>(cst_s + i * CST);
+        const float4 csn = wc.get(k, 0);
         row[2 * k] = real ? fmaf(csn.x, cm1, -csn.y * sn) : (bus ? bcm : 0.f);
         row[2 * k + 1] = real ? fmaf(csn.y, cm1, csn.x * sn) : (bus ? -bsn : 0.f);
     }
@@ -210,7 +236,8 @@ template <int NMT, int ND, bool TCN, int H = 4, bool BUS = false>
 __global__ void __launch_bounds__(H * 128, 4 / H)
     simulate_wide_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                          const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
-                         const __grid_constant__ CUtensorMap mN, const __grid_constant__ WideArgs a)
+                         const __grid_constant__ CUtensorMap mN, const __grid_constant__ WideArgs a,
+                         const __grid_constant__ WideConsts<NMT, ND, TCN, H> wcp)
 {
     constexpr int NMTP = wide_nmtp(NMT);
     constexpr int KP = NMT > 10 ? 8 : NMT;  // machine slots per pass over the network sum
@@ -230,7 +257,8 @@ __global__ void __launch_bounds__(H * 128, 4 / H)
     __shared__ int abort_flag;
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int q = warp & 3, h = warp >> 2;
+    const int q = warp & 3;
+    const int h = __shfl_sync(0xffffffffu, warp >> 2, 0);  // (uniform: constants are addressed by it)
     const int n = a.n, d = a.d, S = 2 * n, S3 = 3 * S;
     constexpr int GS = 6 * NMT;  // floats per (step, sample group, h) slot: ref | dev | m2 of 2 NMT states
     const int r = 32 * q + lane;  // sample row within the tile = TMEM lane
@@ -272,25 +300,22 @@ __global__ void __launch_bounds__(H * 128, 4 / H)
     float* racc_s = w0buf + 256;                                        // [128] (warps h = 0)
     // TCN: [2][4 (h)][128] partial sums of a stage input's deviations over the warp's machines
     float* cpart = w0buf + 384;
-    float* cst_s = w0buf + 384 + (TCN ? 1024 : 0);
+    using WC = WideConsts<NMT, ND, TCN, H>;
+    float* cst_s = w0buf + 384 + (TCN ? 1024 : 0);  // the constant block (FP32 form), or its per-machine rows
     const int dx = a.dx;
-    // TCN keeps only the per-machine rows (the network is in net_s), transposed to
-    // [4 NMT][CST] so that a machine's constants are a few 16-byte loads:
-    // (cos D*, sin D*, u*, v*), (delta*, 1/(2H), D, H / sum H), injection row
-    constexpr int CST = (8 + ND + 3) & ~3;
-    const int nskip = TCN ? 2 * n * 4 * NMTP : 0;
-    const int nconst = wide_const_floats(n, NMT, ND) - nskip;
-    for (int e = tid; e < nconst; e += NTHR) {
-        if (TCN) {
+    if (!TCN) {
+        for (int e = tid; e < wide_const_floats(n, NMT, ND); e += NTHR) cst_s[e] = a.consts[e];
+    } else if (!WC::PARAM) {
+        const int skip = 2 * n * 4 * NMTP;
+        for (int e = tid; e < (8 + ND) * G4; e += NTHR) {
             const int row = e / G4, i = e - row * G4;
-            cst_s[i * CST + row] = a.consts[nskip + e];
-        } else {
-            cst_s[e] = a.consts[nskip + e];
+            cst_s[i * 4 * WC::C4 + row] = a.consts[skip + e];
         }
     }
+    const WideConstsRef<WC> wc{wcp, reinterpret_cast<const float4*>(cst_s), h, H};
     // [j][h][GE row of NMTP | BE row of NMTP]: one address serves both rows
     const float* GB = cst_s;
-    const float* pm = cst_s + 2 * n * 4 * NMTP - nskip;
+    const float* pm = cst_s + 2 * n * 4 * NMTP;
     const float* c_cst = pm;
     const float* c_sst = pm + G4;
     const float* c_ust = pm + 2 * G4;
@@ -298,9 +323,9 @@ __global__ void __launch_bounds__(H * 128, 4 / H)
     const float* c_i2h = pm + 5 * G4;
     const float* c_D = pm + 6 * G4;
     const float* c_inj = pm + 8 * G4;  // [dx][4 NMT]
-    // constant `row` (0 cos D*, 1 sin D*, 2 u*, 3 v*, 4 delta*, 5 1/(2H), 6 D, 7 H / sum H,
-    // 8.. injection) of machine slot i, in either layout
-    auto cst = [&](int row, int i) -> float { return TCN ? cst_s[i * CST + row] : pm[row * G4 + i]; };
+    // delta* and H / sum H of machine slot k of this warp, in either layout
+    auto cst_delta = [&](int k) -> float { return TCN ? wc.get(k, TCN ? 1 : 0).x : pm[4 * G4 + h + H * k]; };
+    auto cst_coi = [&](int k) -> float { return TCN ? wc.get(k, TCN ? 1 : 0).w : pm[7 * G4 + h + H * k]; };
     // per step and warp, the partial centre-of-inertia speed of the warp's machines
     float* coi_part = msum + WI_MS * 4 * H * GS;  // [WI_MS][H (h)][128]
 
@@ -363,7 +388,7 @@ __global__ void __launch_bounds__(H * 128, 4 / H)
         for (int k = 0; k < NMT; ++k) {
             const int i = h + H * k;
             if (i < n) {
-                traj[i] = cst(4, i);
+                traj[i] = cst_delta(k);
                 traj[n + i] = 0.f;
             }
         }
@@ -549,9 +574,9 @@ if constexpr (TCN) {
                         ps += (k < KREAL || h + H * k < n) ? yn[k] : 0.f;
                     }
                     if constexpr (AB2) {
-                        publish_angles<NMT, CST, H>(a_hi + an, a_lo + an, yn, csh, cst_s, h, n, nb);
+                        publish_angles<NMT, H>(a_hi + an, a_lo + an, yn, csh, wc, h, n, nb);
                     } else {
-                        stash_angles<NMT, CST, H>(wbuf + lane * WROW, yn, csh, cst_s, h, n, nb, pub);
+                        stash_angles<NMT, H>(wbuf + lane * WROW, yn, csh, wc, h, n, nb, pub);
                     }
                     cpart[(gb ^ 1) * (H * 128) + h * 128 + r] = ps;
                 }
@@ -605,7 +630,7 @@ if constexpr (TCN) {
                         const int c = 2 * (k % RP);
                         const float du = dd[c], dv = dd[c + 1];
                         const float gi = ah[c] + al[c], ei = ah[c + 1] + al[c + 1];
-                        const float4 ca = *reinterpret_cast<const float4*>(cst_s + i * CST);
+                        const float4 ca = wc.get(k, 0);
                         const float cs = ca.x, ss = ca.y;
                         float dpe = fmaf(cs, du, ss * dv);
                         dpe = fmaf(gi, ca.z + du, dpe);
@@ -614,13 +639,13 @@ if constexpr (TCN) {
 #pragma unroll
                         for (int e4 = 0; e4 < ND; e4 += 4) {
                             // rows past the slots in use are zero
-                            const float4 cj = *reinterpret_cast<const float4*>(cst_s + i * CST + 8 + e4);
+                            const float4 cj = wc.get(k, 2 + e4 / 4);
                             const float cjv[4] = {cj.x, cj.y, cj.z, cj.w};
 #pragma unroll
                             for (int e = e4; e < ND && e < e4 + 4; ++e) f = fmaf(cjv[e - e4], xs[e], f);
                         }
                         // delta*, 1/(2H), D, H / sum H
-                        const float4 cb = *reinterpret_cast<const float4*>(cst_s + i * CST + 4);
+                        const float4 cb = wc.get(k, 1);
                         const float kw = (f - dpe - cb.z * yw[k]) * cb.y;
                         if constexpr (!EARLY) {
                             const float kd = a.omega_s * (yw[k] - w0);
@@ -827,7 +852,7 @@ if constexpr (TCN) {
                 float ps = 0.f;
 #pragma unroll
                 for (int k = 0; k < NMT; ++k) ps += (k < KREAL || h + H * k < n) ? del[k] : 0.f;
-                publish_angles<NMT, CST, H>(a_hi, a_lo, del, csh, cst_s, h, n, nb);
+                publish_angles<NMT, H>(a_hi, a_lo, del, csh, wc, h, n, nb);
                 cpart[(gb ^ 1) * (H * 128) + h * 128 + r] = ps;
                 if (h == 0) w0buf[(gb ^ 1) * 128 + r] = w[0];
                 gb ^= 1;
@@ -850,7 +875,7 @@ if constexpr (TCN) {
                 for (int k = 0; k < NMT; ++k) {
                     const int i = h + H * k;
                     if (i < n) {
-                        o[i] = (theta + del[k]) + cst(4, i);
+                        o[i] = (theta + del[k]) + cst_delta(k);
                         o[n + i] = w[k];
                     }
                 }
@@ -878,7 +903,7 @@ if constexpr (TCN) {
             if (a.rrf) {
                 float cp = 0.f;
 #pragma unroll
-                for (int k = 0; k < NMT; ++k) cp = fmaf(cst(7, h + H * k), w[k], cp);
+                for (int k = 0; k < NMT; ++k) cp = fmaf(cst_coi(k), w[k], cp);
                 coi_part[(ms * H + h) * 128 + r] = cp;
             }
             __syncwarp();
@@ -939,7 +964,8 @@ inline int wide_smem_bytes(int TC, int split, int n, int ns)
     const int mom = wide_mom_floats<NMT, H>() * 4;
     const int u = ((ns * stage > mom ? ns * stage : mom) + 1023) & ~1023;
     if (TCN)
-        return 1024 + u + wide_tc_net_bytes(NMT, H) + (384 + 1024) * 4 + 4 * NMT * ((8 + ND + 3) & ~3) * 4;
+        return 1024 + u + wide_tc_net_bytes(NMT, H) + (384 + 1024) * 4 +
+               (WideConsts<NMT, ND, TCN, H>::PARAM ? 0 : 4 * NMT * WideConsts<NMT, ND, TCN, H>::C4 * 16);
     return 1024 + u + 2 * n * 128 * 8 + 384 * 4 + wide_const_floats(n, NMT, ND) * 4;
 }
 
@@ -948,6 +974,13 @@ inline int wide_smem_bytes(int TC, int split, int n, int ns)
 template <int NMT, int ND, bool TCN = false, int H = 4, bool BUS = false>
 cudaError_t launch_wide_t(const CUtensorMap* maps, const WideArgs& args, cudaStream_t st, int* occ_out)
 {
+    WideConsts<NMT, ND, TCN, H> wc{};
+    if constexpr (WideConsts<NMT, ND, TCN, H>::PARAM)
+        for (int h = 0; h < H; ++h)
+            for (int k = 0; k < NMT; ++k) {
+                float* c = reinterpret_cast<float*>(wc.c[h][k]);
+                for (int row = 0; row < 8 + ND; ++row) c[row] = args.rows[row * 4 * NMT + h + H * k];
+            }
     static_assert(!BUS || (TCN && H == 4), "the infinite-bus form is built for four warps per sample");
     // (the tensor-core form shifts the angles: exact with a network alone, or with
     // the infinite bus held in its slot)
@@ -972,7 +1005,7 @@ cudaError_t launch_wide_t(const CUtensorMap* maps, const WideArgs& args, cudaStr
     if (occ < 1 || (uint32_t)occ * a.tmem_cols > 512u) return cudaErrorInvalidConfiguration;
     const int64_t ntiles = (a.count + TC_M - 1) / TC_M;
     if (ntiles > 2147483647LL) return cudaErrorInvalidValue;
-    kern<<<(unsigned)ntiles, H * 128, smem, st>>>(maps[0], maps[1], maps[2], maps[3], maps[TCN ? 4 : 0], a);
+    kern<<<(unsigned)ntiles, H * 128, smem, st>>>(maps[0], maps[1], maps[2], maps[3], maps[TCN ? 4 : 0], a, wc);
     return cudaGetLastError();
 }
 
