@@ -1326,11 +1326,11 @@ static int prepare(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s, int64_t k
         // (outside any stream capture)
         std::vector<float> wc;
         build_wide_consts(s, delta0.data(), P.nmt, P.nd, P.tcn, P.H, wc);
-        if ((rc = ensure(ctx, ws.wconst, wc.size() * sizeof(float)))) return rc;
         // the per-machine rows stay on the host too: the launches pass them as parameters
         const float* rows = wc.data() + 2 * (size_t)n * 4 * wide_nmtp(P.nmt);
         P.params.resize((8 + (size_t)P.nd) * 4 * P.nmt * sizeof(float));
         memcpy(P.params.data(), rows, P.params.size());
+        if ((rc = ensure(ctx, ws.wconst, wc.size() * sizeof(float)))) return rc;
         FMC_CUDA(ctx, cudaMemcpyAsync(ws.wconst.ptr, wc.data(), wc.size() * sizeof(float), cudaMemcpyHostToDevice, st),
                  "copy constants");
         FMC_CUDA(ctx, cudaStreamSynchronize(st), "sync");
@@ -1603,6 +1603,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             wa.ou_s[q] = (float)s->sigma[q];
         }
         wa.consts = (const float*)ws.wconst.ptr;
+        wa.rows = reinterpret_cast<const float*>(P.params.data());
         wa.part = per_tile_partials ? (float*)ws.part.ptr : nullptr;
         wa.S1 = per_tile_partials ? nullptr : S1;
         wa.S2 = per_tile_partials ? nullptr : S2;
@@ -1669,7 +1670,6 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
                          launch_fused_sums((const float*)ws.part.ptr + (size_t)k * tiles * Nt1 * 3 * S, (int)tiles,
                                            Nt1, S, count / R, shape.rows, S1 + (size_t)k * Nt1 * S,
                                            S2 + (size_t)k * Nt1 * S, st),
-        wa.rows = reinterpret_cast<const float*>(P.params.data());
                          "moment sums");
         } else {
             FMC_CUDA(ctx, launch_fused_sums((const float*)ws.part.ptr, (int)ntiles, Nt1, S, count, shape.rows, S1, S2, st),

@@ -115,6 +115,7 @@ struct WideArgs {
     float omega_s, dt;
     float ou_a[8], ou_s[8];
     const float* consts;  // device copy of the constant block (wide_const_floats floats)
+    const float* rows;    // host copy of its per-machine rows (tensor-core form; read by the launcher)
     float* part;          // [tiles][Nt+1][4n], or nullptr: add into S1, S2 with FP64 atomics
     double* S1;           // [Nt+1][2n] when part == nullptr
     double* S2;
@@ -126,7 +127,6 @@ struct WideArgs {
     double* rrf;          // [2]: sums of the response function and its square, or nullptr
     ItoParams<8> ito;     // general disturbances (ito.on == 0: all OU)
 };
-    const float* rows;    // host copy of its per-machine rows (tensor-core form; read by the launcher)
 
 __host__ __device__ constexpr int wide_nmtp(int nmt) { return (nmt + 3) & ~3; }
 
