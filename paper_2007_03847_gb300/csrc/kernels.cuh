@@ -76,13 +76,24 @@ struct L2Keep {
     int64_t row_bytes;
     int tiles;
 };
+// The sliced form of a fused launch (FusedArgs): a grid of `ctas` (0: one CTA per tile)
+// takes the tiles from a ticket, the last ntiles - whole of them `steps` at a time.
+// ticket: 1 + ntiles - whole words; state: fused_state_floats x rows floats per sliced tile
+struct SlicePlan {
+    int ctas;
+    int64_t whole;
+    int steps;
+    uint32_t* ticket;
+    float* state;
+};
+size_t fused_state_floats(int nm_bucket, int nd_bucket);
 // rows: samples per CTA, 128 (four warps) or 64 (two warps); max_ctas: resident
 // CTAs per SM allowed (further limited by the TMEM columns)
 cudaError_t launch_simulate_fused(int nm_bucket, int nd_bucket, const void* params, const CUtensorMap* maps,
                                   int64_t count, int Nt, int TC, int d, int Ks, int nkb, int split, uint32_t tmem_cols,
                                   int rows, int max_ctas, const double* eq, float* part, double* S1, double* S2,
                                   float* traj, int* err, const EmSpec& em, double* rrf, const L2Keep& keep,
-                                  int smooth, cudaStream_t st, int* max_ctas_per_sm);
+                                  int smooth, const SlicePlan& slices, cudaStream_t st, int* max_ctas_per_sm);
 // Few samples of up to 12 machines: the team kernel (simulate_team.cuh), 32 samples
 // per CTA; part [groups of 32][Nt+1][3][2n]; maps as above with design boxes of 32 rows
 constexpr int TEAM_GROUP = 32, TEAM_MAX_NM = 12;

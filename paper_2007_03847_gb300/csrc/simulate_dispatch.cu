@@ -76,6 +76,8 @@ int fused_ring_stages(int TC, int split, int max_ctas_per_sm, int rows)
     return ns < 2 ? 2 : (ns > TC_MAX_STAGES ? TC_MAX_STAGES : ns);
 }
 
+size_t fused_state_floats(int nm_bucket, int nd_bucket) { return (size_t)fu_state(nm_bucket, nd_bucket); }
+
 int fused_smem_bytes(int nm_bucket, int TC, int split, int max_ctas_per_sm, int rows)
 {
     const int stage = (rows * 64 + TC * 64) * (split ? 2 : 1);
@@ -93,17 +95,29 @@ cudaError_t launch_simulate_fused(int nm_bucket, int nd_bucket, const void* para
                                   int64_t count, int Nt, int TC, int d, int Ks, int nkb, int split, uint32_t tmem_cols,
                                   int rows, int max_ctas, const double* eq, float* part, double* S1, double* S2,
                                   float* traj, int* err, const EmSpec& em, double* rrf, const L2Keep& keep,
-                                  int smooth, cudaStream_t st, int* max_ctas_per_sm)
+                                  int smooth, const SlicePlan& slices, cudaStream_t st, int* max_ctas_per_sm)
 {
     if (rows != TC_M && rows != TC_M / 2) return cudaErrorInvalidValue;
     int cap = (int)(512u / tmem_cols) < max_ctas ? (int)(512u / tmem_cols) : max_ctas;
     const int cw = smooth ? 2 * TC : TC;  // basis rows of a chunk (the smooth form's half steps)
     FusedArgs a{count, Nt, TC, d, Ks, nkb, split, fused_ring_stages(cw, split, cap, rows), tmem_cols, eq, part,
                 traj, err, S1, S2, em, rrf, static_cast<const uint8_t*>(keep.hi), static_cast<const uint8_t*>(keep.lo),
-                keep.row_bytes, keep.tiles, smooth};
+                keep.row_bytes, keep.tiles, smooth, 0, 0, 0, 0, nullptr, nullptr};
     const int smem = fused_smem_bytes(nm_bucket, cw, split, cap, rows);
-    const int64_t ntiles = (count + rows - 1) / rows;
+    int64_t ntiles = (count + rows - 1) / rows;
     if (ntiles > 2147483647LL) return cudaErrorInvalidValue;
+    if (slices.ctas > 0) {
+        a.ntiles = ntiles;
+        a.whole = slices.whole;
+        a.slice = slices.steps;
+        a.nslice = (Nt + slices.steps - 1) / slices.steps;
+        a.ticket = slices.ticket;
+        a.state = slices.state;
+        // the ticket and every sliced tile's count of slices start at zero
+        cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(uint32_t) * (size_t)(1 + ntiles - slices.whole), st);
+        if (e != cudaSuccess) return e;
+        ntiles = slices.ctas;  // the grid
+    }
     switch (nm_bucket) {
         case 1: return launch_fused_nm1(nd_bucket, params, maps, a, smem, (int)ntiles, rows, st, max_ctas_per_sm);
         case 2: return launch_fused_nm2(nd_bucket, params, maps, a, smem, (int)ntiles, rows, st, max_ctas_per_sm);

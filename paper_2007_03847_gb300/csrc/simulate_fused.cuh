@@ -64,10 +64,38 @@ struct FusedArgs {
     // carried from the chunk before, and a first contraction over rows up to 0
     // gives f(0)), and the step loop forms the disturbances' RK stage values
     int smooth;
+    // the sliced form (see slice_shape in api.cu): the grid is a fixed number of CTAs per
+    // SM, which take work items in order from a ticket: first `whole` tiles over the
+    // whole horizon, then the other tiles slice by slice, `slice` steps at a time
+    // (a multiple of TC), each tile's state kept in `state` between its slices
+    int64_t ntiles, whole;
+    int slice, nslice;
+    uint32_t* ticket;  // [1] next item, then [ntiles - whole] slices done per tile
+    float* state;      // [ntiles - whole][FU_STATE(NM, ND)][rows]
 };
 
-template <int NM, int ND, bool SMOOTH>
-__global__ void __launch_bounds__(FU_THREADS, 4)
+// Values of a sample's state between two slices of its tile.
+__host__ __device__ constexpr int fu_state(int nm, int nd) { return 2 * nm + 2 + nd; }
+
+// Polls of a slice's wait for the one before it (about 64 ns apart): seconds, since the
+// slice before may be a millisecond's work.
+constexpr uint32_t FU_SLICE_WAIT = 1u << 24;
+
+// One thread waits until *done reaches `want` (release / acquire with the writer's
+// atomicExch after its fence).  The writer holds an earlier ticket, so it is running.
+__device__ __forceinline__ bool slice_wait(const uint32_t* done, uint32_t want)
+{
+    for (uint32_t it = 0; it < FU_SLICE_WAIT; ++it) {
+        uint32_t v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
+        if (v >= want) return true;
+        __nanosleep(64);
+    }
+    return false;
+}
+
+template <int NM, int ND, bool SMOOTH, bool SLICED>
+__global__ void __launch_bounds__(FU_THREADS, SLICED ? 3 : 4)
     simulate_fused_kernel(const __grid_constant__ SwingParams<NM, ND> p, const __grid_constant__ CUtensorMap mAh,
                           const __grid_constant__ CUtensorMap mAl, const __grid_constant__ CUtensorMap mBh,
                           const __grid_constant__ CUtensorMap mBl, FusedArgs a)
@@ -80,15 +108,13 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
     __shared__ uint64_t bars[2 * TC_MAX_STAGES + 1];  // full[ns], freed[ns], done
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
+    __shared__ uint32_t item_s;
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int rows = blockDim.x, warps = rows / 32;  // samples (= threads) and warps of this CTA
     const int n = p.n, d = p.d, S = 2 * n, S3 = 3 * S;
     constexpr int FU_MS = fu_ms(NM);
     constexpr int MSLOT = 6 * NM;  // floats per (step, warp) slot: ref | dev | m2 of up to 2 NM states
-    const int64_t row0 = (int64_t)blockIdx.x * rows;
-    const int64_t srow = row0 + tid;
-    const bool active = srow < a.count;
     const int TC = a.TC;
     const int CW = SMOOTH ? 2 * TC : TC;  // TMEM columns per disturbance and chunk
 
@@ -102,7 +128,6 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
     r.full = &bars[0];
     r.freed = &bars[TC_MAX_STAGES];
     r.a_policy = 0;
-    if (a.keep_tiles > 0) r.a_policy = (int)blockIdx.x < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
     uint64_t* done = &bars[2 * TC_MAX_STAGES];
     const int WROW = 2 * NM + 1;
     float* wbuf = reinterpret_cast<float*>(smem) + warp * 32 * WROW;           // [32][WROW] per warp
@@ -127,6 +152,36 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
     const int J = d * a.nkb;  // K blocks of a chunk
     const uint32_t idesc = umma_idesc_bf16(TC_M, CW);
 
+    uint32_t g = 0;  // K blocks issued so far (thread 0)
+    uint32_t cp = 0;  // contractions so far (parity of their barrier)
+    bool failed = false;  // (sliced) a bounded wait gave up: the CTA takes no more items
+    for (;;) {
+    // ---- the next work item: a tile, steps n_first .. n_last - 1 ----
+    int64_t tile = blockIdx.x;
+    int n_first = 0, n_last = a.Nt;
+    int64_t sl_tile = -1;  // (sliced) the tile's place among the sliced ones
+    uint32_t sl = 0;
+    if constexpr (SLICED) {
+        if (tid == 0) item_s = atomicAdd(a.ticket, 1u);
+        __syncthreads();
+        const int64_t item = item_s;
+        __syncthreads();
+        tile = item;
+        if (item >= a.whole) {
+            const int64_t nsl = a.ntiles - a.whole;
+            sl = nsl > 0 ? (uint32_t)((item - a.whole) / nsl) : (uint32_t)a.nslice;
+            if (sl >= (uint32_t)a.nslice) break;
+            sl_tile = (item - a.whole) % nsl;
+            tile = a.whole + sl_tile;
+            n_first = (int)sl * a.slice;
+            n_last = a.Nt - n_first < a.slice ? a.Nt : n_first + a.slice;
+        }
+    }
+    const int64_t row0 = tile * rows;
+    const int64_t srow = row0 + tid;
+    const bool active = srow < a.count;
+    if (a.keep_tiles > 0) r.a_policy = tile < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
+
     float del[NM], w[NM], theta = 0.f;   // deviations from the equilibrium (see swing_step)
     float x0[ND];
 #pragma unroll
@@ -136,29 +191,52 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
     }
 #pragma unroll
     for (int q = 0; q < ND; ++q) x0[q] = 0.f;
+    float racc = 0.f;  // sum over the grid of the squared centre-of-inertia speed
 
     const int64_t trow = 2 * (int64_t)n;
     float* traj = (a.traj != nullptr && active) ? a.traj + srow * (int64_t)(a.Nt + 1) * trow : nullptr;
-    if (traj) {
+    float* part_tile = nullptr;
+    if constexpr (SLICED) part_tile = a.part ? a.part + tile * (a.Nt + 1) * S3 : nullptr;
+    if (SLICED && n_first > 0) {
+        // the state the tile's last slice left (from L2: this SM may hold older lines)
+        if (tid == 0) abort_flag = slice_wait(a.ticket + 1 + sl_tile, sl) ? 0 : 1;
+        __syncthreads();
+        if (abort_flag) {
+            if (tid == 0) atomicExch(a.err, DEV_TIMEOUT_MMA);
+            break;
+        }
+        const float* st = a.state + sl_tile * (int64_t)fu_state(NM, ND) * rows + tid;
 #pragma unroll
-        for (int i = 0; i < NM; ++i)
-            if (i < n) {
-                traj[i] = p.dst[i];
-                traj[n + i] = 0.f;
-            }
+        for (int i = 0; i < NM; ++i) {
+            del[i] = __ldcg(st + i * rows);
+            w[i] = __ldcg(st + (NM + i) * rows);
+        }
+        theta = __ldcg(st + 2 * NM * rows);
+        racc = __ldcg(st + (2 * NM + 1) * rows);
+#pragma unroll
+        for (int q = 0; q < ND; ++q) x0[q] = __ldcg(st + (2 * NM + 2 + q) * rows);
+    } else {
+        if (traj) {
+#pragma unroll
+            for (int i = 0; i < NM; ++i)
+                if (i < n) {
+                    traj[i] = p.dst[i];
+                    traj[n + i] = 0.f;
+                }
+        }
+        // time 0: every sample sits at the (rounded) shift, so both sums are zero.  (The
+        // pointer is formed here in the unsliced form and before the branch in the sliced
+        // one: the other way round the kernels of 10 machines and 4 disturbances spill 176
+        // and 224 bytes instead of 64 and 12, and 2^20 samples take 427 ms instead of 387.)
+        if constexpr (!SLICED) part_tile = a.part ? a.part + tile * (a.Nt + 1) * S3 : nullptr;
+        if (part_tile)
+            for (int v = tid; v < S3; v += rows) part_tile[v] = 0.f;
     }
-    // time 0: every sample sits at the (rounded) shift, so both sums are zero
-    float* part_tile = a.part ? a.part + (int64_t)blockIdx.x * (a.Nt + 1) * S3 : nullptr;
-    if (part_tile)
-        for (int v = tid; v < S3; v += rows) part_tile[v] = 0.f;
-
-    uint32_t g = 0;  // K blocks issued so far (thread 0)
-    float racc = 0.f;  // sum over the grid of the squared centre-of-inertia speed
 
     float f0[ND];  // the smooth form's forcing at the chunk's first grid time
 #pragma unroll
     for (int q = 0; q < ND; ++q) f0[q] = 0.f;
-    for (int c = 0, n0 = SMOOTH ? -TC : 0; n0 < a.Nt; ++c, n0 += TC) {
+    for (int n0 = SMOOTH ? -TC : n_first; n0 < (SLICED ? n_last : a.Nt); n0 += TC) {
         // ---- tensor cores: dW of this chunk into TMEM ----
         if (!em) {
         tc_fence_before();
@@ -195,11 +273,15 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
         }
         __syncthreads();
         bool ok = (abort_flag == 0);
-        if (ok && !mbar_wait(done, (uint32_t)c & 1u)) {
+        if (ok && !mbar_wait(done, cp & 1u)) {
             ok = false;
             atomicExch(a.err, DEV_TIMEOUT_MMA);
         }
-        if (!__syncthreads_and(ok)) break;
+        ++cp;
+        if (!__syncthreads_and(ok)) {
+            failed = true;
+            break;
+        }
         tc_fence_after();
         }
 
@@ -213,7 +295,7 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
                 continue;
             }
         }
-        const int steps = (a.Nt - n0) < TC ? (a.Nt - n0) : TC;
+        const int steps = SLICED ? ((n_last - n0) < TC ? (n_last - n0) : TC) : ((a.Nt - n0) < TC ? (a.Nt - n0) : TC);
         // ---- disturbance paths of this chunk into TMEM (each warp its own lanes) ----
         if constexpr (!SMOOTH)
             disturbance_chunk<ND, ND, true>(lane_addr, TC, steps, n0, d, -1, x0, p.ou_a, p.ou_s, p.ito, p.dt, a.em,
@@ -331,8 +413,25 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
             }
         }
     }
+    if (SLICED && n_last < a.Nt && !failed) {
+        // the tile goes on in a later item, on whichever CTA takes it
+        float* st = a.state + sl_tile * (int64_t)fu_state(NM, ND) * rows + tid;
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+            st[i * rows] = del[i];
+            st[(NM + i) * rows] = w[i];
+        }
+        st[2 * NM * rows] = theta;
+        st[(2 * NM + 1) * rows] = racc;
+#pragma unroll
+        for (int q = 0; q < ND; ++q) st[(2 * NM + 2 + q) * rows] = x0[q];
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) atomicExch(a.ticket + 1 + sl_tile, sl + 1u);
+        continue;
+    }
     if (a.rrf) rrf_accumulate(active ? sqrtf(racc / (float)a.Nt) : 0.f, a.rrf);
-    if (!em && (int)blockIdx.x < a.keep_tiles) {
+    if (!em && tile < a.keep_tiles) {
         // the tile's design rows back to normal L2 priority
         const int64_t left = a.count - row0;
         const int64_t bytes = (left < rows ? left : rows) * a.zeta_row_bytes;
@@ -340,6 +439,8 @@ __global__ void __launch_bounds__(FU_THREADS, 4)
             l2_priority_normal(a.zeta_hi + row0 * a.zeta_row_bytes + o);
             if (a.split) l2_priority_normal(a.zeta_lo + row0 * a.zeta_row_bytes + o);
         }
+    }
+    if (!SLICED || failed) break;
     }
     tc_fence_before();
     __syncthreads();
@@ -351,7 +452,10 @@ cudaError_t launch_fused_t(const void* params, const CUtensorMap* maps, const Fu
                            int rows, cudaStream_t st, int* max_ctas_per_sm)
 {
     const SwingParams<NM, ND>& p = *static_cast<const SwingParams<NM, ND>*>(params);
-    auto kern = a.smooth ? simulate_fused_kernel<NM, ND, true> : simulate_fused_kernel<NM, ND, false>;
+    const bool sliced = a.ticket != nullptr;
+    if (sliced && a.smooth) return cudaErrorInvalidValue;
+    auto kern = a.smooth ? simulate_fused_kernel<NM, ND, true, false>
+                : sliced ? simulate_fused_kernel<NM, ND, false, true> : simulate_fused_kernel<NM, ND, false, false>;
     // the attribute is process-wide and launches from several host threads may
     // race on it: always the same (largest) bound, the launch passes its own size
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_DYN_MAX);
