@@ -1252,12 +1252,13 @@ static size_t team_part_bytes(int n, int Nt, int64_t count)
 
 // Whether a fused launch that would take the per-sample kernel takes the team kernel
 // (the same results; simulate_team.cuh): while its groups of 32 samples get an SM each
-// (count <= 32 SMs).  Measured (GB300, 10 machines, 3 disturbances, 1000 steps, the
-// whole call, per-sample -> team): 1000 samples 3.44 -> 2.14 ms, 4864 3.72 -> 2.20,
-// 9728 3.68 -> 4.17; 4000 samples of 1 machine 0.99 -> 0.75, 4 machines 1.36 -> 1.20,
-// 8 machines 2.10 -> 1.68, 12 machines 3.47 -> 2.03.  The same line where other launches
-// share the GPU (four arms of 10007 samples at once: 10.6 ms, by teams 19.5).  Its
-// partials are four times the per-sample kernel's: not past 512 MiB, and not in a
+// (count <= 32 SMs).  Measured (GB300, 1000 steps, the whole call, per-sample -> team):
+// 10 machines, 3 disturbances: 1000 samples 3.44 -> 1.96 ms; 4000 samples, 2 disturbances:
+// 1 machine 0.99 -> 0.75, 4 machines 1.36 -> 1.10, 8 machines 2.10 -> 1.48, 12 machines
+// 4.1 -> 1.8, 13 machines (slots of 16) 8.5 -> 3.6, 16 machines 7.4 -> 2.9.  Above the
+// line it loses (10 machines, 9728 samples: 3.68 -> 4.17).  The same line where other
+// launches share the GPU (four arms of 10007 samples at once: 10.6 ms, by teams 19.5).
+// Its partials are four times the per-sample kernel's: not past 512 MiB, and not in a
 // context with a memory budget.
 static constexpr size_t TEAM_PART_MAX = (size_t)512 << 20;
 

@@ -94,9 +94,9 @@ cudaError_t launch_simulate_fused(int nm_bucket, int nd_bucket, const void* para
                                   int rows, int max_ctas, const double* eq, float* part, double* S1, double* S2,
                                   float* traj, int* err, const EmSpec& em, double* rrf, const L2Keep& keep,
                                   int smooth, const SlicePlan& slices, cudaStream_t st, int* max_ctas_per_sm);
-// Few samples of up to 12 machines: the team kernel (simulate_team.cuh), 32 samples
+// Few samples of up to 16 machines: the team kernel (simulate_team.cuh), 32 samples
 // per CTA; part [groups of 32][Nt+1][3][2n]; maps as above with design boxes of 32 rows
-constexpr int TEAM_GROUP = 32, TEAM_MAX_NM = 12;
+constexpr int TEAM_GROUP = 32, TEAM_MAX_NM = 16;
 cudaError_t launch_simulate_team(int nm_bucket, int nd_bucket, const void* params, const CUtensorMap* maps,
                                  int64_t count, int Nt, int TC, int d, int Ks, int nkb, int split, uint32_t tmem_cols,
                                  float* part, float* traj, int* err, const EmSpec& em, double* rrf, int smooth,

@@ -37,6 +37,7 @@ cudaError_t launch_team_nm4(int, const void*, const CUtensorMap*, const TeamArgs
 cudaError_t launch_team_nm8(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
 cudaError_t launch_team_nm10(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
 cudaError_t launch_team_nm12(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
+cudaError_t launch_team_nm16(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
 
 int wide_nmt_for(int n)
 {
@@ -158,6 +159,7 @@ cudaError_t launch_simulate_team(int nm_bucket, int nd_bucket, const void* param
         case 8: return launch_team_nm8(nd_bucket, params, maps, a, smooth, st);
         case 10: return launch_team_nm10(nd_bucket, params, maps, a, smooth, st);
         case 12: return launch_team_nm12(nd_bucket, params, maps, a, smooth, st);
+        case 16: return launch_team_nm16(nd_bucket, params, maps, a, smooth, st);
         default: return cudaErrorInvalidValue;
     }
 }

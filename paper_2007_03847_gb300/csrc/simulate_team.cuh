@@ -1,4 +1,4 @@
-// Algorithm 1 steps 2-4 fused for few samples (up to 12 machines): one CTA per 32
+// Algorithm 1 steps 2-4 fused for few samples (up to 16 machines): one CTA per 32
 // samples, the machines of a sample spread over a team of L warps.
 //
 // What bounds a small study is the latency of one sample's step: with one thread per
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(team_threads(NM), NM > 8 ? 1 : 2)
         }
         const float dt = p.dt;
         const bool rk4 = (p.integrator == FMC_RK4);
-        const int nst = rk4 ? 4 : 2;
+        const float dth = 0.5f * dt, dtw = dt * p.omega_s, dthw = dth * p.omega_s;
         const float ref = p.rel ? 1.f : 0.f;
         const float hh = rk4 ? dt * (1.0f / 6.0f) : 0.5f * dt;
         const float hhw = hh * p.omega_s;
@@ -427,68 +427,66 @@ __global__ void __launch_bounds__(team_threads(NM), NM > 8 ? 1 : 2)
                         }
                     }
                 }
-                float ad = 0.f, aw = 0.f, yd = del, yw = w, ath = 0.f;
-#pragma unroll 1
-                for (int st = 0; st < nst; ++st) {
-                    float b, cn, xw;
-                    if (rk4) {
-                        b = (st == 1 || st == 2) ? 2.f : 1.f;
-                        cn = (st == 2) ? dt : 0.5f * dt;
-                        xw = (st == 0) ? 0.f : ((st == 3) ? 1.f : 0.5f);
+                // the forcing at the stage times (the two middle stages share theirs)
+                float f0 = 0.f, fm = 0.f, fm2 = 0.f, f1 = 0.f;
+#pragma unroll
+                for (int q = 0; q < ND; ++q) {
+                    if constexpr (SMOOTH) {
+                        f0 = fmaf(inj[q], xst[0][q], f0);
+                        fm = fmaf(inj[q], xst[1][q], fm);
+                        fm2 = fmaf(inj[q], xst[2][q], fm2);
+                        f1 = fmaf(inj[q], xst[3][q], f1);
                     } else {
-                        b = 1.f;
-                        cn = dt;
-                        xw = (st == 0) ? 0.f : 1.f;
+                        const float dx = x1[q] - x0[q];
+                        f0 = fmaf(inj[q], fmaf(0.f, dx, x0[q]), f0);
+                        fm = fmaf(inj[q], fmaf(0.5f, dx, x0[q]), fm);
+                        f1 = fmaf(inj[q], fmaf(1.f, dx, x0[q]), f1);
                     }
+                }
+                if (!SMOOTH) fm2 = fm;
+                float ad = 0.f, aw = 0.f, yd = del, yw = w, ath = 0.f;
+                auto stage = [&](float b, float cn, float cnw, float f) {
                     // publish the stage input's sines (at the last stage's tier) and machine
                     // 0's speed
                     float2* cs = reinterpret_cast<float2*>(exch + gb * EXCH);
                     float* w0s = reinterpret_cast<float*>(exch + gb * EXCH + NM * 256);
                     uint8_t* tiers = exch + gb * EXCH + NM * 256 + 128;
-                    const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(0.f, fabsf(yd))));
-                    int mine = mx <= __float_as_uint(0.8f) ? 2 : 3;
-                    if (SHORT) mine = mx <= __float_as_uint(0.05f) ? 0 : (mx <= __float_as_uint(0.25f) ? 1 : mine);
-                    float2 my = team_trig(tier, yd);
-                    float w0 = yw;
-                    int now = mine;
+                    gb ^= 1;
+                    float2 my;
+                    if (tier == TIER0)
+                        deviation_trig1<TIER0>(yd, &my.y, &my.x);
+                    else
+                        my = team_trig(tier, yd);
+                    float w0 = yw * ref;
                     if constexpr (NM > 1) {
                         cs[i * 32 + lane] = my;
-                        if (i == 0) w0s[lane] = yw;
-                        bool ask = true;
-                        if (tier == TIER0) ask = !team_all<NM>(mine == TIER0);
-                        if (ask) {
-                            // some warp is past the shortest series (or the last stage was)
-                            if (lane == 0) tiers[i] = (uint8_t)mine;
-                            team_bar<NM>();
-                            now = 0;
-#pragma unroll
-                            for (int j = 0; j < NM; ++j) now = max(now, (int)tiers[j]);
-                        } else {
-                            now = TIER0;
-                        }
-                        w0 = w0s[lane];
+                        if (i == 0) w0s[lane] = w0;
                     }
-                    if (now != tier) {
-                        // (uniform over the team) another tier: the sines again
-                        tier = now;
-                        my = team_trig(tier, yd);
+                    const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(0.f, fabsf(yd))));
+                    bool ask = tier != TIER0;
+                    if (!ask) ask = !team_all<NM>(mx <= __float_as_uint(SHORT ? 0.05f : 0.8f));
+                    if (ask) {
+                        // some warp is past the shortest series (or the last stage was)
+                        int now = mx <= __float_as_uint(0.8f) ? 2 : 3;
+                        if (SHORT) now = mx <= __float_as_uint(0.05f) ? 0 : (mx <= __float_as_uint(0.25f) ? 1 : now);
                         if constexpr (NM > 1) {
-                            cs[i * 32 + lane] = my;
+                            if (lane == 0) tiers[i] = (uint8_t)now;
                             team_bar<NM>();
+#pragma unroll 1
+                            for (int j = 0; j < NM; ++j) now = max(now, (int)tiers[j]);
+                        }
+                        if (now != tier) {
+                            // (uniform over the team) another tier: the sines again
+                            tier = now;
+                            my = team_trig(tier, yd);
+                            if constexpr (NM > 1) {
+                                cs[i * 32 + lane] = my;
+                                team_bar<NM>();
+                            }
                         }
                     }
-                    w0 *= ref;
+                    if constexpr (NM > 1) w0 = w0s[lane];
                     ath = fmaf(b, w0, ath);
-                    float f = 0.f;
-#pragma unroll
-                    for (int q = 0; q < ND; ++q) {
-                        float xs;
-                        if constexpr (SMOOTH)
-                            xs = st == 0 ? xst[0][q] : (st == 1 ? xst[1][q] : (st == 2 ? xst[2][q] : xst[3][q]));
-                        else
-                            xs = fmaf(xw, x1[q] - x0[q], x0[q]);
-                        f = fmaf(inj[q], xs, f);
-                    }
                     // network sums (row_network)
                     unsigned long long au = 0ull, av = 0ull;
                     if constexpr (NM > 1) {
@@ -511,9 +509,17 @@ __global__ void __launch_bounds__(team_threads(NM), NM > 8 ? 1 : 2)
                     const float kv = yw - w0;
                     ad = fmaf(b, kv, ad);
                     aw = fmaf(b, kw, aw);
-                    yd = fmaf(cn * p.omega_s, kv, del);
+                    yd = fmaf(cnw, kv, del);
                     yw = fmaf(cn, kw, w);
-                    gb ^= 1;
+                };
+                if (rk4) {
+                    stage(1.f, dth, dthw, f0);
+                    stage(2.f, dth, dthw, fm);
+                    stage(2.f, dt, dtw, fm2);
+                    stage(1.f, dth, dthw, f1);
+                } else {
+                    stage(1.f, dt, dtw, f0);
+                    stage(1.f, dt, dtw, SMOOTH ? fm : f1);
                 }
                 del = fmaf(hhw, ad, del);
                 w = fmaf(hh, aw, w);

@@ -74,3 +74,15 @@ def test_team_response_function_and_blocks(fmc):
     assert np.allclose(r.cpu().numpy(), r1.cpu().numpy(), rtol=1e-9)
     s, s1 = _both(fmc, lambda: fmc.simulate_sums(sc, 100, 130))
     assert all(torch.equal(a, b) for a, b in zip(s, s1))
+
+
+@pytest.mark.parametrize("n,d,N,T", [(13, 3, 70, 0.2), (14, 1, 33, 0.165), (16, 8, 300, 0.1)])
+@pytest.mark.parametrize("precision", ["bf16x3", "bf16"])
+def test_team_of_sixteen_equals_per_sample(fmc, n, d, N, T, precision):
+    # without launch rules (a measured one may take the split kernel for these systems)
+    from paper_2007_03847_gb300 import autotune
+    fmc.set_launch_rules([])
+    try:
+        _equal(fmc, fs.multimachine_case(n=n, d=d, K=37, T=T, dt=0.005, N=N, seed=n * 100 + d), precision=precision)
+    finally:
+        autotune.apply_cached(fmc.default_context())
