@@ -1145,6 +1145,7 @@ struct Prepared {
     bool bus = false;  // ... for a system with an infinite bus (its own instantiations)
     bool exclusive = true;  // the launch has the GPU to itself (see fused_shape)
     bool team = false;      // few samples: the team kernel (see team_wanted)
+    int share = 0;          // CTAs of a sliced launch among others of its batch (batch_shares)
     int64_t k0 = 0, count = 0;
     std::vector<unsigned char> params;
 };
@@ -1384,12 +1385,12 @@ struct FusedShape {
 // last round of 4 SMs tiles is more than a sixteenth empty (in the steady state four
 // CTAs per SM are 2 % faster: 2^20 samples 387 ms, sliced 394 with three and 397 with
 // four); with more than 2 SMs tiles, two CTAs per SM while that is the shorter (t / 2
-// rounds of 4.2 against one of 5.8).  Exclusive launches only (others fill the idle SMs of
-// a shared one), not the smooth form, and not in a context with a memory budget.  Measured
-// (GB300, 10 machines, 4000 steps): 65536 samples 31.2 -> 24.9 ms; 1000 steps of 45000
-// samples 5.9 -> 4.6 ms.
+// rounds of 4.2 against one of 5.8).  A launch that shares the GPU is sliced over the
+// CTAs that its batch gives it (batch_shares).  Not the smooth form, and not in a context
+// with a memory budget.  Measured (GB300, 10 machines, 4000 steps): 65536 samples
+// 31.2 -> 24.9 ms; 1000 steps of 45000 samples 5.9 -> 4.6 ms.
 struct SliceShape {
-    int per_sm;
+    int ctas;  // grid (0: not sliced)
     int64_t whole, tiles;
     int steps;
 };
@@ -1397,28 +1398,25 @@ struct SliceShape {
 static SliceShape slice_shape(const fmc_ctx* ctx, const Prepared& P, int TC)
 {
     SliceShape s{0, 0, (P.count + TC_M - 1) / TC_M, 0};
-    if (!P.exclusive || P.nmt > 0 || P.team || P.s.forcing == FMC_FORCING_SMOOTH || ctx->budget != 0) return s;
+    if (P.nmt > 0 || P.team || P.s.forcing == FMC_FORCING_SMOOTH || ctx->budget != 0) return s;
     const int64_t sms = ctx->sms, t = s.tiles;
-    int per = 0;
-    const int64_t rounds = (t + 4 * sms - 1) / (4 * sms);  // of the unsliced launch
-    if (t > 3 * sms && 16 * t < 15 * rounds * 4 * sms)
-        per = 3;
-    else if (t <= 3 * sms && t > 2 * sms && 5 * t < 14 * sms)
-        per = 2;
-    if (per == 0 || t % (per * sms) == 0) return s;
-    s.per_sm = per;
-    const int64_t slots = per * sms;
-    s.whole = (t / slots - 1) * slots;  // (>= 0: t > slots)
+    int64_t slots = 0;
+    if (!P.exclusive) {
+        slots = P.share;
+    } else {
+        const int64_t rounds = (t + 4 * sms - 1) / (4 * sms);  // of the unsliced launch
+        if (t > 3 * sms && 16 * t < 15 * rounds * 4 * sms)
+            slots = 3 * sms;
+        else if (t <= 3 * sms && t > 2 * sms && 5 * t < 14 * sms)
+            slots = 2 * sms;
+    }
+    if (slots <= 0 || t <= slots || t % slots == 0) return s;
+    s.ctas = (int)slots;
+    s.whole = (t / slots - 1) * slots;
     int steps = (P.Nt + 47) / 48;
     steps = (steps + TC - 1) / TC * TC;
     s.steps = steps;
     return s;
-}
-
-static int slice_ctas(const fmc_ctx* ctx, const Prepared& P)
-{
-    // (TC does not enter the choice)
-    return slice_shape(ctx, P, 16).per_sm;
 }
 
 static FusedShape fused_shape(const fmc_ctx* ctx, const Prepared& P)
@@ -1437,14 +1435,26 @@ static FusedShape fused_shape(const fmc_ctx* ctx, const Prepared& P)
         f.ctas = (P.count + f.rows - 1) / f.rows;
         return f;
     }
+    const fmc_launch_rule* rule = find_rule(ctx, &P.s, P.count);
     if (P.exclusive) {
         const int64_t need = (full + sms - 1) / sms;
         f.max_ctas = wide ? 1 : (need >= 3 ? 4 : (int)(need < 1 ? 1 : need));
+        // (a rule for one CTA per SM was measured on fewer tiles than SMs: past them it
+        // runs the tiles left over in a second round; 1000 steps of 10 machines, 19500
+        // to 32767 samples: 8.0 -> 4.7 ms)
+        if (rule && rule->max_ctas > 0 && !wide) f.max_ctas = rule->max_ctas == 1 && need > 1 ? 2 : rule->max_ctas;
+    } else if (full <= 2 * sms) {
+        // among other launches: room for two CTAs per SM, whatever a rule measured alone
+        // says.  With one, the launches run one after another once their tiles pass the
+        // SMs; with four, several launches' CTAs pile up on the same SMs.  Two, three and
+        // four launches of 79 tiles (9 machines, 1000 steps), by CTAs per SM 1, 2, 3, 4:
+        // 6.9, 5.1, 5.5, 6.1; 7.1, 5.6, 7.6, 9.2; 10.4, 8.4, 7.6, 10.0 ms
+        f.max_ctas = 2;
+    } else if (rule && rule->max_ctas > 0 && !wide) {
+        f.max_ctas = rule->max_ctas;
     }
-    const fmc_launch_rule* rule = find_rule(ctx, &P.s, P.count);
-    if (rule && rule->max_ctas > 0 && !wide) f.max_ctas = rule->max_ctas;
-    const int sliced = slice_ctas(ctx, P);
-    if (sliced > 0) f.max_ctas = sliced;
+    const int sliced = slice_shape(ctx, P, 16).ctas;  // (TC does not enter the choice)
+    if (sliced > 0) f.max_ctas = sliced > 2 * sms ? 3 : 2;
     // a CTA's TMEM columns: the largest power of two within its share of the SM's
     // 512 (allocations are powers of two)
     int cols = 512;
@@ -1509,7 +1519,7 @@ static int reserve(fmc_ctx* ctx, Workspace& ws, const Prepared& P, bool want_tra
     {
         const FusedShape f = fused_shape(ctx, P);
         const SliceShape sl = slice_shape(ctx, P, f.TC);
-        if (sl.per_sm > 0 && (rc = ensure(ctx, ws.slices, slice_bytes(P, sl)))) return rc;
+        if (sl.ctas > 0 && (rc = ensure(ctx, ws.slices, slice_bytes(P, sl)))) return rc;
     }
     if (!em) {
         if ((rc = ensure(ctx, ws.zeta_hi, zbytes))) return rc;
@@ -1710,8 +1720,8 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
         }
         SlicePlan slices{};
         const SliceShape sl = slice_shape(ctx, P, TC);
-        if (sl.per_sm > 0) {
-            slices.ctas = sl.per_sm * ctx->sms;
+        if (sl.ctas > 0) {
+            slices.ctas = sl.ctas;
             slices.whole = sl.whole;
             slices.steps = sl.steps;
             slices.ticket = (uint32_t*)ws.slices.ptr;
@@ -1990,6 +2000,38 @@ static void batch_free(fmc_batch* b)
     delete b;
 }
 
+// The grids of a batch's per-sample launches, which run side by side two CTAs to an SM.
+// Together past that many tiles, the tiles left over would run a round of their own on a
+// nearly idle GPU, so every launch that can be sliced (slice_shape) gets a share of the
+// CTAs by its work: all are resident from the start and end together.  The work is
+// tiles x steps x n (n + 24), which fits 65536 samples of 4, 8, 12 and 16 machines to
+// 20 % (2.7, 5.1, 8.7 and 13.4 ms per 1000 steps).  Only where every scenario has a stream
+// of its own.  Measured (GB300, one CTA per SM and no shares -> two and shares): four arms
+// of 10007 samples, 9 machines, one of them smooth, 11.2 -> 7.3 ms; four of 20000 samples
+// of 10 machines 20.3 -> 9.6, of 40000 22.0 -> 19.4; twelve of 6000 16.5 -> 8.8.
+static void batch_shares(const fmc_ctx* ctx, std::vector<Prepared>& prep)
+{
+    int64_t slots = 2 * (int64_t)ctx->sms, all = 0;
+    double work = 0;
+    auto tiles = [](const Prepared& P) { return (P.count + TC_M - 1) / TC_M; };
+    auto cost = [&](const Prepared& P) { return (double)tiles(P) * P.Nt * P.nm * (P.nm + 24.0); };
+    auto sliced = [](const Prepared& P) { return P.s.forcing != FMC_FORCING_SMOOTH; };
+    for (const Prepared& P : prep) {
+        if (P.path != FMC_PATH_FUSED || P.nmt > 0 || P.team) continue;
+        all += tiles(P);
+        if (sliced(P))
+            work += cost(P);
+        else
+            slots -= tiles(P);
+    }
+    if (all <= 2 * (int64_t)ctx->sms || slots <= 0 || ctx->budget != 0) return;
+    for (Prepared& P : prep) {
+        if (P.path != FMC_PATH_FUSED || P.nmt > 0 || P.team || !sliced(P)) continue;
+        const int64_t share = (int64_t)((double)slots * (cost(P) / work));
+        P.share = (int)(share < 1 ? 1 : share);
+    }
+}
+
 // Enqueue every scenario: fork from `st` onto the batch's streams, one scenario
 // per stream in turn (so that independent scenarios share the GPU), join back.
 static int batch_enqueue(fmc_batch* b, cudaStream_t st)
@@ -2040,11 +2082,13 @@ int fmc_batch_create(fmc_ctx* ctx, const fmc_scenario* scen, int32_t n_scen, int
         b->owned.push_back(std::make_unique<fmc::OwnedScenario>(scen[i]));
         const fmc_scenario* si = &b->owned.back()->s;
         rc = prepare(ctx, *w, si, 0, si->N, path, st0, b->prep.back(), false);  // scenarios share the GPU
-        if (rc == FMC_OK) rc = reserve(ctx, *w, b->prep.back(), false, path == FMC_PATH_PLAIN);
         b->mean.push_back(mean_dev[i]);
         b->var.push_back(var_dev[i]);
     }
     const int nstreams = n_scen < 16 ? n_scen : 16;
+    if (rc == FMC_OK && nstreams == n_scen) batch_shares(ctx, b->prep);
+    for (int i = 0; i < n_scen && rc == FMC_OK; ++i)
+        rc = reserve(ctx, *b->ws[i], b->prep[i], false, path == FMC_PATH_PLAIN);
     for (int k = 0; k < nstreams && rc == FMC_OK; ++k) {
         cudaStream_t s;
         cudaEvent_t e;
