@@ -130,20 +130,25 @@ __device__ __forceinline__ void net_mma(uint32_t d_tmem, uint32_t ahi_tmem, uint
     constexpr uint32_t KB_BYTES = NN * 64;  // one K block: NN rows of 64 bytes
     constexpr uint32_t LO = (NN / 16) * KB_BYTES;
     constexpr uint32_t idesc = umma_idesc_tf32(TC_M, NN);
+    // one descriptor, stepped by its 16-byte address field (shared addresses end below
+    // its 14 bits): the issuing thread's instructions are on every warp's path to the sums
+    // (65536 samples of 20 machines, 1000 steps: 23.5 -> 23.1 ms)
+    const uint64_t d0 = umma_desc_sw64(net);
+    auto desc = [&](uint32_t off) { return d0 + (uint64_t)(off >> 4); };
 #pragma unroll
     for (int ks = 0; ks < NN / 8; ++ks) {
         const uint32_t off = (uint32_t)(ks >> 1) * KB_BYTES + (uint32_t)(ks & 1) * 32u;
-        umma_tf32_ts(d_tmem, alo_tmem + 8u * ks, umma_desc_sw64(net + off), idesc, ks > 0 ? 1u : 0u);
+        umma_tf32_ts(d_tmem, alo_tmem + 8u * ks, desc(off), idesc, ks > 0 ? 1u : 0u);
     }
 #pragma unroll
     for (int ks = 0; ks < NN / 8; ++ks) {
         const uint32_t off = (uint32_t)(ks >> 1) * KB_BYTES + (uint32_t)(ks & 1) * 32u;
-        umma_tf32_ts(d_tmem, ahi_tmem + 8u * ks, umma_desc_sw64(net + LO + off), idesc, 1u);
+        umma_tf32_ts(d_tmem, ahi_tmem + 8u * ks, desc(LO + off), idesc, 1u);
     }
 #pragma unroll
     for (int ks = 0; ks < NN / 8; ++ks) {
         const uint32_t off = (uint32_t)(ks >> 1) * KB_BYTES + (uint32_t)(ks & 1) * 32u;
-        umma_tf32_ts(d_tmem, ahi_tmem + 8u * ks, umma_desc_sw64(net + off), idesc, 1u);
+        umma_tf32_ts(d_tmem, ahi_tmem + 8u * ks, desc(off), idesc, 1u);
     }
 }
 
