@@ -28,8 +28,8 @@ namespace fmc {
 // by additions modulo the period along a thread's times.  Without room for the table
 // (the allocation-free reconstruction) a thread evaluates the cosine itself.  The
 // operations per entry are the same either way, in the same order.
-// Measured (GB300), split form: K = 200, Nt = 4000 148 -> 11 us; K = 100, Nt = 1000
-// 32 -> 8 us.
+// Measured (GB300), split form: K = 200, Nt = 4000 148 -> 28 us; K = 100, Nt = 1000
+// 32 -> 17 us, the table's 4 us included.
 struct BasisArgs {
     int K, Nt, basis;
     double T;

@@ -4,7 +4,14 @@
 // accumulation in TMEM.  One CTA per [128 samples x TN steps] block of one
 // disturbance; thread 0 streams the K blocks with TMA and issues the MMAs, then
 // each of the four warps reads its 32 TMEM lanes (= its 32 samples) and writes
-// the rows to HBM.  This standalone form serves fmc_kle_reconstruct; the fused
+// the rows to HBM: through bulk copies of rows staged in shared memory where every row
+// starts on 16 bytes, else by transposes of 32 x 32 and plain stores.  What bounds it: the
+// stores' path while they were instructions (plain stores 379 us by lane, 121 us
+// transposed, 94 us as bulk copies for 8192 x 3 rows of 2000 steps, K = 200, split), then
+// the operands' way through L2 (0.7 GB; the products are 59 GFLOP, 31 us at the tensor
+// cores' rate).  Keeping the design tile resident, with four storing warps per SM, was
+// slower (the whole call 225 instead of 218 us).
+// This standalone form serves fmc_kle_reconstruct; the fused
 // simulation consumes the same TMEM tiles without writing them out.
 #include <cuda_bf16.h>
 
@@ -18,11 +25,27 @@ struct ContractArgs {
     int64_t count;
     int d, Ks, nkb, Nt, TN;
     int split, ns;
+    int bulk;  // rows of dW start on 16 bytes: stored by bulk copies
     float* dW;
     int* err;
 };
 
-constexpr int CT_LD = 33;  // floats per row of a warp's 32 x 32 transpose
+constexpr int CT_LD = 33;   // floats per row of a warp's 32 x 32 transpose
+constexpr int CT_LDB = 132;  // and of the block staged for the bulk copies (128 + 16 bytes: no bank conflicts)
+
+// Asynchronous copy of bytes (a multiple of 16) of shared memory to dst, both 16-byte
+// aligned, given up first by L2; the caller's next wait is bulk_read_wait.
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes, uint64_t policy)
+{
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(
+                     __cvta_generic_to_global(dst)),
+                 "r"(smem_u32(src)), "r"(bytes), "l"(policy)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// Until the thread's bulk stores have read their shared memory.
+__device__ __forceinline__ void bulk_read_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
 __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant__ CUtensorMap mAh,
                                                           const __grid_constant__ CUtensorMap mAl,
@@ -106,6 +129,28 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
         const int rows = left <= 0 ? 0 : (left >= 32 ? 32 : (int)left);
         float* out = a.dW + ((row0 + warp * 32) * a.d + w) * (int64_t)a.Nt + n0;
         const int64_t rs = (int64_t)a.d * a.Nt;
+        if (a.bulk) {
+            // a lane stages its sample's row in the ring's place (every product has read its
+            // operands) and hands it to one bulk copy: no store instructions, and the copies
+            // run beside the other CTAs' work
+            float* row = reinterpret_cast<float*>(smem) + (warp * 32 + lane) * CT_LDB;
+            const int cols = a.Nt - n0 < a.TN ? a.Nt - n0 : a.TN;
+            for (int c = 0; c < cols; c += 32) {
+                float v[32];
+#pragma unroll
+                for (int e = 0; e < 32; e += 8)
+                    tmem_ld8(lane_addr + c + e, reinterpret_cast<float(&)[8]>(v[e]));
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 32; e += 4)
+                    *reinterpret_cast<float4*>(row + c + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (lane < rows) {
+                bulk_store(out + lane * rs, row, (uint32_t)cols * 4u, l2_policy_evict_first());
+                bulk_read_wait();
+            }
+        } else
         // a lane holds a sample's row: 32 steps at a time are turned in shared memory, so
         // that a warp stores 128 consecutive bytes of one row
         for (int c = 0; c < a.TN && n0 + c < a.Nt; c += 32) {
@@ -166,10 +211,11 @@ cudaError_t launch_contract_tc(const CUtensorMap* maps, int64_t count, int d, in
     // BF16): one CTA's stores run beside the others' loads and MMAs
     const int stage_bytes = (TC_M * 64 + TN * 64) * (split ? 2 : 1);
     const int ns = split ? 2 : 3;
-    ContractArgs a{count, d, Ks, nkb, Nt, TN, split, ns, dW, err};
+    const int bulk = Nt % 4 == 0 && reinterpret_cast<uintptr_t>(dW) % 16 == 0;
+    ContractArgs a{count, d, Ks, nkb, Nt, TN, split, ns, bulk, dW, err};
     // at least 47 KB so that no more than four CTAs (4 x 128 TMEM columns) share an SM
     int smem = ns * stage_bytes + 1024;
-    const int trans = 4 * 32 * CT_LD * 4 + 1024;
+    const int trans = (bulk ? TC_M * CT_LDB : 4 * 32 * CT_LD) * 4 + 1024;
     if (smem < trans) smem = trans;
     if (smem < 233472 / 5 - 1024 + 64) smem = 233472 / 5 - 1024 + 64;
     static bool attr_done = false;
