@@ -128,9 +128,11 @@ __global__ void __launch_bounds__(FU_THREADS, SLICED ? 3 : 4)
     r.full = &bars[0];
     r.freed = &bars[TC_MAX_STAGES];
     r.a_policy = 0;
-    // (set per tile in the sliced form; there, the smooth kernel of 10 machines and 2
-    // disturbances spilt 196 bytes instead of 8: 4.19 -> 4.55 ms for 10007 samples)
-    if (!SLICED && a.keep_tiles > 0)
+    // (the smooth form sets it here, the others at the tile: the other way round the smooth
+    // kernel of 10 machines and 2 disturbances spills 196 bytes instead of 8, 4.55 instead
+    // of 4.19 ms for 10007 samples, and the others of 10 machines and 4 disturbances 88
+    // instead of 64, 395 instead of 392 ms for 2^20)
+    if (SMOOTH && a.keep_tiles > 0)
         r.a_policy = (int)blockIdx.x < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
     uint64_t* done = &bars[2 * TC_MAX_STAGES];
     const int WROW = 2 * NM + 1;
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(FU_THREADS, SLICED ? 3 : 4)
     const int64_t row0 = tile * rows;
     const int64_t srow = row0 + tid;
     const bool active = srow < a.count;
-    if (SLICED && a.keep_tiles > 0) r.a_policy = tile < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
+    if (!SMOOTH && a.keep_tiles > 0) r.a_policy = tile < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
 
     float del[NM], w[NM], theta = 0.f;   // deviations from the equilibrium (see swing_step)
     float x0[ND];
