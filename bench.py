@@ -574,7 +574,8 @@ def main():
     total_ms = sum(step_ms)
     phase = fmc.PH_FUSED if path == "fused" else fmc.PH_INTEGRATE
     k_ms, k_launches = fmc.profile_read(phase, ctx=ctx)
-    launches_total = sum(fmc.profile_read(p, ctx=ctx)[1] for p in range(8))
+    # one kernel per phase record; the basis is two (its cosine table and the rows)
+    launches_total = sum(fmc.profile_read(p, ctx=ctx)[1] for p in range(8)) + fmc.profile_read(fmc.PH_BASIS, ctx=ctx)[1]
     fmc.profile(False, ctx=ctx)
     fmc.device_status(ctx)
     t_max = torch.tensor([total_ms], dtype=torch.float64, device="cuda")
