@@ -1020,7 +1020,7 @@ int fmc_kle_reconstruct(fmc_ctx* ctx, const float* zeta_dev, int64_t count, int3
     const int Ks = round_up(K, 8);
     const int Kpad = round_up(K, TC_BK);
     const int nkb = (Ks + TC_BK - 1) / TC_BK;
-    const int TN = 128;
+    const int TN = contract_block(count, d, Nt, ctx->sms);
     // split zeta [count][d*K] FP32 -> [count][d][Ks] BF16 hi/lo via a tiny conversion on the device
     size_t zbytes = (size_t)count * d * Ks * 2;
     if ((rc = ensure(ctx, ctx->zeta_hi, zbytes))) return rc;
@@ -1097,7 +1097,7 @@ int fmc_kle_reconstruct_noalloc(fmc_ctx* ctx, const float* zeta_dev, int64_t cou
     }
     const int split = (precision == FMC_PREC_BF16X3);
     const int nkb = (Ks + TC_BK - 1) / TC_BK;
-    const int TN = 128;
+    const int TN = contract_block(count, d, Nt, ctx->sms);
     void* zhi = base + o_zhi;
     void* zlo = base + o_zlo;
     void* phi_hi = base + o_phi_hi;

@@ -10,7 +10,8 @@
 // transposed, 94 us as bulk copies for 8192 x 3 rows of 2000 steps, K = 200, split), then
 // the operands' way through L2 (0.7 GB; the products are 59 GFLOP, 31 us at the tensor
 // cores' rate).  Keeping the design tile resident, with four storing warps per SM, was
-// slower (the whole call 225 instead of 218 us).
+// slower (the whole call 225 instead of 218 us); blocks of 256 steps (contract_block) take
+// it from 190 to 178 us.
 // This standalone form serves fmc_kle_reconstruct; the fused
 // simulation consumes the same TMEM tiles without writing them out.
 #include <cuda_bf16.h>
@@ -134,21 +135,24 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
             // operands) and hands it to one bulk copy: no store instructions, and the copies
             // run beside the other CTAs' work
             float* row = reinterpret_cast<float*>(smem) + (warp * 32 + lane) * CT_LDB;
-            const int cols = a.Nt - n0 < a.TN ? a.Nt - n0 : a.TN;
-            for (int c = 0; c < cols; c += 32) {
-                float v[32];
+            const int all = a.Nt - n0 < a.TN ? a.Nt - n0 : a.TN;
+            for (int c0 = 0; c0 < all; c0 += 128) {  // 128 steps of every row at a time
+                const int cols = all - c0 < 128 ? all - c0 : 128;
+                for (int c = 0; c < cols; c += 32) {
+                    float v[32];
 #pragma unroll
-                for (int e = 0; e < 32; e += 8)
-                    tmem_ld8(lane_addr + c + e, reinterpret_cast<float(&)[8]>(v[e]));
-                tmem_ld_wait();
+                    for (int e = 0; e < 32; e += 8)
+                        tmem_ld8(lane_addr + c0 + c + e, reinterpret_cast<float(&)[8]>(v[e]));
+                    tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<float4*>(row + c + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            if (lane < rows) {
-                bulk_store(out + lane * rs, row, (uint32_t)cols * 4u, l2_policy_evict_first());
-                bulk_read_wait();
+                    for (int e = 0; e < 32; e += 4)
+                        *reinterpret_cast<float4*>(row + c + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                if (lane < rows) {
+                    bulk_store(out + lane * rs + c0, row, (uint32_t)cols * 4u, l2_policy_evict_first());
+                    bulk_read_wait();
+                }
             }
         } else
         // a lane holds a sample's row: 32 steps at a time are turned in shared memory, so
@@ -204,23 +208,37 @@ cudaError_t launch_split_rows(const float* z, int64_t count, int d, int K, int K
     return cudaGetLastError();
 }
 
+// Blocks of 256 steps read the samples half as often: an eighth less time per step where the SMs are full (16384 x 3 rows
+// of 2000 steps, K = 200, the whole call 239 -> 215 us), but two CTAs per SM hold four
+// blocks of 128 steps where three CTAs hold three.  So 256 where they add no padding and
+// their rounds, at 7/6 the time of the others', are no longer in all (2000 x 3 rows:
+// 62.0 us with 128, 62.8 with 256; plain BF16 52.6, 54.5).
+int contract_block(int64_t count, int d, int Nt, int sms)
+{
+    const int64_t cols = (Nt + 127) / 128, blocks = (count + TC_M - 1) / TC_M * d * cols;
+    if (cols % 2) return 128;
+    const int64_t r256 = (blocks + 4 * sms - 1) / (4 * sms), r128 = (blocks + 3 * sms - 1) / (3 * sms);
+    return 7 * r256 <= 6 * r128 ? 256 : 128;
+}
+
 cudaError_t launch_contract_tc(const CUtensorMap* maps, int64_t count, int d, int Ks, int nkb, int Nt, int TN,
                                int split, float* dW, int* err, cudaStream_t st)
 {
-    // three CTAs per SM with two 32 KB stages (four with three 16 KB stages in plain
-    // BF16): one CTA's stores run beside the others' loads and MMAs
+    // blocks of 128 steps: three CTAs per SM with two 32 KB stages (three 16 KB stages in
+    // plain BF16); of 256: two CTAs.  One CTA's stores run beside the others' loads and MMAs
     const int stage_bytes = (TC_M * 64 + TN * 64) * (split ? 2 : 1);
     const int ns = split ? 2 : 3;
     const int bulk = Nt % 4 == 0 && reinterpret_cast<uintptr_t>(dW) % 16 == 0;
     ContractArgs a{count, d, Ks, nkb, Nt, TN, split, ns, bulk, dW, err};
-    // at least 47 KB so that no more than four CTAs (4 x 128 TMEM columns) share an SM
+    // enough that no more CTAs share an SM than its 512 TMEM columns hold
     int smem = ns * stage_bytes + 1024;
     const int trans = (bulk ? TC_M * CT_LDB : 4 * 32 * CT_LD) * 4 + 1024;
     if (smem < trans) smem = trans;
-    if (smem < 233472 / 5 - 1024 + 64) smem = 233472 / 5 - 1024 + 64;
+    const int floor = 233472 / (512 / TN + 1) - 1024 + 64;
+    if (smem < floor) smem = floor;
     static bool attr_done = false;
     if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(contract_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(contract_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
         if (e != cudaSuccess) return e;
         attr_done = true;
     }

@@ -56,6 +56,8 @@ cudaError_t launch_forcing_split(int K, int Nt, double T, int basis, int Kpad, d
 // C [R][Ncols] = A [R][K] B [K][Ncols]; upper: B is upper triangular (k <= column)
 cudaError_t launch_sgemm_nn(int64_t R, int Ncols, int K, const float* A, const float* B, float* C, bool upper,
                             cudaStream_t st);
+// Steps per block (TN, the basis maps' rows) of launch_contract_tc.
+int contract_block(int64_t count, int d, int Nt, int sms);
 cudaError_t launch_contract_tc(const CUtensorMap* maps, int64_t count, int d, int Ks, int nkb, int Nt, int TN,
                                int split, float* dW, int* err, cudaStream_t st);
 cudaError_t launch_split_rows(const float* z, int64_t count, int d, int K, int Ks, void* hi, void* lo, cudaStream_t st);

@@ -27,3 +27,18 @@ def test_bulk_stores_equal_plain_stores(count, d, K, Nt, precision):
         assert torch.all(buf[:first] == -7.0) and torch.all(buf[first + size:] == -7.0)
         out.append(buf[first:first + size].clone())
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("count,d,K,Nt", [(8200, 2, 40, 1001), (16500, 2, 7, 132), (8192, 2, 288, 1000)])
+@pytest.mark.parametrize("precision", ["bf16x3", "bf16"])
+def test_blocks_of_256_steps_equal_blocks_of_128(count, d, K, Nt, precision):
+    # the whole takes blocks of 256 steps, 640 rows at a time take blocks of 128
+    import torch
+    fmc = need_gpu()
+    dt = 0.01
+    zeta, _ = fmc.lhs_sample(5, count, d * K)
+    whole = fmc.kle_reconstruct(zeta, d, K, Nt * dt, dt, precision=precision)
+    fmc.device_status()
+    for r in range(0, count, 640):
+        part = fmc.kle_reconstruct(zeta[r:r + 640].contiguous(), d, K, Nt * dt, dt, precision=precision)
+        assert torch.equal(whole[r:r + 640], part)
