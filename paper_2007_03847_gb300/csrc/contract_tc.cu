@@ -12,8 +12,8 @@
 // cores' rate).  Keeping the design tile resident, with four storing warps per SM, was
 // slower (the whole call 225 instead of 218 us); blocks of 256 steps (contract_block) take
 // it from 190 to 178 us.
-// This standalone form serves fmc_kle_reconstruct; the fused
-// simulation consumes the same TMEM tiles without writing them out.
+// This standalone form serves fmc_kle_reconstruct; the fused simulation consumes the same
+// TMEM tiles without writing them out.
 #include <cuda_bf16.h>
 
 #include "fmc_common.cuh"
@@ -208,11 +208,11 @@ cudaError_t launch_split_rows(const float* z, int64_t count, int d, int K, int K
     return cudaGetLastError();
 }
 
-// Blocks of 256 steps read the samples half as often: an eighth less time per step where the SMs are full (16384 x 3 rows
-// of 2000 steps, K = 200, the whole call 239 -> 215 us), but two CTAs per SM hold four
-// blocks of 128 steps where three CTAs hold three.  So 256 where they add no padding and
-// their rounds, at 7/6 the time of the others', are no longer in all (2000 x 3 rows:
-// 62.0 us with 128, 62.8 with 256; plain BF16 52.6, 54.5).
+// Blocks of 256 steps read the samples half as often: an eighth less time per step where
+// the SMs are full (16384 x 3 rows of 2000 steps, K = 200, the whole call 239 -> 215 us).
+// But two CTAs per SM hold four blocks of 128 steps where three CTAs hold three.  So 256
+// where they add no padding and their rounds, at 7/6 the time of the others', are no
+// longer in all (2000 x 3 rows: 62.0 us with 128, 62.8 with 256; plain BF16 52.6, 54.5).
 int contract_block(int64_t count, int d, int Nt, int sms)
 {
     const int64_t cols = (Nt + 127) / 128, blocks = (count + TC_M - 1) / TC_M * d * cols;
