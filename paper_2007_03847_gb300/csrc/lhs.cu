@@ -254,7 +254,6 @@ template <int OUT>
 static cudaError_t launch_design(DesignArgs& a, int sms, cudaStream_t st)
 {
     if (a.count == 0) return cudaSuccess;
-    a.walk = a.h < 16 && ((uint64_t)1 << (2 * a.h)) > a.N;
     if (a.strata_in) return launch_design_t<PERM_GIVEN, OUT>(a, sms, st);
     if (a.mode == FMC_SRS) return launch_design_t<PERM_NONE, OUT>(a, sms, st);
     const bool rows_enough = a.count >= ((int64_t)2 << a.h);
@@ -276,6 +275,7 @@ static DesignArgs design_args(uint64_t seed, int64_t N, int64_t k0, int64_t coun
     a.mode = mode;
     a.h = f.h;
     a.mask = f.mask;
+    a.walk = f.walk;
     a.rcp = (N & (N - 1)) == 0 ? 0x1p-32f / (float)N : 0.f;
     return a;
 }

@@ -15,9 +15,13 @@ constexpr int kFeistelRounds = 6;
 // f_r(R) = Philox word 0 of the counter (R, dim, 1 + r, 0), masked to h bits;
 // pi_dim(k) is the first iterate of it from k that falls in [0, N) (cycle walking
 // ends: the cycle through k < N returns to [0, N) within 4^h - N + 1 applications).
+// walk: N < 4^h, some values fall outside (every N that is no power of four, also above
+// 2^30, where h = 16 and 4^h no longer fits 32 bits; the correlation-reducing
+// permutation of one column takes N up to 2^31 - 1).
 struct FeistelShape {
     int h;
     uint32_t mask;
+    bool walk;
 };
 
 inline FeistelShape feistel_shape(int64_t N)
@@ -29,6 +33,7 @@ inline FeistelShape feistel_shape(int64_t N)
     FeistelShape f;
     f.h = h;
     f.mask = (h >= 32) ? 0xFFFFFFFFu : ((1u << h) - 1u);
+    f.walk = ((uint64_t)1 << (2 * h)) > (uint64_t)N;
     return f;
 }
 
