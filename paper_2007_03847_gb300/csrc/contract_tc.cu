@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(128) contract_tc_kernel(const __grid_constant_
                     bulk_store(out + lane * rs + c0, row, (uint32_t)cols * 4u, l2_policy_evict_first());
                     bulk_read_wait();
                 }
+                __syncwarp();  // (the next loads from TMEM are the whole warp's)
             }
         } else
         // a lane holds a sample's row: 32 steps at a time are turned in shared memory, so
