@@ -237,12 +237,9 @@ cudaError_t launch_contract_tc(const CUtensorMap* maps, int64_t count, int d, in
     if (smem < trans) smem = trans;
     const int floor = 233472 / (512 / TN + 1) - 1024 + 64;
     if (smem < floor) smem = floor;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(contract_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    // (an attribute of the current device, always the same bound: launches may race on it)
+    cudaError_t e = cudaFuncSetAttribute(contract_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+    if (e != cudaSuccess) return e;
     int64_t gy = (count + TC_M - 1) / TC_M;
     if (gy > 65535) return cudaErrorInvalidValue;
     dim3 grid((Nt + TN - 1) / TN, (unsigned)gy, d);
