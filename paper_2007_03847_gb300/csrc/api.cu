@@ -1188,10 +1188,11 @@ static int choose_kernel(fmc_ctx* ctx, const std::vector<fmc_launch_rule>* rules
     int policy = user_policy;
     if (policy == FMC_KERNEL_AUTO && path == FMC_PATH_FUSED && rules) {
         // (a rule's kernel that cannot take this system is ignored: a bucket's
-        // rule was measured at its largest machine count)
+        // rule was measured at its largest machine count, without smooth forcing)
         const fmc_launch_rule* rule = find_rule_in(*rules, s, count);
         if (rule && rule->kernel != FMC_KERNEL_AUTO && !(rule->kernel == FMC_KERNEL_PER_SAMPLE && C.nm < 0) &&
-            !(rule->kernel == FMC_KERNEL_SPLIT_TC && !wide_tc_built(wide_nmt_for(n))))
+            !(rule->kernel == FMC_KERNEL_SPLIT_TC && !wide_tc_built(wide_nmt_for(n))) &&
+            !(rule->kernel != FMC_KERNEL_PER_SAMPLE && C.nm >= 0 && s->forcing == FMC_FORCING_SMOOTH))
             policy = rule->kernel;
     }
     const bool per_sample = policy == FMC_KERNEL_PER_SAMPLE;
