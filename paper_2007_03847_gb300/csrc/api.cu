@@ -564,8 +564,11 @@ static int run_equilibrium_ws(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s
     if (rc) return rc;
     rc = ensure(ctx, ws.eq, 4 * (size_t)n * sizeof(double));
     if (rc) return rc;
+    const bool fresh = !ws.status.ptr;
     rc = ensure(ctx, ws.status, 64);
     if (rc) return rc;
+    // (a call that runs no kernel with bounded waits leaves the error word as it is)
+    if (fresh) FMC_CUDA(ctx, cudaMemsetAsync(ws.status.ptr, 0, 64, st), "memset");
     std::vector<double> h(nd, 0.0);
     double* G = h.data();
     double* B = G + n * n;
@@ -1560,6 +1563,8 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
     double* trig = trig_if_ready(ws, K, Nt, s->basis, s->forcing == FMC_FORCING_SMOOTH);
     EmSpec ems{em ? 1 : 0, (uint32_t)s->seed, (uint32_t)(s->seed >> 32), k0, (float)std::sqrt(s->dt)};
 
+    // this call's error word (fmc_device_status), on both paths
+    FMC_CUDA(ctx, cudaMemsetAsync((char*)ws.status.ptr + 4, 0, 4, st), "memset");
     if (P.path == FMC_PATH_PLAIN) {
         const int M = d * K;
         float* traj = traj_dev ? traj_dev : (float*)ws.traj.ptr;
@@ -1653,7 +1658,6 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
                                         Ks, smooth ? 2 * Nt + 1 : Nt, Kpad, cw, split, shape.rows)))
             return rc;
     }
-    FMC_CUDA(ctx, cudaMemsetAsync((char*)ws.status.ptr + 4, 0, 4, st), "memset");
     if (!per_tile_partials && !P.team) {
         FMC_CUDA(ctx, cudaMemsetAsync(S1, 0, Nt1 * S * sizeof(double), st), "memset");
         FMC_CUDA(ctx, cudaMemsetAsync(S2, 0, Nt1 * S * sizeof(double), st), "memset");
