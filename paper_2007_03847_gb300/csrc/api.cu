@@ -83,7 +83,9 @@ struct fmc_ctx {
     size_t prof_cap = 0;
     int last_fused_ctas_per_sm = 0;
     int kernel_policy = FMC_KERNEL_AUTO;
-    bool team = true;  // the team kernel may be taken (the server: where its partials were charged)
+    // (the server: where a request was charged for them)
+    bool team = true;   // the team kernel may be taken
+    bool table = true;  // the basis kernels may tabulate their cosines
     std::vector<fmc_launch_rule> rules;  // measured launch shapes (fmc_set_launch_rules)
     // Contexts used on one stream only (the server's) grow their workspace in
     // stream order on that stream (cudaFreeAsync / cudaMallocAsync) instead of
@@ -133,10 +135,13 @@ static int cuda_fail(fmc_ctx* ctx, cudaError_t e, const char* what)
         if (_e != cudaSuccess) return cuda_fail(ctx, _e, what); \
     } while (0)
 
+// What a buffer of `bytes` grows to.
+static size_t grown(size_t bytes) { return bytes + bytes / 8; }
+
 static int ensure(fmc_ctx* ctx, DevBuf& b, size_t bytes)
 {
     if (b.bytes >= bytes) return FMC_OK;
-    size_t want = bytes + bytes / 8;
+    size_t want = grown(bytes);
     if (ctx->budget && ctx->used - b.bytes + want > ctx->budget) {
         want = bytes;
         if (ctx->used - b.bytes + want > ctx->budget)
@@ -165,11 +170,12 @@ static int ensure(fmc_ctx* ctx, DevBuf& b, size_t bytes)
 }
 
 // The basis kernels' table of cosines (basis_table_doubles), grown if need be; null
-// where a memory budget has no room for it: the kernels then do without.
+// in a context with a memory budget or a request not charged for it: the kernels then
+// do without.
 static double* trig_table(fmc_ctx* ctx, Workspace& ws, int K, int Nt, int basis, int forcing)
 {
     const size_t bytes = (size_t)basis_table_doubles(K, Nt, basis, forcing) * sizeof(double);
-    if (ctx->budget && ws.trig.bytes < bytes) return nullptr;
+    if (!ctx->table || (ctx->budget && ws.trig.bytes < bytes)) return nullptr;
     if (ensure(ctx, ws.trig, bytes) != FMC_OK) return nullptr;
     return (double*)ws.trig.ptr;
 }
@@ -1835,12 +1841,21 @@ size_t fmc::team_bytes(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, 
 {
     const int Nt = (int)std::llround(s->T / s->dt);
     const int nm = nm_bucket_for(s->n);
-    return team_fits(ctx->sms, nm, 0, path, s->n, Nt, count) ? team_part_bytes(s->n, Nt, count) : 0;
+    return team_fits(ctx->sms, nm, 0, path, s->n, Nt, count) ? grown(team_part_bytes(s->n, Nt, count)) : 0;
 }
 
-void fmc::set_team(fmc_ctx* ctx, bool on)
+size_t fmc::table_bytes(const fmc_scenario* s)
 {
-    if (ctx) ctx->team = on;
+    if (s->sampling == FMC_SRS_EM) return 0;
+    const int Nt = (int)std::llround(s->T / s->dt);
+    return grown((size_t)basis_table_doubles(s->K, Nt, s->basis, s->forcing == FMC_FORCING_SMOOTH) * sizeof(double));
+}
+
+void fmc::set_extras(fmc_ctx* ctx, bool team, bool table)
+{
+    if (!ctx) return;
+    ctx->team = team;
+    ctx->table = table;
 }
 
 void fmc::set_stream_ordered(fmc_ctx* ctx, bool on)

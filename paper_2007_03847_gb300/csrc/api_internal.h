@@ -68,11 +68,13 @@ int release_workspace(fmc_ctx* ctx, cudaStream_t st);
 // (without solving anything), on stream st when the context is stream-ordered.
 int reserve_workspace(fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count, cudaStream_t st);
 
-// Bytes of per-group partials that simulate_moments of `count` samples of s holds
-// beyond the design and basis (the team kernel's), 0 where it takes another kernel;
-// and whether ctx may take that kernel.
+// Bytes that simulate_moments of `count` samples of s holds beyond the design and
+// basis, as its buffers grow: the team kernel's per-group partials (0 where it takes
+// another kernel), and the basis kernels' cosine table; and whether ctx may take them
+// (the results are the same without).
 size_t team_bytes(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count);
-void set_team(fmc_ctx* ctx, bool on);
+size_t table_bytes(const fmc_scenario* s);
+void set_extras(fmc_ctx* ctx, bool team, bool table);
 
 // fmc_simulate with a choice of how the fused kernel combines its per-time sums:
 // per_tile_partials = true writes FP32 partials per 128-sample tile and adds them

@@ -32,7 +32,8 @@ struct Request {
     double* mean = nullptr;
     double* var = nullptr;
     size_t bytes = 0;  // device memory charged against the budget
-    bool team = true;  // the team kernel's partials are part of the charge
+    bool team = true;   // the team kernel's partials are part of the charge
+    bool table = true;  // the basis kernels' cosine table is
     int status = FMC_NOT_READY;
     bool started = false;
     std::string error;
@@ -266,7 +267,7 @@ static void worker_loop(fmc_server* srv, int slot)
         }
         // moments summed with FP64 atomics (no per-tile partial buffers to hold), or
         // by the team kernel where its partials were charged
-        for (int k = 0; k < kReplicates; ++k) fmc::set_team(rctx[k], r->team);
+        for (int k = 0; k < kReplicates; ++k) fmc::set_extras(rctx[k], r->team, r->table);
         int rc;
         if (r->tol_E > 0 || r->tol_Var > 0) {
             rc = run_target(rctx, rst, r);
@@ -389,8 +390,12 @@ static int submit_request(fmc_server* srv, const fmc_scenario* scen, int32_t pat
     }
     r->bytes = request_bytes(largest, path) * (target ? (size_t)kReplicates : 1u) +
                (n_mm > 0 ? (size_t)merged_part_bytes(*scen, kReplicates * n_mm) : 0u);
-    // small designs take the team kernel, whose partials are charged for the largest
-    // round that takes it; a request they alone would put past the budget does without
+    // the basis' cosine table, in every context that a round uses, and the team kernel's
+    // partials for the largest round that takes it: a request that one of them alone would
+    // put past the budget does without it
+    const size_t table = fmc::table_bytes(scen) * (target && n_mm < largest.N ? (size_t)kReplicates : 1u);
+    r->table = r->bytes + table <= srv->budget;
+    if (r->table) r->bytes += table;
     size_t team = 0;
     for (int64_t n = scen->N; n <= largest.N; n *= 4) {
         const size_t t = !target     ? fmc::team_bytes(srv->ctxs[0], scen, path, n)
