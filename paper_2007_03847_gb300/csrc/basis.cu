@@ -25,8 +25,9 @@ namespace fmc {
 // only P' distinct cosines for K Nt entries.  FP64 arithmetic is the bound (two FMA
 // per SM and clock on this part), so the cosines of all residues are tabulated once
 // per call (trig_table_kernel) and an entry costs two FP64 products, the residue kept
-// by additions modulo the period along a thread's times.  Without room for the table
-// (the allocation-free reconstruction) a thread evaluates the cosine itself.  The
+// by additions modulo the period along a thread's times.  Without the table (few
+// entries, no room for it, the allocation-free reconstruction) a thread evaluates the
+// cosine itself.  The
 // operations per entry are the same either way, in the same order.
 // Measured (GB300), split form: K = 200, Nt = 4000 148 -> 28 us; K = 100, Nt = 1000
 // 32 -> 17 us, the table's 4 us included.
@@ -62,6 +63,11 @@ __device__ __forceinline__ double basis_cos(int64_t m, int Nt, int basis)
     return cospi((double)m / (basis == FMC_BASIS_COSINE ? 2.0 * Nt : 4.0 * Nt));
 }
 
+// The forcing of the smooth form (Eq. eqkl as a random ODE): the time
+// derivative of the basis function at the half-step times t = j T / (2 Nt),
+// j = 0..2 Nt.  Brownian eigenbasis: sqrt(2/T) cos((k+1/2) pi t / T) =
+// sqrt(2/T) cospi((2k+1) j / (4 Nt)), the argument reduced modulo 8 Nt; the
+// paper's basis: 1/sqrt(T) (k = 0), sqrt(2/T) cospi(k j / (2 Nt)) (mod 4 Nt).
 // What an entry of row k needs besides its cosine: value = (amp cos) sine (increments)
 // or amp cos (forcing); the constant mode of the cosine basis has no cosine.
 struct BasisRow {
@@ -151,12 +157,12 @@ __device__ __forceinline__ int64_t basis_advance(const BasisArgs& a, const Basis
 __global__ void __launch_bounds__(256) basis_f32_kernel(BasisArgs a, int J, float* __restrict__ phi)
 {
     const int64_t P = basis_period(a.Nt, a.basis);
-    const int64_t step = (int64_t)gridDim.x * 256;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
     for (int k = blockIdx.y; k < a.K; k += gridDim.y) {
         const BasisRow r = basis_row_of(a, k);
-        int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x;
+        int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
         int64_t m = basis_residue(a, r, j);
-        const int64_t dm = basis_advance(a, r, step);
+        const int64_t dm = j + step < J ? basis_advance(a, r, step) : 0;
         for (; j < J; j += step) {
             phi[(int64_t)k * J + j] = basis_entry(a, r, m);
             m += dm;
@@ -166,20 +172,19 @@ __global__ void __launch_bounds__(256) basis_f32_kernel(BasisArgs a, int J, floa
 }
 
 // Time-major split BF16 for the tensor-core B operand: hi/lo [J][Kpad], zeros for
-// k >= K.  A thread keeps its k and steps over times.
-constexpr int BASIS_TIMES = 8;  // times per CTA of 8 x 32 threads and pass
-
+// k >= K.  A thread keeps its k and steps over times, a warp (32 k) per time.
 __global__ void __launch_bounds__(256) basis_split_kernel(BasisArgs a, int J, int Kpad, __nv_bfloat16* __restrict__ hi,
                                                           __nv_bfloat16* __restrict__ lo)
 {
     const int64_t P = basis_period(a.Nt, a.basis);
-    const int64_t step = (int64_t)gridDim.x * BASIS_TIMES;
+    const int times = (int)blockDim.x / 32;
+    const int64_t step = (int64_t)gridDim.x * times;
     for (int k = blockIdx.y * 32 + threadIdx.x % 32; k < Kpad; k += gridDim.y * 32) {
         const bool real = k < a.K;
         const BasisRow r = basis_row_of(a, real ? k : 0);
-        int64_t j = blockIdx.x * (int64_t)BASIS_TIMES + threadIdx.x / 32;
+        int64_t j = blockIdx.x * (int64_t)times + threadIdx.x / 32;
         int64_t m = basis_residue(a, r, j);
-        const int64_t dm = basis_advance(a, r, step);
+        const int64_t dm = j + step < J ? basis_advance(a, r, step) : 0;
         for (; j < J; j += step) {
             const float v = real ? basis_entry(a, r, m) : 0.f;
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
@@ -191,15 +196,15 @@ __global__ void __launch_bounds__(256) basis_split_kernel(BasisArgs a, int J, in
     }
 }
 
-// The forcing of the smooth form (Eq. eqkl as a random ODE): the time
-// derivative of the basis function at the half-step times t = j T / (2 Nt),
-// j = 0..2 Nt.  Brownian eigenbasis: sqrt(2/T) cos((k+1/2) pi t / T) =
-// sqrt(2/T) cospi((2k+1) j / (4 Nt)), the argument reduced modulo 8 Nt; the
-// paper's basis: 1/sqrt(T) (k = 0), sqrt(2/T) cospi(k j / (2 Nt)) (mod 4 Nt).
-static cudaError_t basis_prepare(BasisArgs& a, double* table, cudaStream_t st)
+// The table pays from some ten thousand entries on: filling it is a launch of its own
+// (50 x 500 entries, FP32 result of 128 rows: 27 us with it, 25 without; 6 x 12000 split:
+// 35 with it, 62 without).
+constexpr int64_t BASIS_TABLE_MIN = 32768;
+
+static cudaError_t basis_prepare(BasisArgs& a, double* table, int64_t entries, cudaStream_t st)
 {
     a.table = nullptr;
-    if (!table) return cudaSuccess;
+    if (!table || entries < BASIS_TABLE_MIN) return cudaSuccess;
     a.cosines = basis_table_entries(a.Nt, a.basis, a.forcing);
     const int odd = a.basis == FMC_BASIS_SINE && !a.forcing;
     trig_table_kernel<<<(unsigned)((a.cosines + a.K + 63) / 64), 64, 0, st>>>(a, odd, table);
@@ -207,34 +212,54 @@ static cudaError_t basis_prepare(BasisArgs& a, double* table, cudaStream_t st)
     return cudaGetLastError();
 }
 
+// Threads per block and entries per thread.  A thread's row constants and residue cost a
+// few entries' work, so it takes up to eight entries once there are enough of them; and
+// since a lone SM's FP64 pipe takes 16 cycles per warp instruction, small tables go to
+// the SMs in blocks of 64 threads.  Measured (GB300, FP32 rows without the table, launches
+// in a row; eight entries per thread in blocks of 256 -> now): 6 x 400 entries 12.4 ->
+// 7.6 us, 60 x 4000 39 -> 25, 200 x 4000 70 either way.
+struct BasisShape {
+    int threads;
+    int64_t entries;
+};
+
+static BasisShape basis_shape(int64_t entries, int sms)
+{
+    const int64_t e = entries / ((int64_t)sms * 128);
+    return BasisShape{e < 8 ? 64 : 256, e < 1 ? 1 : (e > 8 ? 8 : e)};
+}
+
 static cudaError_t launch_f32(BasisArgs a, double* table, float* phi, int sms, cudaStream_t st)
 {
-    cudaError_t e = basis_prepare(a, table, st);
-    if (e != cudaSuccess) return e;
     const int64_t J = a.forcing ? 2 * (int64_t)a.Nt + 1 : a.Nt;
     if (J > 2147483647LL) return cudaErrorInvalidValue;
+    cudaError_t e = basis_prepare(a, table, a.K * J, st);
+    if (e != cudaSuccess) return e;
+    const BasisShape b = basis_shape(a.K * J, sms);
     const int gy = a.K < 65535 ? a.K : 65535;
-    // eight entries or more per thread: its row and residue cost a few entries' work
-    int64_t gx = (J + 256 * 8 - 1) / (256 * 8);
+    const int64_t per = b.threads * b.entries;
+    int64_t gx = (J + per - 1) / per;
     const int64_t cap = ((int64_t)sms * 16 + gy - 1) / gy;
     if (gx > cap) gx = cap;
-    basis_f32_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(a, (int)J, phi);
+    basis_f32_kernel<<<dim3((unsigned)gx, (unsigned)gy), b.threads, 0, st>>>(a, (int)J, phi);
     return cudaGetLastError();
 }
 
 static cudaError_t launch_split(BasisArgs a, double* table, int Kpad, void* hi, void* lo, int sms, cudaStream_t st)
 {
-    cudaError_t e = basis_prepare(a, table, st);
-    if (e != cudaSuccess) return e;
     const int64_t J = a.forcing ? 2 * (int64_t)a.Nt + 1 : a.Nt;
     if (J > 2147483647LL) return cudaErrorInvalidValue;
+    cudaError_t e = basis_prepare(a, table, a.K * J, st);
+    if (e != cudaSuccess) return e;
+    const BasisShape b = basis_shape(Kpad * J, sms);
     const int ky = Kpad / 32;
     const int gy = ky < 65535 ? ky : 65535;
-    int64_t gx = (J + BASIS_TIMES * 8 - 1) / (BASIS_TIMES * 8);
+    const int64_t per = b.threads / 32 * b.entries;
+    int64_t gx = (J + per - 1) / per;
     const int64_t cap = ((int64_t)sms * 16 + gy - 1) / gy;
     if (gx > cap) gx = cap;
-    basis_split_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(a, (int)J, Kpad, (__nv_bfloat16*)hi,
-                                                                         (__nv_bfloat16*)lo);
+    basis_split_kernel<<<dim3((unsigned)gx, (unsigned)gy), b.threads, 0, st>>>(a, (int)J, Kpad, (__nv_bfloat16*)hi,
+                                                                              (__nv_bfloat16*)lo);
     return cudaGetLastError();
 }
 
