@@ -25,25 +25,29 @@ constexpr int DESIGN_SMEM_MAX = 224 * 1024;
 // up to 16 x 2^h.
 //
 // Layout: a thread keeps one position (column) and steps over rows, with DB
-// neighbouring positions in neighbouring lanes, so that a row's outputs go out as
-// whole 32-byte sectors and no index division is left in the loop.  Strata go
+// neighbouring positions in neighbouring lanes (16 bytes of a row; the rest of a
+// sector meets them in L2), and no index division is left in the loop.  Strata go
 // through a short per-thread list in shared memory: walking lanes take their next
 // row as soon as their value is found instead of waiting for the warp's longest
 // walk, and the list is read transposed where strata themselves are stored or
 // loaded (their rows run along the samples).
 //
-// Measured (GB300): 65536 x 600 values and strata 735 -> 361 us (entries computed
-// one by one from the definition before; 0.9 TB/s of output, the uniform's Philox
-// call and the two branches of the inverse CDF now take the issue slots); the
-// split-BF16 rows of 19001 x 2400 (domain 4^8, 3.4 walks per entry) 6.99 -> 0.70 ms.
+// Measured (GB300, launches in a row): 65536 x 600 values and strata 735 -> 308 us
+// (entries computed one by one from the definition before; 1 TB/s of output, the
+// uniform's Philox call and the two branches of the inverse CDF now take the issue
+// slots); the split-BF16 rows of 19001 x 2400 (domain 4^8, 3.4 walks per entry) 6.98 ->
+// 0.60 ms.  With 16 positions per CTA (8 with uint16 tables) these took 361 us and
+// 0.69 ms, the tables' filling being four times as long, and few columns left lanes
+// idle: 2^20 x 20 by simple random sampling 179 us (one by one 125, now 115),
+// 4.2e6 x 4 by the definition 4.61 ms (2.93, 1.37), 2^20 x 1 325 us (25, 23).
 // ---------------------------------------------------------------------------
 enum { PERM_NONE = 0, PERM_DIRECT, PERM_TAB8, PERM_TAB16, PERM_GIVEN };
 enum { OUT_F32 = 0, OUT_SPLIT, OUT_SCORE };
 
-template <int PERM>
+template <int PERM, int DBN>
 struct DesignTile {
     static constexpr int THREADS = PERM == PERM_TAB16 ? 512 : 256;
-    static constexpr int DB = PERM == PERM_TAB16 ? 8 : 16;   // positions per CTA
+    static constexpr int DB = DBN;  // positions per CTA
     static constexpr int RPI = THREADS / DB;                 // rows per pass of the CTA
     static constexpr int LCAP = PERM == PERM_TAB16 ? 4 : 16; // list entries per thread
     static constexpr int SUB = RPI * LCAP;                   // rows per list filling
@@ -93,10 +97,10 @@ __device__ __forceinline__ uint32_t permute(const void* tab, uint32_t x, const D
     return (L << a.h) | R;
 }
 
-template <int PERM, int OUT>
-__global__ void __launch_bounds__(DesignTile<PERM>::THREADS) design_kernel(const DesignArgs a)
+template <int PERM, int OUT, int DB>
+__global__ void __launch_bounds__(DesignTile<PERM, DB>::THREADS) design_kernel(const DesignArgs a)
 {
-    using T = DesignTile<PERM>;
+    using T = DesignTile<PERM, DB>;
     extern __shared__ __align__(16) unsigned char dsm[];
     uint32_t* list = reinterpret_cast<uint32_t*>(dsm);
     unsigned char* tabs = dsm + T::LIST_BYTES;
@@ -218,10 +222,10 @@ __global__ void __launch_bounds__(DesignTile<PERM>::THREADS) design_kernel(const
     }
 }
 
-template <int PERM, int OUT>
-static cudaError_t launch_design_t(DesignArgs& a, int sms, cudaStream_t st)
+template <int PERM, int OUT, int DB>
+static cudaError_t launch_design_db(DesignArgs& a, int sms, cudaStream_t st)
 {
-    using T = DesignTile<PERM>;
+    using T = DesignTile<PERM, DB>;
     constexpr bool TAB = PERM == PERM_TAB8 || PERM == PERM_TAB16;
     a.npos = (a.cols + T::DB - 1) / T::DB;
     // rows per CTA: four CTAs per SM in all, but 2 .. 16 rows per table entry where
@@ -235,7 +239,7 @@ static cudaError_t launch_design_t(DesignArgs& a, int sms, cudaStream_t st)
     while ((a.count + rows - 1) / rows * a.npos > 2147483647LL) rows *= 2;
     a.rows = rows;
     const int smem = T::LIST_BYTES + (TAB ? T::DB * (kFeistelRounds << a.h) * (PERM == PERM_TAB8 ? 1 : 2) : 0);
-    auto kern = design_kernel<PERM, OUT>;
+    auto kern = design_kernel<PERM, OUT, DB>;
     if (smem > 48 * 1024) {
         // process-wide attribute: always the same bound (launches may race on it)
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DESIGN_SMEM_MAX);
@@ -246,8 +250,15 @@ static cudaError_t launch_design_t(DesignArgs& a, int sms, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// The rule: tables while they fit (uint8 up to h = 8, 24 KB; uint16 up to h = 11,
-// 192 KB) and a block of rows at least 2^(h+1) long repays them; the rounds from
+// Four positions per CTA, or one where there are fewer than four (idle lanes).
+template <int PERM, int OUT>
+static cudaError_t launch_design_t(DesignArgs& a, int sms, cudaStream_t st)
+{
+    return a.cols < 4 ? launch_design_db<PERM, OUT, 1>(a, sms, st) : launch_design_db<PERM, OUT, 4>(a, sms, st);
+}
+
+// The rule: tables while they fit (uint8 up to h = 8, 6 KB; uint16 up to h = 11,
+// 96 KB) and a block of rows at least 2^(h+1) long repays them; the rounds from
 // their definition above (more than 2^22 samples) and for short blocks of a large
 // design; no permutation for simple random sampling.
 template <int OUT>
