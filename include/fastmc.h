@@ -552,8 +552,8 @@ int fmc_set_kernel_policy(fmc_ctx* ctx, int32_t policy);
  * what the TMEM share of max_ctas CTAs holds (and to 16 at least); the
  * large-system kernel keeps one CTA per SM.  max_ctas is a bound for a launch
  * that needs no more: one per SM becomes two where the 128-sample tiles are
- * more than the SMs, and launches of up to two tiles per SM that share the GPU
- * (a batch, a server) take two.  The rules are copied; count 0
+ * more than the SMs, and the launches of a batch take one to three as they need
+ * together (those of a server, two).  The rules are copied; count 0
  * clears them.  FMC_EINVAL on a malformed rule (empty range, kernel not an
  * FMC_KERNEL_* value, max_ctas outside 0..4, TC not 0 or a power of two in
  * 16..256).

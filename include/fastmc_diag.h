@@ -77,6 +77,16 @@ int fmc_diag_net_matrix(const fmc_scenario* scen, int32_t nmt, int32_t H, float*
  */
 int fmc_diag_kernel_choice(const fmc_scenario* scen, int32_t path, int32_t policy, int64_t count, int32_t* out);
 
+/*
+ * How a batch's launches share a GPU of `sms` SMs (host only, no device; no launch
+ * rules, no memory budget): per scenario i out[3 i] 1 where it takes the team kernel
+ * (few samples), out[3 i + 1] the resident CTAs per SM of its per-sample launch (0 for
+ * other kernels and where no plan applies), out[3 i + 2] the CTAs that its tiles are
+ * dealt to (0: one CTA per tile).  Returns a scenario's refusal (FMC_EUNSUPPORTED).
+ * Errors: FMC_EINVAL (arguments).
+ */
+int fmc_diag_batch_plan(const fmc_scenario* scen, int32_t n_scen, int32_t path, int32_t sms, int32_t* out);
+
 /* CTAs per SM the last fused launch could keep resident (occupancy API). */
 int fmc_last_fused_occupancy(const fmc_ctx* ctx, int* ctas_per_sm);
 

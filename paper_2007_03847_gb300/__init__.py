@@ -16,7 +16,7 @@ Entry points (same names as the C ABI without the ``fmc_`` prefix):
 (``set_kernel_policy``: "auto", "per_sample", "split", "split_tc";
 ``set_launch_rules``) and the diagnostics of ``include/fastmc_diag.h``
 (``profile``/``profile_read``, ``check_wait_path``, ``kernel_choice``,
-``net_matrix``).
+``batch_plan``, ``net_matrix``).
 """
 from __future__ import annotations
 
@@ -124,6 +124,7 @@ def load_library():
             "fmc_profile_read": ([vp, i32, ctypes.POINTER(dbl), ctypes.POINTER(i64)], ctypes.c_int),
             "fmc_last_fused_occupancy": ([vp, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
             "fmc_diag_net_matrix": ([vp, i32, i32, vp, i64], ctypes.c_int),
+            "fmc_diag_batch_plan": ([vp, i32, i32, i32, vp], ctypes.c_int),
             "fmc_diag_kernel_choice": ([vp, i32, i32, i64, vp], ctypes.c_int),
             "fmc_set_kernel_policy": ([vp, ctypes.c_int32], ctypes.c_int),
             "fmc_test_sincos": ([vp, vp, i64, vp, vp, vp, vp, vp], ctypes.c_int),
@@ -705,6 +706,20 @@ def kernel_choice(scenario, policy="auto", path="fused", count=None):
     names = {KERNEL_PER_SAMPLE: "per_sample", KERNEL_SPLIT: "split", KERNEL_SPLIT_TC: "split_tc"}
     return {"kernel": names[int(out[0])], "nmt": int(out[1]), "H": int(out[2]), "nd": int(out[3]),
             "bus": bool(out[4])}
+
+
+def batch_plan(scenarios, path="fused", sms: int = 152):
+    """fmc_diag_batch_plan: how a batch's launches share the GPU (host only, no GPU), per
+    scenario as a dict: "team", "per_sm" and "ctas" (0: one CTA per tile)."""
+    lib = load_library()
+    structs = [ScenarioStruct(sc, precision="bf16x3") for sc in scenarios]
+    arr = (_Scenario * len(structs))(*[s.s for s in structs])
+    out = np.zeros((len(structs), 3), dtype=np.int32)
+    p = _PATH.get(path, path) if isinstance(path, str) else path
+    rc = lib.fmc_diag_batch_plan(arr, len(structs), int(p), int(sms), out.ctypes.data)
+    if rc != OK:
+        raise FastMCError(rc, "fmc_diag_batch_plan refused")
+    return [{"team": bool(t), "per_sm": int(s), "ctas": int(c)} for t, s, c in out]
 
 
 def set_kernel_policy(policy, ctx: Context | None = None) -> None:

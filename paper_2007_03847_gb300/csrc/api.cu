@@ -1154,7 +1154,8 @@ struct Prepared {
     bool bus = false;  // ... for a system with an infinite bus (its own instantiations)
     bool exclusive = true;  // the launch has the GPU to itself (see fused_shape)
     bool team = false;      // few samples: the team kernel (see team_wanted)
-    int share = 0;          // CTAs of a sliced launch among others of its batch (batch_shares)
+    int share = 0;          // CTAs of a sliced launch among others of its batch (batch_shares),
+    int per_sm = 0;         // and resident CTAs per SM of its per-sample launches (0: no plan)
     int64_t k0 = 0, count = 0;
     std::vector<unsigned char> params;
 };
@@ -1355,25 +1356,15 @@ static int prepare(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s, int64_t k
 
 // Time chunk TC of the fused kernels.  A CTA's accumulator holds d x TC FP32
 // TMEM columns (512 per SM), and every chunk boundary reloads the CTA's design
-// tile through the shared-memory ring (a latency the CTA waits out).  When the
-// GPU is the call's alone and the tiles need fewer than four CTAs per SM, each
-// CTA may take more columns, so the chunk grows (up to 256 steps) and the
-// boundaries become rarer; launches that share the GPU (batches, the server)
-// keep 128 columns per CTA.
+// tile through the shared-memory ring (a latency the CTA waits out).  Where the
+// tiles need fewer than four CTAs per SM, each CTA may take more columns, so the
+// chunk grows (up to 256 steps) and the boundaries become rarer.
 //
-// Samples per CTA: 128 (four warps) when the GPU is shared.  The kernel also
-// runs 64-sample CTAs (two warps); they would even out the warps per SM of 2^16
-// samples, but their TMEM share forces 16-step chunks and the doubled
-// design-tile reloads cost more than the balance gains (38.9 vs 35.1 ms), so the
-// automatic shape keeps 128.
-//
-// With N = 2^16 the 2048 warps of 4-warp CTAs leave 3.37 warps per SM
-// sub-partition on average against at most 4 (56 SMs with four CTAs, 96 with
-// three), and the launch lasts as long as the 4-warp sub-partitions: a
-// quantisation of whole warps that no CTA shape removes.  (A form with one CTA
-// of 14 integrating warps and a producer warp per SM, the contraction
-// double-buffered in TMEM, measured no faster: two of its four sub-partitions
-// still hold four warps.)
+// Samples per CTA: 128 (four warps).  The kernel also runs 64-sample CTAs (two
+// warps); they would even out the warps per SM of 2^16 samples, but their TMEM
+// share forces 16-step chunks and the doubled design-tile reloads cost more than
+// the balance gains (38.9 vs 35.1 ms), so the automatic shape keeps 128 (and evens
+// out the SMs by slices, below).
 struct FusedShape {
     int rows;       // samples per CTA
     int max_ctas;   // resident CTAs per SM allowed
@@ -1405,11 +1396,11 @@ struct SliceShape {
     int steps;
 };
 
-static SliceShape slice_shape(const fmc_ctx* ctx, const Prepared& P, int TC)
+static SliceShape slice_shape(int64_t sms, bool budget, const Prepared& P, int TC)
 {
     SliceShape s{0, 0, (P.count + TC_M - 1) / TC_M, 0};
-    if (P.nmt > 0 || P.team || P.s.forcing == FMC_FORCING_SMOOTH || ctx->budget != 0) return s;
-    const int64_t sms = ctx->sms, t = s.tiles;
+    if (P.nmt > 0 || P.team || P.s.forcing == FMC_FORCING_SMOOTH || budget) return s;
+    const int64_t t = s.tiles;
     int64_t slots = 0;
     if (!P.exclusive) {
         slots = P.share;
@@ -1420,9 +1411,10 @@ static SliceShape slice_shape(const fmc_ctx* ctx, const Prepared& P, int TC)
         else if (t <= 3 * sms && t > 2 * sms && 5 * t < 14 * sms)
             slots = 2 * sms;
     }
-    if (slots <= 0 || t <= slots || t % slots == 0) return s;
+    if (slots <= 0 || t <= slots || (P.exclusive && t % slots == 0)) return s;
     s.ctas = (int)slots;
-    s.whole = (t / slots - 1) * slots;
+    // (a share's CTAs take whole tiles to the end where they come out even)
+    s.whole = t % slots == 0 ? t : (t / slots - 1) * slots;
     int steps = (P.Nt + 47) / 48;
     steps = (steps + TC - 1) / TC * TC;
     s.steps = steps;
@@ -1453,17 +1445,20 @@ static FusedShape fused_shape(const fmc_ctx* ctx, const Prepared& P)
         // runs the tiles left over in a second round; 1000 steps of 10 machines, 19500
         // to 32767 samples: 8.0 -> 4.7 ms)
         if (rule && rule->max_ctas > 0 && !wide) f.max_ctas = rule->max_ctas == 1 && need > 1 ? 2 : rule->max_ctas;
+    } else if (P.per_sm > 0) {
+        f.max_ctas = P.per_sm;
     } else if (full <= 2 * sms) {
-        // among other launches: room for two CTAs per SM, whatever a rule measured alone
-        // says.  With one, the launches run one after another once their tiles pass the
-        // SMs; with four, several launches' CTAs pile up on the same SMs.  Two, three and
-        // four launches of 79 tiles (9 machines, 1000 steps), by CTAs per SM 1, 2, 3, 4:
-        // 6.9, 5.1, 5.5, 6.1; 7.1, 5.6, 7.6, 9.2; 10.4, 8.4, 7.6, 10.0 ms
+        // among launches that no plan covers (the server's): room for two CTAs per SM,
+        // whatever a rule measured alone says.  With one, the launches run one after
+        // another once their tiles pass the SMs; with four, several launches' CTAs pile
+        // up on the same SMs.  Two, three and four launches of 79 tiles (9 machines, 1000
+        // steps), by CTAs per SM 1, 2, 3, 4: 6.9, 5.1, 5.5, 6.1; 7.1, 5.6, 7.6, 9.2;
+        // 10.4, 8.4, 7.6, 10.0 ms
         f.max_ctas = 2;
     } else if (rule && rule->max_ctas > 0 && !wide) {
         f.max_ctas = rule->max_ctas;
     }
-    const int sliced = slice_shape(ctx, P, 16).ctas;  // (TC does not enter the choice)
+    const int sliced = P.exclusive ? slice_shape(sms, ctx->budget != 0, P, 16).ctas : 0;  // (TC does not enter the choice)
     if (sliced > 0) f.max_ctas = sliced > 2 * sms ? 3 : 2;
     // a CTA's TMEM columns: the largest power of two within its share of the SM's
     // 512 (allocations are powers of two)
@@ -1528,7 +1523,7 @@ static int reserve(fmc_ctx* ctx, Workspace& ws, const Prepared& P, bool want_tra
     size_t zbytes = (size_t)count * d * Ks * 2;
     {
         const FusedShape f = fused_shape(ctx, P);
-        const SliceShape sl = slice_shape(ctx, P, f.TC);
+        const SliceShape sl = slice_shape(ctx->sms, ctx->budget != 0, P, f.TC);
         if (sl.ctas > 0 && (rc = ensure(ctx, ws.slices, slice_bytes(P, sl)))) return rc;
     }
     if (!em) {
@@ -1730,7 +1725,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
             keep.tiles = t >= (double)ntiles ? (int)ntiles : (int)t;
         }
         SlicePlan slices{};
-        const SliceShape sl = slice_shape(ctx, P, TC);
+        const SliceShape sl = slice_shape(ctx->sms, ctx->budget != 0, P, TC);
         if (sl.ctas > 0) {
             slices.ctas = sl.ctas;
             slices.whole = sl.whole;
@@ -2020,35 +2015,77 @@ static void batch_free(fmc_batch* b)
     delete b;
 }
 
-// The grids of a batch's per-sample launches, which run side by side two CTAs to an SM.
-// Together past that many tiles, the tiles left over would run a round of their own on a
-// nearly idle GPU, so every launch that can be sliced (slice_shape) gets a share of the
-// CTAs by its work: all are resident from the start and end together.  The work is
-// tiles x steps x n (n + 24), which fits 65536 samples of 4, 8, 12 and 16 machines to
-// 20 % (2.7, 5.1, 8.7 and 13.4 ms per 1000 steps).  Only where every scenario has a stream
-// of its own.  Measured (GB300, one CTA per SM and no shares -> two and shares): four arms
-// of 10007 samples, 9 machines, one of them smooth, 11.2 -> 7.3 ms; four of 20000 samples
-// of 10 machines 20.3 -> 9.6, of 40000 22.0 -> 19.4; twelve of 6000 16.5 -> 8.8.
-static void batch_shares(const fmc_ctx* ctx, std::vector<Prepared>& prep)
+constexpr int BATCH_STREAMS = 16;  // of a batch's launches at once
+
+// The grids of a batch's per-sample launches, which run side by side.  While all launches
+// together (teams and split-kernel CTAs an SM each) need no more than the SMs, one CTA to
+// an SM: room for two puts them in pairs on some SMs beside idle ones (four launches of
+// 4800 samples, 10 machines, 1000 steps: 4.4 ms, one by one 3.6).  Up to twice the SMs,
+// two.  Past that the tiles left over would run a round of their own on a nearly idle GPU,
+// so every launch that can be sliced (slice_shape) gets a share of the CTAs by its part of
+// all their work, the smooth launches' included: all are resident from the start and end
+// together.  A launch with fewer tiles than its share leaves the rest to the others.
+//
+// The work is tiles x steps x n (n + 24), which fits 65536 samples of 4, 8, 12 and 16
+// machines to 20 % (2.7, 5.1, 8.7 and 13.4 ms per 1000 steps); a smooth step is 1.4 of
+// another.  Three CTAs to an SM where each launch has the SMs' tiles (four launches of
+// 20000 samples of 10 machines: 9.1 ms with two, 8.3 with three; of 40000 18.1, 15.7), two
+// for smaller ones (twelve of 6000 8.6, 11.0) and beside a smooth launch, whose CTAs come
+// and go tile by tile (four arms of 20000 samples, 9 machines, one smooth, 14.7, 16.6).
+// Shares only where every scenario has a stream of its own and the context no memory
+// budget.  None where the last round is a small part of the whole anyway: from 6 SMs of tiles
+// on beside a smooth launch (arms of 38000 samples 24.9 -> 22.6, 4 machines, 32768 samples
+// 10.0 -> 9.2), and from 64 SMs of tiles on without.
+// Measured (GB300, 1000 steps, the launches by the rules for single ones, one CTA per SM
+// -> now): the four arms of 10007 samples 11.2 -> 7.3 ms, of 30000 27.7 -> 20, of 38000 27.6
+// -> 22.6; four launches of 10 machines, 20000 samples, 18.6 -> 8.3; twelve of 6000
+// 15.1 -> 8.6; two of 65536 14.1 -> 13.0.
+static void batch_shares(int sms, bool shares, std::vector<Prepared>& prep)
 {
-    int64_t slots = 2 * (int64_t)ctx->sms, all = 0;
-    double work = 0;
+    int64_t all = 0, need = 0, least = INT64_MAX;
+    bool smooth = false;
     auto tiles = [](const Prepared& P) { return (P.count + TC_M - 1) / TC_M; };
-    auto cost = [&](const Prepared& P) { return (double)tiles(P) * P.Nt * P.nm * (P.nm + 24.0); };
-    auto sliced = [](const Prepared& P) { return P.s.forcing != FMC_FORCING_SMOOTH; };
-    for (const Prepared& P : prep) {
-        if (P.path != FMC_PATH_FUSED || P.nmt > 0 || P.team) continue;
-        all += tiles(P);
-        if (sliced(P))
-            work += cost(P);
-        else
-            slots -= tiles(P);
-    }
-    if (all <= 2 * (int64_t)ctx->sms || slots <= 0 || ctx->budget != 0) return;
+    auto cost = [&](const Prepared& P) {
+        return (double)tiles(P) * P.Nt * P.nm * (P.nm + 24.0) * (P.s.forcing == FMC_FORCING_SMOOTH ? 1.4 : 1.0);
+    };
+    std::vector<Prepared*> left;
     for (Prepared& P : prep) {
-        if (P.path != FMC_PATH_FUSED || P.nmt > 0 || P.team || !sliced(P)) continue;
-        const int64_t share = (int64_t)((double)slots * (cost(P) / work));
-        P.share = (int)(share < 1 ? 1 : share);
+        if (P.path != FMC_PATH_FUSED) continue;
+        need += P.team ? (P.count + TEAM_GROUP - 1) / TEAM_GROUP : tiles(P);
+        if (P.team || P.nmt > 0) continue;
+        all += tiles(P);
+        least = tiles(P) < least ? tiles(P) : least;
+        smooth = smooth || P.s.forcing == FMC_FORCING_SMOOTH;
+        left.push_back(&P);
+    }
+    if (all > (smooth ? 6 : 64) * (int64_t)sms) {
+        if (smooth)
+            for (Prepared* P : left) P->per_sm = 2;
+        return;
+    }
+    const int per_sm = need <= sms ? 1 : (!smooth && least >= sms ? 3 : 2);
+    if (all > 2 * (int64_t)sms && !shares) return;
+    for (Prepared* P : left) P->per_sm = per_sm;
+    if (all <= 2 * (int64_t)sms) return;
+    int64_t slots = (int64_t)per_sm * sms;
+    // (shares are rounded down: twelve of 26 CTAs for 304 places ended 1.1 ms later than of 25)
+    for (bool again = true; again && !left.empty() && slots > 0;) {
+        double work = 0;
+        for (const Prepared* P : left) work += cost(*P);
+        again = false;
+        const int64_t now = slots;
+        std::vector<Prepared*> rest;
+        for (Prepared* P : left) {
+            const int64_t share = (int64_t)((double)now * (cost(*P) / work));
+            P->share = (int)(share < 1 ? 1 : share);
+            if (share >= tiles(*P)) {
+                slots -= tiles(*P);
+                again = true;
+            } else {
+                rest.push_back(P);
+            }
+        }
+        left.swap(rest);
     }
 }
 
@@ -2105,8 +2142,8 @@ int fmc_batch_create(fmc_ctx* ctx, const fmc_scenario* scen, int32_t n_scen, int
         b->mean.push_back(mean_dev[i]);
         b->var.push_back(var_dev[i]);
     }
-    const int nstreams = n_scen < 16 ? n_scen : 16;
-    if (rc == FMC_OK && nstreams == n_scen) batch_shares(ctx, b->prep);
+    const int nstreams = n_scen < BATCH_STREAMS ? n_scen : BATCH_STREAMS;
+    if (rc == FMC_OK) batch_shares(ctx->sms, nstreams == n_scen && ctx->budget == 0, b->prep);
     for (int i = 0; i < n_scen && rc == FMC_OK; ++i)
         rc = reserve(ctx, *b->ws[i], b->prep[i], false, path == FMC_PATH_PLAIN);
     for (int k = 0; k < nstreams && rc == FMC_OK; ++k) {
@@ -2375,6 +2412,38 @@ int fmc_diag_kernel_choice(const fmc_scenario* scen, int32_t path, int32_t polic
     out[2] = C.H;
     out[3] = C.nd;
     out[4] = C.bus ? 1 : 0;
+    return FMC_OK;
+}
+
+int fmc_diag_batch_plan(const fmc_scenario* scen, int32_t n_scen, int32_t path, int32_t sms, int32_t* out)
+{
+    if (!scen || !out || n_scen < 1 || sms < 1 || (path != FMC_PATH_FUSED && path != FMC_PATH_PLAIN)) return FMC_EINVAL;
+    std::vector<Prepared> prep(n_scen);
+    for (int32_t i = 0; i < n_scen; ++i) {
+        const fmc_scenario* s = &scen[i];
+        if (s->n < 1 || s->n > FMC_MAX_MACHINES || s->d < 1 || s->d > 8 || s->N < 1 || !(s->dt > 0.0) || !(s->T > 0.0))
+            return FMC_EINVAL;
+        KernelChoice C;
+        const int rc = choose_kernel(nullptr, nullptr, s, s->N, path, FMC_KERNEL_AUTO, C);
+        if (rc) return rc;
+        Prepared& P = prep[i];
+        P.s = *s;
+        P.Nt = (int)std::llround(s->T / s->dt);
+        P.nm = C.nm;
+        P.nmt = C.nmt;
+        P.H = C.H;
+        P.path = path;
+        P.count = s->N;
+        P.exclusive = false;
+        P.team = team_fits(sms, P.nm, P.nmt, path, s->n, P.Nt, P.count);
+    }
+    batch_shares(sms, n_scen <= BATCH_STREAMS, prep);
+    for (int32_t i = 0; i < n_scen; ++i) {
+        const Prepared& P = prep[i];
+        out[3 * i] = P.team ? 1 : 0;
+        out[3 * i + 1] = P.team || P.nmt > 0 ? 0 : P.per_sm;
+        out[3 * i + 2] = P.path == FMC_PATH_FUSED ? slice_shape(sms, false, P, 16).ctas : 0;
+    }
     return FMC_OK;
 }
 

@@ -1,0 +1,82 @@
+"""How a batch's launches share the GPU (host logic, no GPU; 152 SMs): the CTAs that each
+per-sample launch's tiles are dealt to, and the resident CTAs per SM."""
+import math
+
+import pytest
+
+import fmc_synth as fs
+
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def fmc():
+    import paper_2007_03847_gb300 as m
+    m.build()
+    return m
+
+
+def _sc(n, N, Nt=1000, d=2, **kw):
+    return fs.multimachine_case(n=n, d=d, K=20, T=Nt * 0.005, dt=0.005, N=N, seed=n).replace(**kw)
+
+
+def _arms(n, N):
+    return [_sc(n, N), _sc(n, N, sampling=fs.SRS), _sc(n, N, sampling=fs.SRS_EM), _sc(n, N, forcing=fs.FORCING_SMOOTH)]
+
+
+@pytest.mark.parametrize("N", [10007, 16000, 20000, 24000, 28000])
+def test_a_smooth_arm_takes_its_part_only(fmc, N):
+    # its tiles are no CTAs of the others': each arm keeps its part of the 304 by its work
+    tiles = math.ceil(N / 128)
+    plan = fmc.batch_plan(_arms(9, N), sms=SMS)
+    assert [p["per_sm"] for p in plan] == [2] * 4
+    assert plan[3]["ctas"] == 0  # one CTA per tile
+    part = 2 * SMS / 4.4  # the smooth arm's work is 1.4 of another's
+    for p in plan[:3]:
+        assert int(part) <= p["ctas"] <= min(tiles, math.ceil(2 * SMS - min(tiles, 1.4 * part)) / 3 + 1)
+
+
+@pytest.mark.parametrize("N", [31000, 38000, 100000])
+def test_large_arms_beside_a_smooth_one_keep_a_cta_per_tile(fmc, N):
+    plan = fmc.batch_plan(_arms(9, N), sms=SMS)
+    assert all(p["ctas"] == 0 and p["per_sm"] == 2 for p in plan)
+
+
+def test_equal_launches_get_equal_shares(fmc):
+    # an SM's tiles each: three CTAs per SM; fewer: two
+    assert fmc.batch_plan([_sc(10, 20000)] * 4, sms=SMS) == [{"team": False, "per_sm": 3, "ctas": 3 * SMS // 4}] * 4
+    plan = fmc.batch_plan([_sc(10, 6000)] * 12, sms=SMS)
+    assert plan == [{"team": False, "per_sm": 2, "ctas": 2 * SMS // 12}] * 12
+
+
+def test_a_share_may_divide_the_tiles(fmc):
+    # 304 tiles on 152 CTAs, and a launch so small beside the other that one CTA is its part:
+    # dealt out all the same, not a CTA per tile
+    plan = fmc.batch_plan([_sc(10, 304 * 128)] * 3, sms=SMS)
+    assert [p["ctas"] for p in plan] == [SMS] * 3
+    plan = fmc.batch_plan([_sc(16, 200000, Nt=4000), _sc(1, 6000, Nt=40, d=1)], sms=SMS)
+    assert plan[1]["ctas"] == 1
+
+
+def test_fewer_tiles_than_a_share(fmc):
+    # the small launch runs all its tiles at once, the others share what it leaves
+    plan = fmc.batch_plan([_sc(10, 6000, Nt=4000), _sc(10, 20000, Nt=500), _sc(10, 20000, Nt=500)], sms=SMS)
+    assert plan[0]["ctas"] == 0 and plan[0]["per_sm"] == 2
+    assert plan[1]["ctas"] == plan[2]["ctas"] == (2 * SMS - 47) // 2
+
+
+def test_few_tiles_take_an_sm_each(fmc):
+    # 4 x 38 tiles fit the SMs; 5 x 38 take two CTAs per SM
+    assert [p["per_sm"] for p in fmc.batch_plan([_sc(10, 4864 + 1)] * 3, sms=SMS)] == [1] * 3
+    assert [p["per_sm"] for p in fmc.batch_plan([_sc(10, 4864 + 1)] * 5, sms=SMS)] == [2] * 5
+    # a split kernel's CTAs count
+    assert [p["per_sm"] for p in fmc.batch_plan([_sc(10, 9000), _sc(30, 12000)], sms=SMS)] == [2, 0]
+    # and many launches share, whatever their streams
+    plan = fmc.batch_plan([_sc(10, 6000)] * 18, sms=SMS)
+    assert all(p["ctas"] == 0 for p in plan)
+
+
+def test_no_refusal_is_lost(fmc):
+    with pytest.raises(fmc.FastMCError):
+        fmc.batch_plan([_sc(20, 100, forcing=fs.FORCING_SMOOTH)])
+    assert fmc.batch_plan([_sc(5, 100)], path="plain")[0]["ctas"] == 0
