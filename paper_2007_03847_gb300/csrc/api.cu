@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1268,8 +1269,8 @@ static size_t team_part_bytes(int n, int Nt, int64_t count)
 // 10 machines, 3 disturbances: 1000 samples 3.44 -> 1.96 ms; 4000 samples, 2 disturbances:
 // 1 machine 0.99 -> 0.75, 4 machines 1.36 -> 1.10, 8 machines 2.10 -> 1.48, 12 machines
 // 4.1 -> 1.8, 13 machines (slots of 16) 8.5 -> 3.6, 16 machines 7.4 -> 2.9.  Above the
-// line it loses (10 machines, 9728 samples: 3.68 -> 4.17).  The same line where other
-// launches share the GPU (four arms of 10007 samples at once: 10.6 ms, by teams 19.5).
+// line it loses (10 machines, 9728 samples: 3.68 -> 4.17).  In a batch, whose launches
+// share the SMs, batch_teams decides among the launches below the line.
 // Its partials are four times the per-sample kernel's: not past 512 MiB, and not in a
 // context with a memory budget.
 static constexpr size_t TEAM_PART_MAX = (size_t)512 << 20;
@@ -2017,6 +2018,73 @@ static void batch_free(fmc_batch* b)
 
 constexpr int BATCH_STREAMS = 16;  // of a batch's launches at once
 
+// Which launches of a batch take the team kernel, of those that would alone (P.team).  A
+// team halves the chain of its launch's steps but costs three times the SM time per
+// sample, so it pays while the SMs have room for it and its launch is what the batch waits
+// for.  The launches with the longest chains take it, as many of them as shorten the
+// batch's estimated time: the longest chain of a stream, the SM time of all launches over
+// the SMs, or the rounds of the teams.  Step times (us, GB300, fits of the measured
+// ones): per-sample 0.65 + 0.022 nm^2 alone, and 0.68 of that as SM time where two CTAs
+// share an SM; teams 0.45 + 0.075 nm, a fifth more where two share an SM and three
+// quarters more with 16 slots; split kernel 3 + 0.3 n.  Two teams of up to 8 machines fit an SM, but launches of more than two
+// thirds of the SMs were seen to wait for one another all the same (two of 4400 samples and
+// more, 8 machines: 2.9 ms or 1.7), so those count an SM per team.
+// Measured (GB300, 1000 steps, teams by each launch alone -> now; in brackets without
+// teams, by the rules for single launches): 10 machines, four launches of 4800 samples
+// 6.17 -> 3.03 ms (3.60), sixteen of 1000 6.06 -> 3.15 (3.48), eight of 1000 3.05 -> 3.04
+// (3.20); 8 machines, four of 4800 4.44 -> 2.15 (2.74), four of 2400 1.71 either way
+// (2.34); 4 machines, eight of 2400 2.25 -> 1.38 (1.78); 12 machines, eight of 4800
+// 12.7 -> 6.5 (11.8).
+static void batch_teams(int sms, int nstreams, std::vector<Prepared>& prep)
+{
+    const size_t n = prep.size();
+    auto tiles = [](const Prepared& P) { return (double)((P.count + TC_M - 1) / TC_M); };
+    auto chain = [](const Prepared& P) {
+        return P.Nt * (P.nmt > 0 ? 3.0 + 0.3 * P.s.n : 0.65 + 0.022 * P.nm * P.nm);
+    };
+    auto team_chain = [](const Prepared& P) {
+        return P.Nt * (0.45 + 0.075 * P.nm) * (P.nm > 12 ? 1.75 : P.nm > 8 ? 1.0 : 1.2);
+    };
+    auto room = [&](const Prepared& P) {  // SMs of its groups
+        const double g = (double)((P.count + TEAM_GROUP - 1) / TEAM_GROUP);
+        return P.nm > 8 || 3 * g > 2 * sms ? g : 0.5 * g;
+    };
+    std::vector<size_t> order;
+    for (size_t i = 0; i < n; ++i)
+        if (prep[i].team) order.push_back(i);
+    if (order.empty()) return;
+    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return chain(prep[a]) > chain(prep[b]); });
+    std::vector<char> team(n, 0);
+    double best = 0;
+    size_t take = 0;
+    for (size_t k = 0; k <= order.size(); ++k) {
+        if (k > 0) team[order[k - 1]] = 1;
+        double area = 0, teams = 0, round = 0, longest = 0;
+        std::vector<double> stream((size_t)nstreams, 0.0);
+        for (size_t i = 0; i < n; ++i) {
+            const Prepared& P = prep[i];
+            double c = chain(P);
+            if (team[i]) {
+                c = team_chain(P);
+                teams += room(P);
+                round = c > round ? c : round;
+                area += room(P) * c;
+            } else {
+                area += tiles(P) * c * (P.nmt > 0 ? (P.H == 2 ? 0.6 : 1.0) : 0.68);
+            }
+            stream[i % (size_t)nstreams] += c;
+        }
+        for (double c : stream) longest = c > longest ? c : longest;
+        double t = area / sms > longest ? area / sms : longest;
+        if (std::ceil(teams / sms) * round > t) t = std::ceil(teams / sms) * round;
+        if (k == 0 || t < 0.98 * best) {
+            best = t;
+            take = k;
+        }
+    }
+    for (size_t k = take; k < order.size(); ++k) prep[order[k]].team = false;
+}
+
 // The grids of a batch's per-sample launches, which run side by side.  While all launches
 // together (teams and split-kernel CTAs an SM each) need no more than the SMs, one CTA to
 // an SM: room for two puts them in pairs on some SMs beside idle ones (four launches of
@@ -2143,6 +2211,7 @@ int fmc_batch_create(fmc_ctx* ctx, const fmc_scenario* scen, int32_t n_scen, int
         b->var.push_back(var_dev[i]);
     }
     const int nstreams = n_scen < BATCH_STREAMS ? n_scen : BATCH_STREAMS;
+    if (rc == FMC_OK) batch_teams(ctx->sms, nstreams, b->prep);
     if (rc == FMC_OK) batch_shares(ctx->sms, nstreams == n_scen && ctx->budget == 0, b->prep);
     for (int i = 0; i < n_scen && rc == FMC_OK; ++i)
         rc = reserve(ctx, *b->ws[i], b->prep[i], false, path == FMC_PATH_PLAIN);
@@ -2437,6 +2506,7 @@ int fmc_diag_batch_plan(const fmc_scenario* scen, int32_t n_scen, int32_t path, 
         P.exclusive = false;
         P.team = team_fits(sms, P.nm, P.nmt, path, s->n, P.Nt, P.count);
     }
+    batch_teams(sms, n_scen < BATCH_STREAMS ? n_scen : BATCH_STREAMS, prep);
     batch_shares(sms, n_scen <= BATCH_STREAMS, prep);
     for (int32_t i = 0; i < n_scen; ++i) {
         const Prepared& P = prep[i];

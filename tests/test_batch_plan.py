@@ -80,3 +80,34 @@ def test_no_refusal_is_lost(fmc):
     with pytest.raises(fmc.FastMCError):
         fmc.batch_plan([_sc(20, 100, forcing=fs.FORCING_SMOOTH)])
     assert fmc.batch_plan([_sc(5, 100)], path="plain")[0]["ctas"] == 0
+
+
+def _teams(fmc, scs):
+    return [p["team"] for p in fmc.batch_plan(scs, sms=SMS)]
+
+
+@pytest.mark.parametrize("n,N,count,team", [
+    (10, 1000, 1, True), (10, 4864, 1, True), (10, 4865, 1, False),
+    (10, 2400, 2, True),      # 150 groups: an SM each
+    (10, 1000, 8, True),      # two rounds of teams are still shorter than one of tiles
+    (10, 1000, 16, False), (10, 4800, 4, False), (12, 4800, 8, False), (16, 4800, 16, False),
+    (8, 1000, 8, True), (8, 2400, 4, True),   # two teams to an SM
+    (8, 4800, 2, False), (8, 2400, 8, False), (4, 2400, 8, False), (1, 4800, 16, False)])
+def test_teams_while_the_batch_has_room(fmc, n, N, count, team):
+    assert _teams(fmc, [_sc(n, N, d=1)] * count) == [team] * count
+
+
+def test_the_launch_that_the_batch_waits_for(fmc):
+    # a long horizon beside short ones; not beside a split kernel's longer chain, nor where
+    # the SMs are full for longer than its chain
+    assert _teams(fmc, [_sc(10, 1000, Nt=4000)] + [_sc(10, 4800)] * 4) == [True] + [False] * 4
+    assert _teams(fmc, [_sc(10, 1000), _sc(50, 1000)]) == [False, False]
+    assert _teams(fmc, [_sc(10, 1000), _sc(10, 60000)]) == [False, False]
+    # launches of a stream follow one another
+    assert sum(_teams(fmc, [_sc(10, 100)] * 33)) > 0
+
+
+def test_what_is_no_team_alone_is_none_in_a_batch(fmc):
+    # (four groups' partials, 240 bytes a time: past 512 MiB from 559241 steps on)
+    assert _teams(fmc, [_sc(20, 100), _sc(10, 100, Nt=560000)]) == [False, False]
+    assert [p["team"] for p in fmc.batch_plan([_sc(5, 100)], path="plain")] == [False]

@@ -43,3 +43,35 @@ def test_planned_batches(shapes):
     b.close()
     ctx.close()
     alone.close()
+
+
+@pytest.mark.parametrize("shapes,teams", [
+    ([(10, 3, 1000, 400), (10, 3, 4800, 60), (9, 2, 4800, 60), (10, 1, 4500, 60), (10, 2, 4800, 60)], 1),
+    ([(10, 2, 1000, 100)] * 8, 8), ([(10, 2, 700, 100)] * 17, 17), ([(8, 2, 4800, 70), (8, 1, 4700, 70)], 0),
+    ([(4, 1, 4800, 90), (2, 1, 33, 900), (12, 3, 2000, 90)], 1)])
+@pytest.mark.parametrize("use_graph", [False, True])
+def test_batches_with_teams(shapes, teams, use_graph):
+    import torch
+    fmc = need_gpu()
+    ctx, alone = fmc.Context(0), fmc.Context(0, mem_budget_bytes=64 << 30)  # (no teams with a budget)
+    fmc.set_launch_rules([], ctx=ctx)
+    fmc.set_launch_rules([], ctx=alone)
+    scs = [fs.multimachine_case(n=n, d=d, K=24, T=Nt * 0.005, dt=0.005, N=N, seed=n + k)
+           for k, (n, d, N, Nt) in enumerate(shapes)]
+    if ctx.info()[0] == 152:
+        assert sum(p["team"] for p in fmc.batch_plan(scs)) == teams
+    b = fmc.Batch(scs, use_graph=use_graph, ctx=ctx)
+    for _ in range(2):
+        b.launch()
+        fmc.device_status(ctx=ctx)
+    for i, sc in enumerate(scs):
+        a = fmc.Batch([sc], use_graph=False, ctx=alone)
+        a.launch()
+        torch.cuda.synchronize()
+        for x, y in ((b.mean[i], a.mean[0]), (b.var[i], a.var[0])):
+            x, y = x.cpu().numpy(), y.cpu().numpy()
+            assert np.max(np.abs(x - y)) <= 1e-9 * np.max(np.abs(y))
+        a.close()
+    b.close()
+    ctx.close()
+    alone.close()
