@@ -1281,6 +1281,15 @@ static bool team_fits(int sms, int nm, int nmt, int32_t path, int n, int Nt, int
     return count <= (int64_t)sms * TEAM_GROUP && team_part_bytes(n, Nt, count) <= TEAM_PART_MAX;
 }
 
+// Half SMs that a launch's teams hold.  Two teams of up to 8 machines fit an SM, but with
+// 8 slots launches of more than two thirds of the SMs were seen to wait for one another
+// all the same (two of 4400 samples and more: 2.9 ms or 1.7), so those count an SM per team.
+static int64_t team_halves(int sms, int nm, int64_t count)
+{
+    const int64_t g = (count + TEAM_GROUP - 1) / TEAM_GROUP;
+    return nm > 8 || (nm > 4 && 3 * g > 2 * (int64_t)sms) ? 2 * g : g;
+}
+
 static bool team_wanted(const fmc_ctx* ctx, int nm, int nmt, int32_t path, int n, int Nt, int64_t count,
                         bool exclusive)
 {
@@ -1840,6 +1849,20 @@ size_t fmc::team_bytes(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, 
     return team_fits(ctx->sms, nm, 0, path, s->n, Nt, count) ? grown(team_part_bytes(s->n, Nt, count)) : 0;
 }
 
+int64_t fmc::team_room(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count)
+{
+    const int Nt = (int)std::llround(s->T / s->dt);
+    const int nm = nm_bucket_for(s->n);
+    return team_fits(ctx->sms, nm, 0, path, s->n, Nt, count) ? team_halves(ctx->sms, nm, count) : 0;
+}
+
+// Two rounds of the SMs: eight slots with requests of 10 machines, 4800 samples, 1000 steps,
+// sixteen in all, 24.7 ms without a bound, 16.1 with three rounds, 13.8 with two, 11.6 with
+// one (19.2 before there were teams); sixteen slots with requests of 1000 samples, 32 in
+// all, 11.5, 12.3, 14.8, 17.4 (33.3); five requests of 4 to 15 machines 9.9, 9.9, 10.0,
+// 14.6 (21.3).
+int64_t fmc::team_room_total(const fmc_ctx* ctx) { return 4 * (int64_t)ctx->sms; }
+
 size_t fmc::table_bytes(const fmc_scenario* s)
 {
     if (s->sampling == FMC_SRS_EM) return 0;
@@ -2026,9 +2049,8 @@ constexpr int BATCH_STREAMS = 16;  // of a batch's launches at once
 // the SMs, or the rounds of the teams.  Step times (us, GB300, fits of the measured
 // ones): per-sample 0.65 + 0.022 nm^2 alone, and 0.68 of that as SM time where two CTAs
 // share an SM; teams 0.45 + 0.075 nm, a fifth more where two share an SM and three
-// quarters more with 16 slots; split kernel 3 + 0.3 n.  Two teams of up to 8 machines fit an SM, but launches of more than two
-// thirds of the SMs were seen to wait for one another all the same (two of 4400 samples and
-// more, 8 machines: 2.9 ms or 1.7), so those count an SM per team.
+// quarters more with 16 slots; split kernel 3 + 0.3 n.  The
+// SMs that teams hold: team_halves.
 // Measured (GB300, 1000 steps, teams by each launch alone -> now; in brackets without
 // teams, by the rules for single launches): 10 machines, four launches of 4800 samples
 // 6.17 -> 3.03 ms (3.60), sixteen of 1000 6.06 -> 3.15 (3.48), eight of 1000 3.05 -> 3.04
@@ -2045,10 +2067,7 @@ static void batch_teams(int sms, int nstreams, std::vector<Prepared>& prep)
     auto team_chain = [](const Prepared& P) {
         return P.Nt * (0.45 + 0.075 * P.nm) * (P.nm > 12 ? 1.75 : P.nm > 8 ? 1.0 : 1.2);
     };
-    auto room = [&](const Prepared& P) {  // SMs of its groups
-        const double g = (double)((P.count + TEAM_GROUP - 1) / TEAM_GROUP);
-        return P.nm > 8 || 3 * g > 2 * sms ? g : 0.5 * g;
-    };
+    auto room = [&](const Prepared& P) { return 0.5 * (double)team_halves(sms, P.nm, P.count); };
     std::vector<size_t> order;
     for (size_t i = 0; i < n; ++i)
         if (prep[i].team) order.push_back(i);

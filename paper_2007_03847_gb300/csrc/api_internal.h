@@ -74,6 +74,10 @@ int reserve_workspace(fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t
 // (the results are the same without).
 size_t team_bytes(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count);
 size_t table_bytes(const fmc_scenario* s);
+// Half SMs that such a launch's teams hold (0: no teams), and the bound for all that run
+// at once.
+int64_t team_room(const fmc_ctx* ctx, const fmc_scenario* s, int32_t path, int64_t count);
+int64_t team_room_total(const fmc_ctx* ctx);
 void set_extras(fmc_ctx* ctx, bool team, bool table);
 
 // fmc_simulate with a choice of how the fused kernel combines its per-time sums:

@@ -34,6 +34,8 @@ struct Request {
     size_t bytes = 0;  // device memory charged against the budget
     bool team = true;   // the team kernel's partials are part of the charge
     bool table = true;  // the basis kernels' cosine table is
+    int64_t room = 0;   // half SMs that its teams hold at most
+    bool teams = false;  // it runs them
     int status = FMC_NOT_READY;
     bool started = false;
     std::string error;
@@ -226,6 +228,8 @@ struct fmc_server {
     int device = 0;
     size_t budget = 0;
     size_t in_use = 0;
+    int64_t room = 0;       // half SMs that teams may hold (team_room_total),
+    int64_t room_used = 0;  // and those of the running requests
     bool stopping = false;
     uint64_t next_id = 1;
     std::mutex mu;
@@ -262,12 +266,16 @@ static void worker_loop(fmc_server* srv, int slot)
             r = srv->reqs[srv->queue.front()].get();
             srv->queue.pop_front();
             srv->in_use += r->bytes;
+            // teams while those of the running requests stay within team_room_total: past
+            // it their SM time, three times the per-sample kernel's, makes all wait
+            r->teams = r->team && r->room > 0 && srv->room_used + r->room <= srv->room;
+            if (r->teams) srv->room_used += r->room;
             r->started = true;
             r->t_start = Clock::now();
         }
         // moments summed with FP64 atomics (no per-tile partial buffers to hold), or
         // by the team kernel where its partials were charged
-        for (int k = 0; k < kReplicates; ++k) fmc::set_extras(rctx[k], r->team, r->table);
+        for (int k = 0; k < kReplicates; ++k) fmc::set_extras(rctx[k], r->teams, r->table);
         int rc;
         if (r->tol_E > 0 || r->tol_Var > 0) {
             rc = run_target(rctx, rst, r);
@@ -291,6 +299,7 @@ static void worker_loop(fmc_server* srv, int slot)
             if (rc != FMC_OK && r->error.empty()) r->error = fmc_last_error(ctx);
             r->t_done = Clock::now();
             srv->in_use -= r->bytes;
+            if (r->teams) srv->room_used -= r->room;
         }
         srv->cv_done.notify_all();
         srv->cv_work.notify_all();
@@ -335,6 +344,7 @@ int fmc_server_create(int device, int32_t slots, size_t mem_budget_bytes, fmc_se
         fmc::set_stream_ordered(c, true);  // each is used on its worker's replicate stream only
         srv->ctxs.push_back(c);
     }
+    srv->room = fmc::team_room_total(srv->ctxs[0]);
     for (int i = 0; i < slots; ++i) srv->workers.emplace_back(worker_loop, srv, i);
     *out = srv;
     return FMC_OK;
@@ -402,6 +412,10 @@ static int submit_request(fmc_server* srv, const fmc_scenario* scen, int32_t pat
                          : n <= n_mm ? fmc::team_bytes(srv->ctxs[0], scen, path, kReplicates * n)
                                      : kReplicates * fmc::team_bytes(srv->ctxs[0], scen, path, n);
         team = t > team ? t : team;
+        const int64_t m = !target     ? fmc::team_room(srv->ctxs[0], scen, path, n)
+                          : n <= n_mm ? fmc::team_room(srv->ctxs[0], scen, path, kReplicates * n)
+                                      : kReplicates * fmc::team_room(srv->ctxs[0], scen, path, n);
+        r->room = m > r->room ? m : r->room;
         if (!target) break;
     }
     r->team = r->bytes + team <= srv->budget;

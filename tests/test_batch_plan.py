@@ -92,7 +92,7 @@ def _teams(fmc, scs):
     (10, 1000, 8, True),      # two rounds of teams are still shorter than one of tiles
     (10, 1000, 16, False), (10, 4800, 4, False), (12, 4800, 8, False), (16, 4800, 16, False),
     (8, 1000, 8, True), (8, 2400, 4, True),   # two teams to an SM
-    (8, 4800, 2, False), (8, 2400, 8, False), (4, 2400, 8, False), (1, 4800, 16, False)])
+    (8, 4800, 2, False), (4, 4800, 2, True), (8, 2400, 8, False), (4, 2400, 8, False), (1, 4800, 16, False)])
 def test_teams_while_the_batch_has_room(fmc, n, N, count, team):
     assert _teams(fmc, [_sc(n, N, d=1)] * count) == [team] * count
 
