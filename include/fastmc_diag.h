@@ -87,6 +87,18 @@ int fmc_diag_kernel_choice(const fmc_scenario* scen, int32_t path, int32_t polic
  */
 int fmc_diag_batch_plan(const fmc_scenario* scen, int32_t n_scen, int32_t path, int32_t sms, int32_t* out);
 
+/*
+ * The form of the context's last simulation (FMC_FORM_*; NONE for the plain path; of a
+ * batch the last scenario, as it was enqueued or captured) and the CTAs of its grid.
+ */
+#define FMC_FORM_NONE 0
+#define FMC_FORM_PER_SAMPLE 1 /* one CTA per 128 samples */
+#define FMC_FORM_SLICED 2     /* the same tiles dealt to a fixed grid */
+#define FMC_FORM_TEAM 3       /* one CTA per 32 samples, a warp per machine */
+#define FMC_FORM_SPLIT 4
+#define FMC_FORM_SPLIT_TC 5
+int fmc_diag_last_form(const fmc_ctx* ctx, int32_t* form, int64_t* ctas);
+
 /* CTAs per SM the last fused launch could keep resident (occupancy API). */
 int fmc_last_fused_occupancy(const fmc_ctx* ctx, int* ctas_per_sm);
 

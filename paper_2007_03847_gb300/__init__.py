@@ -16,7 +16,8 @@ Entry points (same names as the C ABI without the ``fmc_`` prefix):
 (``set_kernel_policy``: "auto", "per_sample", "split", "split_tc";
 ``set_launch_rules``) and the diagnostics of ``include/fastmc_diag.h``
 (``profile``/``profile_read``, ``check_wait_path``, ``kernel_choice``,
-``batch_plan``, ``net_matrix``).
+``batch_plan``, ``last_form``,
+``fused_occupancy``, ``net_matrix``).
 """
 from __future__ import annotations
 
@@ -124,6 +125,7 @@ def load_library():
             "fmc_profile_read": ([vp, i32, ctypes.POINTER(dbl), ctypes.POINTER(i64)], ctypes.c_int),
             "fmc_last_fused_occupancy": ([vp, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
             "fmc_diag_net_matrix": ([vp, i32, i32, vp, i64], ctypes.c_int),
+            "fmc_diag_last_form": ([vp, ctypes.POINTER(i32), ctypes.POINTER(i64)], ctypes.c_int),
             "fmc_diag_batch_plan": ([vp, i32, i32, i32, vp], ctypes.c_int),
             "fmc_diag_kernel_choice": ([vp, i32, i32, i64, vp], ctypes.c_int),
             "fmc_set_kernel_policy": ([vp, ctypes.c_int32], ctypes.c_int),
@@ -727,6 +729,15 @@ def set_kernel_policy(policy, ctx: Context | None = None) -> None:
     "split_tc"."""
     ctx = ctx or default_context()
     ctx.check(ctx.lib.fmc_set_kernel_policy(ctx.h, _KERNEL.get(policy, policy)))
+
+
+def last_form(ctx: Context | None = None):
+    """fmc_diag_last_form: (form, CTAs) of the context's last simulation, the form as "none",
+    "per_sample", "sliced", "team", "split" or "split_tc"."""
+    ctx = ctx or default_context()
+    form, ctas = ctypes.c_int32(), ctypes.c_int64()
+    ctx.check(ctx.lib.fmc_diag_last_form(ctx.h, ctypes.byref(form), ctypes.byref(ctas)))
+    return ("none", "per_sample", "sliced", "team", "split", "split_tc")[form.value], ctas.value
 
 
 def fused_occupancy(ctx: Context | None = None) -> int:

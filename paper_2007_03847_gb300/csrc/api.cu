@@ -83,6 +83,8 @@ struct fmc_ctx {
     std::vector<ProfRec> recs;
     size_t prof_cap = 0;
     int last_fused_ctas_per_sm = 0;
+    int last_form = FMC_FORM_NONE;  // of the last simulation enqueued, and its grid
+    int64_t last_ctas = 0;
     int kernel_policy = FMC_KERNEL_AUTO;
     // (the server: where a request was charged for them)
     bool team = true;   // the team kernel may be taken
@@ -1574,6 +1576,8 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
     double* trig = trig_if_ready(ws, K, Nt, s->basis, s->forcing == FMC_FORCING_SMOOTH);
     EmSpec ems{em ? 1 : 0, (uint32_t)s->seed, (uint32_t)(s->seed >> 32), k0, (float)std::sqrt(s->dt)};
 
+    ctx->last_form = FMC_FORM_NONE;
+    ctx->last_ctas = 0;
     // this call's error word (fmc_device_status), on both paths
     FMC_CUDA(ctx, cudaMemsetAsync((char*)ws.status.ptr + 4, 0, 4, st), "memset");
     if (P.path == FMC_PATH_PLAIN) {
@@ -1723,7 +1727,7 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
         }
     } else if (P.team) {
         e = launch_simulate_team(P.nm, P.nd, P.params.data(), maps, count, Nt, TC, d, Ks, nkb, split, tmem_cols,
-                                 (float*)ws.part.ptr, traj_dev, (int*)ws.status.ptr + 1, ems, rrf, smooth ? 1 : 0, st);
+                                 (float*)ws.part.ptr, traj_dev, (int*)ws.status.ptr + 1, ems, rrf, smooth ? 1 : 0, st, &occ);
     } else {
         // a launch that has the GPU to itself keeps as many design tiles in L2 as
         // 60 % of it holds: every chunk re-reads each tile, and the whole design
@@ -1749,6 +1753,11 @@ static int enqueue(fmc_ctx* ctx, Workspace& ws, const Prepared& P, double* S1, d
                                   (int*)ws.status.ptr + 1, ems, rrf, keep, smooth ? 1 : 0, slices, st, &occ);
     }
     ctx->last_fused_ctas_per_sm = occ;
+    const int sliced = slice_shape(ctx->sms, ctx->budget != 0, P, TC).ctas;
+    ctx->last_form = P.nmt > 0 ? (P.tcn ? FMC_FORM_SPLIT_TC : FMC_FORM_SPLIT)
+                     : P.team  ? FMC_FORM_TEAM
+                     : sliced > 0 ? FMC_FORM_SLICED : FMC_FORM_PER_SAMPLE;
+    ctx->last_ctas = sliced > 0 ? sliced : ntiles;
     if (e == cudaErrorInvalidConfiguration)
         return fail(ctx, FMC_EUNSUPPORTED, "fused kernel: %d CTAs per SM x %u TMEM columns exceeds 512", occ,
                     tmem_cols);
@@ -2470,6 +2479,14 @@ int fmc_last_fused_occupancy(const fmc_ctx* ctx, int* ctas_per_sm)
 {
     if (!ctx || !ctas_per_sm) return FMC_EINVAL;
     *ctas_per_sm = ctx->last_fused_ctas_per_sm;
+    return FMC_OK;
+}
+
+int fmc_diag_last_form(const fmc_ctx* ctx, int32_t* form, int64_t* ctas)
+{
+    if (!ctx || !form || !ctas) return FMC_EINVAL;
+    *form = ctx->last_form;
+    *ctas = ctx->last_ctas;
     return FMC_OK;
 }
 

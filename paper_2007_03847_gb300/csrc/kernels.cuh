@@ -102,7 +102,7 @@ constexpr int TEAM_GROUP = 32, TEAM_MAX_NM = 16;
 cudaError_t launch_simulate_team(int nm_bucket, int nd_bucket, const void* params, const CUtensorMap* maps,
                                  int64_t count, int Nt, int TC, int d, int Ks, int nkb, int split, uint32_t tmem_cols,
                                  float* part, float* traj, int* err, const EmSpec& em, double* rrf, int smooth,
-                                 cudaStream_t st);
+                                 cudaStream_t st, int* max_ctas_per_sm);
 cudaError_t launch_moments(const float* x, int64_t N, int64_t C, double* mean, double* var, int sms, cudaStream_t st);
 cudaError_t launch_traj_sums(const float* x, int64_t N, int64_t C, const double* shift, int S, double* S1, double* S2,
                              int sms, cudaStream_t st);

@@ -4,13 +4,13 @@
 namespace fmc {
 
 cudaError_t launch_team_nm12(int nd, const void* params, const CUtensorMap* maps, const TeamArgs& a, int smooth,
-                            cudaStream_t st)
+                            cudaStream_t st, int* max_ctas_per_sm)
 {
     switch (nd) {
-        case 1: return launch_team_t<12, 1>(params, maps, a, smooth, st);
-        case 2: return launch_team_t<12, 2>(params, maps, a, smooth, st);
-        case 4: return launch_team_t<12, 4>(params, maps, a, smooth, st);
-        case 8: return launch_team_t<12, 8>(params, maps, a, smooth, st);
+        case 1: return launch_team_t<12, 1>(params, maps, a, smooth, st, max_ctas_per_sm);
+        case 2: return launch_team_t<12, 2>(params, maps, a, smooth, st, max_ctas_per_sm);
+        case 4: return launch_team_t<12, 4>(params, maps, a, smooth, st, max_ctas_per_sm);
+        case 8: return launch_team_t<12, 8>(params, maps, a, smooth, st, max_ctas_per_sm);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -31,13 +31,13 @@ cudaError_t launch_wide_nmt7(int, const CUtensorMap*, const WideArgs&, cudaStrea
 cudaError_t launch_wide_nmt10(int, const CUtensorMap*, const WideArgs&, cudaStream_t, int*);
 cudaError_t launch_wide_nmt13(int, const CUtensorMap*, const WideArgs&, cudaStream_t, int*);
 
-cudaError_t launch_team_nm1(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
-cudaError_t launch_team_nm2(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
-cudaError_t launch_team_nm4(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
-cudaError_t launch_team_nm8(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
-cudaError_t launch_team_nm10(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
-cudaError_t launch_team_nm12(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
-cudaError_t launch_team_nm16(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t);
+cudaError_t launch_team_nm1(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
+cudaError_t launch_team_nm2(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
+cudaError_t launch_team_nm4(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
+cudaError_t launch_team_nm8(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
+cudaError_t launch_team_nm10(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
+cudaError_t launch_team_nm12(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
+cudaError_t launch_team_nm16(int, const void*, const CUtensorMap*, const TeamArgs&, int, cudaStream_t, int*);
 
 int wide_nmt_for(int n)
 {
@@ -149,17 +149,17 @@ cudaError_t launch_simulate_plain(int nm_bucket, int nd_bucket, const void* para
 cudaError_t launch_simulate_team(int nm_bucket, int nd_bucket, const void* params, const CUtensorMap* maps,
                                  int64_t count, int Nt, int TC, int d, int Ks, int nkb, int split, uint32_t tmem_cols,
                                  float* part, float* traj, int* err, const EmSpec& em, double* rrf, int smooth,
-                                 cudaStream_t st)
+                                 cudaStream_t st, int* max_ctas_per_sm)
 {
     TeamArgs a{count, Nt, TC, d, Ks, nkb, split, 3, tmem_cols, part, traj, err, em, rrf};
     switch (nm_bucket) {
-        case 1: return launch_team_nm1(nd_bucket, params, maps, a, smooth, st);
-        case 2: return launch_team_nm2(nd_bucket, params, maps, a, smooth, st);
-        case 4: return launch_team_nm4(nd_bucket, params, maps, a, smooth, st);
-        case 8: return launch_team_nm8(nd_bucket, params, maps, a, smooth, st);
-        case 10: return launch_team_nm10(nd_bucket, params, maps, a, smooth, st);
-        case 12: return launch_team_nm12(nd_bucket, params, maps, a, smooth, st);
-        case 16: return launch_team_nm16(nd_bucket, params, maps, a, smooth, st);
+        case 1: return launch_team_nm1(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
+        case 2: return launch_team_nm2(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
+        case 4: return launch_team_nm4(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
+        case 8: return launch_team_nm8(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
+        case 10: return launch_team_nm10(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
+        case 12: return launch_team_nm12(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
+        case 16: return launch_team_nm16(nd_bucket, params, maps, a, smooth, st, max_ctas_per_sm);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -549,7 +549,8 @@ __global__ void __launch_bounds__(team_threads(NM), NM > 8 ? 1 : 2)
 }
 
 template <int NM, int ND>
-cudaError_t launch_team_t(const void* params, const CUtensorMap* maps, const TeamArgs& a, int smooth, cudaStream_t st)
+cudaError_t launch_team_t(const void* params, const CUtensorMap* maps, const TeamArgs& a, int smooth, cudaStream_t st,
+                          int* max_ctas_per_sm)
 {
     const SwingParams<NM, ND>& p = *static_cast<const SwingParams<NM, ND>*>(params);
     auto kern = smooth ? simulate_team_kernel<NM, ND, true> : simulate_team_kernel<NM, ND, false>;
@@ -561,6 +562,10 @@ cudaError_t launch_team_t(const void* params, const CUtensorMap* maps, const Tea
     const int floor = 233472 / (512 / (int)a.tmem_cols + 1) - 1024 + 64;
     if (smem < floor) smem = floor;
     if (smem > TC_SMEM_DYN_MAX) return cudaErrorInvalidValue;
+    if (max_ctas_per_sm) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(max_ctas_per_sm, kern, team_threads(NM), smem);
+        if (e != cudaSuccess) return e;
+    }
     const int64_t groups = (a.count + TEAM_ROWS - 1) / TEAM_ROWS;
     kern<<<(unsigned)groups, team_threads(NM), smem, st>>>(p, maps[0], maps[1], maps[2], maps[3], a);
     return cudaGetLastError();
