@@ -523,8 +523,9 @@ int fmc_device_status(fmc_ctx* ctx, int* eq_iterations, int* kernel_error);
 
 
 /* ---- kernel choice of the fused path (no counterpart in the paper) -------- */
-#define FMC_KERNEL_AUTO 0        /* per sample for n <= 16, split with the tensor-core network sum above */
-#define FMC_KERNEL_PER_SAMPLE 1  /* one thread integrates a whole sample (n <= FMC_MAX_MACHINES_PLAIN) */
+#define FMC_KERNEL_AUTO 0        /* per sample for n <= 16 (few samples: by teams of warps, one per machine),
+                                    split with the tensor-core network sum above */
+#define FMC_KERNEL_PER_SAMPLE 1  /* one thread integrates a whole sample (n <= FMC_MAX_MACHINES_PLAIN), no teams */
 #define FMC_KERNEL_SPLIT 2       /* four warps share each sample's machines (any n up to FMC_MAX_MACHINES) */
 #define FMC_KERNEL_SPLIT_TC 3    /* the split kernel with each RK stage's network sums over the CTA's 128
                                     samples as one tcgen05 TF32x3 product (13 <= n <= FMC_MAX_MACHINES) */
@@ -553,7 +554,11 @@ int fmc_set_kernel_policy(fmc_ctx* ctx, int32_t policy);
  * large-system kernel keeps one CTA per SM.  max_ctas is a bound for a launch
  * that needs no more: one per SM becomes two where the 128-sample tiles are
  * more than the SMs, and the launches of a batch take one to three as they need
- * together (those of a server, two).  The rules are copied; count 0
+ * together (those of a server, two).  Few samples (up to 32 per SM) of up to 16
+ * machines that AUTO gives to teams of warps keep the teams' own shape; a rule for
+ * FMC_KERNEL_PER_SAMPLE keeps them off.  A context with a memory budget takes no
+ * teams and deals no tiles to a fixed number of CTAs (both need further memory).
+ * A rule's kernel that cannot take the scenario is ignored.  The rules are copied; count 0
  * clears them.  FMC_EINVAL on a malformed rule (empty range, kernel not an
  * FMC_KERNEL_* value, max_ctas outside 0..4, TC not 0 or a power of two in
  * 16..256).

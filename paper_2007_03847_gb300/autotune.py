@@ -1,12 +1,11 @@
 """Measured launch shapes of the fused path.
 
 For buckets of machine count, disturbance count and sample count, every
-candidate shape -- the kernel (per-sample up to 16 machines; split with the
-network sums on the FP32 pipes or on the tensor cores, the latter from 13
-machines), the resident CTAs per SM and the time chunk -- is timed with CUDA
-events on a seeded
-system of the bucket's largest size, and the fastest per machine-step becomes a
-launch rule (``fmc_set_launch_rules``).  The table is cached per GPU model and
+candidate shape -- the kernel (the library's own choice up to 16 machines:
+per-sample, or teams where samples are few; split with the network sums on the
+FP32 pipes or on the tensor cores, the latter from 13 machines), the resident
+CTAs per SM and the time chunk -- is timed with CUDA events on a seeded system of
+the bucket's largest size, and the fastest per machine-step becomes a launch rule (``fmc_set_launch_rules``).  The table is cached per GPU model and
 SM count under ``tuning/`` and applied to every new context on that GPU.
 
     python -m paper_2007_03847_gb300.autotune [--quick]
@@ -33,12 +32,12 @@ def table_path(name: str, sms: int) -> str:
 
 def candidates(n: int):
     """(kernel, max_ctas, TC) triples; 0 = the library's own choice."""
-    from . import KERNEL_PER_SAMPLE, KERNEL_SPLIT, KERNEL_SPLIT_TC
+    from . import KERNEL_AUTO, KERNEL_SPLIT, KERNEL_SPLIT_TC
     out = []
     if n <= 16:
         for mc in (0, 4, 2, 1):
             for tc in (0, 32, 16):
-                out.append((KERNEL_PER_SAMPLE, mc, tc))
+                out.append((KERNEL_AUTO, mc, tc))
         out.append((KERNEL_SPLIT, 0, 0))
         out.append((KERNEL_SPLIT, 0, 32))
     else:

@@ -1292,12 +1292,15 @@ static int64_t team_halves(int sms, int nm, int64_t count)
     return nm > 8 || (nm > 4 && 3 * g > 2 * (int64_t)sms) ? 2 * g : g;
 }
 
-static bool team_wanted(const fmc_ctx* ctx, int nm, int nmt, int32_t path, int n, int Nt, int64_t count,
-                        bool exclusive)
+static bool team_wanted(const fmc_ctx* ctx, const fmc_scenario* s, int nm, int nmt, int32_t path, int Nt,
+                        int64_t count, bool exclusive)
 {
     if (ctx->budget != 0 || !ctx->team) return false;
-    if (exclusive && ctx->kernel_policy != FMC_KERNEL_AUTO) return false;  // (the per-sample kernel by request)
-    return team_fits(ctx->sms, nm, nmt, path, n, Nt, count);
+    // (the per-sample kernel by request: a policy, or a launch rule that names it)
+    if (exclusive && ctx->kernel_policy != FMC_KERNEL_AUTO) return false;
+    const fmc_launch_rule* rule = find_rule(ctx, s, count);
+    if (rule && rule->kernel == FMC_KERNEL_PER_SAMPLE) return false;
+    return team_fits(ctx->sms, nm, nmt, path, s->n, Nt, count);
 }
 
 static int prepare(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s, int64_t k0, int64_t count, int32_t path,
@@ -1333,7 +1336,7 @@ static int prepare(fmc_ctx* ctx, Workspace& ws, const fmc_scenario* s, int64_t k
     P.path = path;
     P.k0 = k0;
     P.count = count;
-    P.team = team_wanted(ctx, P.nm, P.nmt, path, n, Nt, count, exclusive);
+    P.team = team_wanted(ctx, s, P.nm, P.nmt, path, Nt, count, exclusive);
     // FP64 Newton on the GPU; its angles come back to the host (one stream
     // synchronisation) to form the integrator's constants in the parameter block
     if ((rc = run_equilibrium_ws(ctx, ws, s, st))) return rc;
@@ -1929,7 +1932,7 @@ int fmc::reserve_workspace(fmc_ctx* ctx, const fmc_scenario* s, int32_t path, in
     P.exclusive = false;
     P.k0 = 0;
     P.count = count;
-    P.team = team_wanted(ctx, P.nm, P.nmt, path, s->n, Nt, count, false);
+    P.team = team_wanted(ctx, s, P.nm, P.nmt, path, Nt, count, false);
     return reserve(ctx, ctx->ws, P, false, path == FMC_PATH_PLAIN);
 }
 
