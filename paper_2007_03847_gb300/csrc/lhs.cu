@@ -4,6 +4,8 @@
 // bit-identically without sorting or communication.
 #include <cuda_bf16.h>
 
+#include <cmath>
+
 #include "fmc_common.cuh"
 #include "kernels.cuh"
 #include "lhs_feistel.cuh"
@@ -228,10 +230,13 @@ static cudaError_t launch_design_db(DesignArgs& a, int sms, cudaStream_t st)
     using T = DesignTile<PERM, DB>;
     constexpr bool TAB = PERM == PERM_TAB8 || PERM == PERM_TAB16;
     a.npos = (a.cols + T::DB - 1) / T::DB;
-    // rows per CTA: four CTAs per SM in all, but 2 .. 16 rows per table entry where
-    // there are tables (their filling is at most three Philox calls per entry, at
-    // most 3/8 for large designs), and whole list fillings (whole passes below one)
-    int64_t rows = (a.count * a.npos + 4 * sms - 1) / (4 * (int64_t)sms);
+    // rows per CTA: four CTAs per SM in all (eight where no walks need evening out: 2^20 x 8
+    // by simple random sampling 54 -> 45 us), but 2 .. 16 rows per table entry where there
+    // are tables (their filling is at most three Philox calls per entry, at most 3/8 for
+    // large designs), and whole list fillings (whole passes below one)
+    const bool even = PERM == PERM_NONE || (PERM == PERM_DIRECT && !a.walk);
+    const int64_t ctas = (even ? 8 : 4) * (int64_t)sms;
+    int64_t rows = (a.count * a.npos + ctas - 1) / ctas;
     const int64_t lo = TAB ? (int64_t)2 << a.h : 1, hi = TAB ? (int64_t)16 << a.h : (int64_t)1 << 14;
     rows = rows < lo ? lo : (rows > hi ? hi : rows);
     const int64_t unit = rows < T::SUB ? T::RPI : T::SUB;
@@ -257,19 +262,41 @@ static cudaError_t launch_design_t(DesignArgs& a, int sms, cudaStream_t st)
     return a.cols < 4 ? launch_design_db<PERM, OUT, 1>(a, sms, st) : launch_design_db<PERM, OUT, 4>(a, sms, st);
 }
 
-// The rule: tables while they fit (uint8 up to h = 8, 6 KB; uint16 up to h = 11,
-// 96 KB) and a block of rows at least 2^(h+1) long repays them; the rounds from
-// their definition above (more than 2^22 samples) and for short blocks of a large
-// design; no permutation for simple random sampling.
+// Whether tables pay for a design that fits them (h <= 11).  Blocks of 2^(h+1) rows at
+// least repay the filling; where they are fewer than four per SM, the threads' chains
+// decide: the filling and the lookups against the rounds by definition of fewer rows per
+// thread, in Philox calls (the uniform and the inverse CDF are worth three, a lookup half a
+// call), the definition a fifth off since its SMs are the fuller.  With and without tables
+// (us, launches in a row): 30000 rows of a 2^22-sample design, 20 columns, 47 and 15; 60000
+// rows of 2^18, 10 columns, 23 and 16; 65536 x 20 25 and 27.
+static bool tables_pay(const DesignArgs& a, int sms)
+{
+    const int64_t least = (int64_t)2 << a.h;
+    if (a.count < least) return false;
+    const int db = a.cols < 4 ? 1 : 4, threads = a.h <= 8 ? 256 : 512;
+    const int64_t npos = (a.cols + db - 1) / db, rows = (a.count * npos + 4 * sms - 1) / (4 * (int64_t)sms);
+    if (rows >= least) return true;
+    auto passes = [db](int64_t r, int t) { return (double)((r * db + t - 1) / t); };
+    // (a warp's lanes wait for the longest of their walks: the largest of 32 geometric numbers)
+    const double stay = (double)a.N / (double)((uint64_t)1 << (2 * a.h));
+    const double walk = a.walk ? 0.5 - std::log(32.0) / std::log1p(-stay) : 1.0;
+    const double table = kFeistelRounds * (double)((int64_t)db << a.h) / threads + 3.5 * passes(least, threads);
+    return 0.8 * (kFeistelRounds * walk + 3.0) * passes(rows, 256) >= table;
+}
+
+// The rule: tables while they fit (uint8 up to h = 8, 6 KB; uint16 up to h = 11, 96 KB) and
+// pay; the rounds from their definition above (more than 2^22 samples) and for short blocks
+// of a large design; no permutation for simple random sampling.
 template <int OUT>
 static cudaError_t launch_design(DesignArgs& a, int sms, cudaStream_t st)
 {
     if (a.count == 0) return cudaSuccess;
     if (a.strata_in) return launch_design_t<PERM_GIVEN, OUT>(a, sms, st);
     if (a.mode == FMC_SRS) return launch_design_t<PERM_NONE, OUT>(a, sms, st);
-    const bool rows_enough = a.count >= ((int64_t)2 << a.h);
-    if (a.h <= 8 && rows_enough) return launch_design_t<PERM_TAB8, OUT>(a, sms, st);
-    if (a.h <= 11 && rows_enough) return launch_design_t<PERM_TAB16, OUT>(a, sms, st);
+    if (a.h <= 11 && tables_pay(a, sms)) {
+        if (a.h <= 8) return launch_design_t<PERM_TAB8, OUT>(a, sms, st);
+        return launch_design_t<PERM_TAB16, OUT>(a, sms, st);
+    }
     return launch_design_t<PERM_DIRECT, OUT>(a, sms, st);
 }
 

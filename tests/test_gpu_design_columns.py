@@ -45,3 +45,16 @@ def test_given_strata(M):
     # every value lies in its own stratum
     p = torch.special.ndtr(zeta.double()).cpu().numpy().T * N
     assert np.all(np.abs(p - (s + 0.5)) <= 0.5 + 1e-6 * N)
+
+
+@pytest.mark.parametrize("N,M,k0,count", [
+    (1 << 22, 20, 70001, 30000), (1 << 22, 2, 5, 9000), (65536, 4, 0, 65536), (65536, 5, 65000, 536),
+    (262144, 4, 100000, 3000), (100000, 9, 0, 100000)])
+def test_where_tables_and_rounds_meet(orc, N, M, k0, count):
+    # blocks whose CTAs with tables would leave SMs idle take the rounds by definition
+    import torch
+    fmc = need_gpu()
+    st = torch.empty((M, count), dtype=torch.int32, device="cuda")
+    fmc.lhs_sample(11, N, M, k0=k0, count=count, strata=st)
+    _, ref = orc.lhs_sample(11, N, M, mode=orc.LHS, k0=k0, count=count, with_strata=True)
+    assert np.array_equal(st.cpu().numpy().view(np.uint32), ref)
