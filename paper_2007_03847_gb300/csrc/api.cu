@@ -2059,25 +2059,32 @@ constexpr int BATCH_STREAMS = 16;  // of a batch's launches at once
 // for.  The launches with the longest chains take it, as many of them as shorten the
 // batch's estimated time: the longest chain of a stream, the SM time of all launches over
 // the SMs, or the rounds of the teams.  Step times (us, GB300, fits of the measured
-// ones): per-sample 0.65 + 0.022 nm^2 alone, and 0.68 of that as SM time where two CTAs
-// share an SM; teams 0.45 + 0.075 nm, a fifth more where two share an SM and three
-// quarters more with 16 slots; split kernel 3 + 0.3 n.  The
-// SMs that teams hold: team_halves.
+// ones, three disturbances): per-sample 0.9 + 0.022 nm^2 alone (twice that with 16 slots,
+// 1.45 of it with smooth forcing, 0.27 more per disturbance with a normal per step), and
+// 0.68 of that as SM time where two CTAs share an SM; teams 0.55 + 0.1 nm, a fifth more
+// where two share an SM and 1.45 of it with 16 slots; split kernel 3 + 0.25 n.  The SMs
+// that teams hold: team_halves.  Teams beside per-sample CTAs on the same SMs slow both: 1.15
+// (four arms of 3316 samples of 5 machines, two of them by teams, 10.2 ms waited for and
+// 12.2 in a row, 9.5 and 9.4 without).
 // Measured (GB300, 1000 steps, teams by each launch alone -> now; in brackets without
 // teams, by the rules for single launches): 10 machines, four launches of 4800 samples
-// 6.17 -> 3.03 ms (3.60), sixteen of 1000 6.06 -> 3.15 (3.48), eight of 1000 3.05 -> 3.04
+// 6.17 -> 3.04 ms (3.60), sixteen of 1000 6.06 -> 3.16 (3.48), eight of 1000 3.05 -> 3.11
 // (3.20); 8 machines, four of 4800 4.44 -> 2.15 (2.74), four of 2400 1.71 either way
-// (2.34); 4 machines, eight of 2400 2.25 -> 1.38 (1.78); 12 machines, eight of 4800
+// (2.34); 4 machines, eight of 2400 2.25 -> 1.40 (1.78); 12 machines, eight of 4800
 // 12.7 -> 6.5 (11.8).
 static void batch_teams(int sms, int nstreams, std::vector<Prepared>& prep)
 {
     const size_t n = prep.size();
     auto tiles = [](const Prepared& P) { return (double)((P.count + TC_M - 1) / TC_M); };
     auto chain = [](const Prepared& P) {
-        return P.Nt * (P.nmt > 0 ? 3.0 + 0.3 * P.s.n : 0.65 + 0.022 * P.nm * P.nm);
+        if (P.nmt > 0) return P.Nt * (3.0 + 0.25 * P.s.n);
+        double step = (0.9 + 0.022 * P.nm * P.nm) * (P.nm > 12 ? 2.0 : 1.0);
+        if (P.s.forcing == FMC_FORCING_SMOOTH) step *= 1.45;
+        if (P.s.sampling == FMC_SRS_EM) step += 0.27 * P.s.d;
+        return P.Nt * step;
     };
     auto team_chain = [](const Prepared& P) {
-        return P.Nt * (0.45 + 0.075 * P.nm) * (P.nm > 12 ? 1.75 : P.nm > 8 ? 1.0 : 1.2);
+        return P.Nt * (0.55 + 0.1 * P.nm) * (P.nm > 12 ? 1.45 : P.nm > 8 ? 1.0 : 1.2);
     };
     auto room = [&](const Prepared& P) { return 0.5 * (double)team_halves(sms, P.nm, P.count); };
     std::vector<size_t> order;
@@ -2090,7 +2097,7 @@ static void batch_teams(int sms, int nstreams, std::vector<Prepared>& prep)
     size_t take = 0;
     for (size_t k = 0; k <= order.size(); ++k) {
         if (k > 0) team[order[k - 1]] = 1;
-        double area = 0, teams = 0, round = 0, longest = 0;
+        double area = 0, teams = 0, others = 0, round = 0, longest = 0;
         std::vector<double> stream((size_t)nstreams, 0.0);
         for (size_t i = 0; i < n; ++i) {
             const Prepared& P = prep[i];
@@ -2102,12 +2109,14 @@ static void batch_teams(int sms, int nstreams, std::vector<Prepared>& prep)
                 area += room(P) * c;
             } else {
                 area += tiles(P) * c * (P.nmt > 0 ? (P.H == 2 ? 0.6 : 1.0) : 0.68);
+                others += P.nmt > 0 ? 0.0 : tiles(P);
             }
             stream[i % (size_t)nstreams] += c;
         }
         for (double c : stream) longest = c > longest ? c : longest;
         double t = area / sms > longest ? area / sms : longest;
         if (std::ceil(teams / sms) * round > t) t = std::ceil(teams / sms) * round;
+        if (teams > 0 && others > 0 && teams + others > sms) t *= 1.15;
         if (k == 0 || t < 0.98 * best) {
             best = t;
             take = k;

@@ -89,8 +89,8 @@ def _teams(fmc, scs):
 @pytest.mark.parametrize("n,N,count,team", [
     (10, 1000, 1, True), (10, 4864, 1, True), (10, 4865, 1, False),
     (10, 2400, 2, True),      # 150 groups: an SM each
-    (10, 1000, 8, True),      # two rounds of teams are still shorter than one of tiles
-    (10, 1000, 16, False), (10, 4800, 4, False), (12, 4800, 8, False), (16, 4800, 16, False),
+    (12, 1000, 8, True),      # two rounds of teams are still shorter than one of tiles
+    (10, 1000, 8, False), (10, 1000, 16, False), (10, 4800, 4, False), (12, 4800, 8, False), (16, 4800, 16, False),
     (8, 1000, 8, True), (8, 2400, 4, True),   # two teams to an SM
     (8, 4800, 2, False), (4, 4800, 2, True), (8, 2400, 8, False), (4, 2400, 8, False), (1, 4800, 16, False)])
 def test_teams_while_the_batch_has_room(fmc, n, N, count, team):
@@ -105,6 +105,13 @@ def test_the_launch_that_the_batch_waits_for(fmc):
     assert _teams(fmc, [_sc(10, 1000), _sc(10, 60000)]) == [False, False]
     # launches of a stream follow one another
     assert sum(_teams(fmc, [_sc(10, 100)] * 33)) > 0
+
+
+def test_a_smooth_launch_is_the_longest(fmc):
+    # 13 to 16 machines: its step alone is twice a split kernel's
+    rules = [_sc(14, 2000, forcing=fs.FORCING_SMOOTH), _sc(20, 2000), _sc(20, 2000)]
+    assert _teams(fmc, rules) == [True, False, False]
+    assert _teams(fmc, [_sc(10, 2000, forcing=fs.FORCING_SMOOTH), _sc(50, 2000)]) == [False, False]
 
 
 def test_what_is_no_team_alone_is_none_in_a_batch(fmc):

@@ -47,7 +47,7 @@ def test_planned_batches(shapes):
 
 @pytest.mark.parametrize("shapes,teams", [
     ([(10, 3, 1000, 400), (10, 3, 4800, 60), (9, 2, 4800, 60), (10, 1, 4500, 60), (10, 2, 4800, 60)], 1),
-    ([(10, 2, 1000, 100)] * 8, 8), ([(10, 2, 700, 100)] * 17, 17), ([(8, 2, 4800, 70), (8, 1, 4700, 70)], 0),
+    ([(12, 2, 1000, 100)] * 8, 8), ([(10, 2, 700, 100)] * 17, 1), ([(8, 2, 4800, 70), (8, 1, 4700, 70)], 0),
     ([(4, 1, 4800, 90), (2, 1, 33, 900), (12, 3, 2000, 90)], 1)])
 @pytest.mark.parametrize("use_graph", [False, True])
 def test_batches_with_teams(shapes, teams, use_graph):
