@@ -162,291 +162,293 @@ __global__ void __launch_bounds__(FU_THREADS, SLICED ? 3 : 4)
     uint32_t cp = 0;  // contractions so far (parity of their barrier)
     bool failed = false;  // (sliced) a bounded wait gave up: the CTA takes no more items
     for (;;) {
-    // ---- the next work item: a tile, steps n_first .. n_last - 1 ----
-    int64_t tile = blockIdx.x;
-    int n_first = 0, n_last = a.Nt;
-    int64_t sl_tile = -1;  // (sliced) the tile's place among the sliced ones
-    uint32_t sl = 0;
-    if constexpr (SLICED) {
-        if (tid == 0) item_s = atomicAdd(a.ticket, 1u);
-        __syncthreads();
-        const int64_t item = item_s;
-        __syncthreads();
-        tile = item;
-        if (item >= a.whole) {
-            const int64_t nsl = a.ntiles - a.whole;
-            sl = nsl > 0 ? (uint32_t)((item - a.whole) / nsl) : (uint32_t)a.nslice;
-            if (sl >= (uint32_t)a.nslice) break;
-            sl_tile = (item - a.whole) % nsl;
-            tile = a.whole + sl_tile;
-            n_first = (int)sl * a.slice;
-            n_last = a.Nt - n_first < a.slice ? a.Nt : n_first + a.slice;
+        // ---- the next work item: a tile, steps n_first .. n_last - 1 ----
+        int64_t tile = blockIdx.x;
+        int n_first = 0, n_last = a.Nt;
+        int64_t sl_tile = -1;  // (sliced) the tile's place among the sliced ones
+        uint32_t sl = 0;
+        if constexpr (SLICED) {
+            if (tid == 0) item_s = atomicAdd(a.ticket, 1u);
+            __syncthreads();
+            const int64_t item = item_s;
+            __syncthreads();
+            tile = item;
+            if (item >= a.whole) {
+                const int64_t nsl = a.ntiles - a.whole;
+                sl = nsl > 0 ? (uint32_t)((item - a.whole) / nsl) : (uint32_t)a.nslice;
+                if (sl >= (uint32_t)a.nslice) break;
+                sl_tile = (item - a.whole) % nsl;
+                tile = a.whole + sl_tile;
+                n_first = (int)sl * a.slice;
+                n_last = a.Nt - n_first < a.slice ? a.Nt : n_first + a.slice;
+            }
         }
-    }
-    const int64_t row0 = tile * rows;
-    const int64_t srow = row0 + tid;
-    const bool active = srow < a.count;
-    if (!SMOOTH && a.keep_tiles > 0) r.a_policy = tile < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
+        const int64_t row0 = tile * rows;
+        const int64_t srow = row0 + tid;
+        const bool active = srow < a.count;
+        if (!SMOOTH && a.keep_tiles > 0)
+            r.a_policy = tile < a.keep_tiles ? l2_policy_evict_last() : l2_policy_evict_first();
 
-    float del[NM], w[NM], theta = 0.f;   // deviations from the equilibrium (see swing_step)
-    float x0[ND];
-#pragma unroll
-    for (int i = 0; i < NM; ++i) {
-        del[i] = 0.f;
-        w[i] = 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < ND; ++q) x0[q] = 0.f;
-    float racc = 0.f;  // sum over the grid of the squared centre-of-inertia speed
-
-    const int64_t trow = 2 * (int64_t)n;
-    float* traj = (a.traj != nullptr && active) ? a.traj + srow * (int64_t)(a.Nt + 1) * trow : nullptr;
-    float* part_tile = nullptr;
-    if constexpr (SLICED) part_tile = a.part ? a.part + tile * (a.Nt + 1) * S3 : nullptr;
-    if (SLICED && n_first > 0) {
-        // the state the tile's last slice left (from L2: this SM may hold older lines)
-        if (tid == 0) abort_flag = slice_wait(a.ticket + 1 + sl_tile, sl) ? 0 : 1;
-        __syncthreads();
-        if (abort_flag) {
-            if (tid == 0) atomicExch(a.err, DEV_TIMEOUT_MMA);
-            break;
-        }
-        const float* st = a.state + sl_tile * (int64_t)fu_state(NM, ND) * rows + tid;
+        float del[NM], w[NM], theta = 0.f;   // deviations from the equilibrium (see swing_step)
+        float x0[ND];
 #pragma unroll
         for (int i = 0; i < NM; ++i) {
-            del[i] = __ldcg(st + i * rows);
-            w[i] = __ldcg(st + (NM + i) * rows);
+            del[i] = 0.f;
+            w[i] = 0.f;
         }
-        theta = __ldcg(st + 2 * NM * rows);
-        racc = __ldcg(st + (2 * NM + 1) * rows);
 #pragma unroll
-        for (int q = 0; q < ND; ++q) x0[q] = __ldcg(st + (2 * NM + 2 + q) * rows);
-    } else {
-        if (traj) {
-#pragma unroll
-            for (int i = 0; i < NM; ++i)
-                if (i < n) {
-                    traj[i] = p.dst[i];
-                    traj[n + i] = 0.f;
-                }
-        }
-        // time 0: every sample sits at the (rounded) shift, so both sums are zero.  (The
-        // pointer is formed here in the unsliced form and before the branch in the sliced
-        // one: the other way round the kernels of 10 machines and 4 disturbances spill 176
-        // and 224 bytes instead of 64 and 12, and 2^20 samples take 427 ms instead of 387.)
-        if constexpr (!SLICED) part_tile = a.part ? a.part + tile * (a.Nt + 1) * S3 : nullptr;
-        if (part_tile)
-            for (int v = tid; v < S3; v += rows) part_tile[v] = 0.f;
-    }
+        for (int q = 0; q < ND; ++q) x0[q] = 0.f;
+        float racc = 0.f;  // sum over the grid of the squared centre-of-inertia speed
 
-    float f0[ND];  // the smooth form's forcing at the chunk's first grid time
-#pragma unroll
-    for (int q = 0; q < ND; ++q) f0[q] = 0.f;
-    for (int n0 = SMOOTH ? -TC : n_first; n0 < (SLICED ? n_last : a.Nt); n0 += TC) {
-        // ---- tensor cores: dW of this chunk into TMEM ----
-        if (!em) {
-        tc_fence_before();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            tc_fence_after();
-            // item j: disturbance wj, K block kb; loads run up to ns - 1 items ahead
-            // of the MMAs (a stage is refilled once its MMAs completed)
-            auto load_item = [&](int j) {
-                const int wj = j / a.nkb, kb = j - wj * a.nkb;
-                return ring_load(r, g + (uint32_t)j, &mAh, &mAl, &mBh, &mBl, wj * a.Ks + kb * TC_BK, (int)row0,
-                                 kb * TC_BK, SMOOTH ? 2 * n0 + 1 : n0);
-            };
-            bool ok = true;
-            int issued = 0;
-            for (; issued < J && issued + 1 < (int)r.ns && ok; ++issued) ok = load_item(issued);
-            for (int j = 0; j < J && ok; ++j) {
-                if (issued < J) {
-                    ok = load_item(issued);
-                    ++issued;
-                    if (!ok) break;
-                }
-                const int wj = j / a.nkb, kb = j - wj * a.nkb;
-                ok = ring_mma(r, g + (uint32_t)j, tmem + (uint32_t)(wj * CW), idesc, kb == 0);
+        const int64_t trow = 2 * (int64_t)n;
+        float* traj = (a.traj != nullptr && active) ? a.traj + srow * (int64_t)(a.Nt + 1) * trow : nullptr;
+        float* part_tile = nullptr;
+        if constexpr (SLICED) part_tile = a.part ? a.part + tile * (a.Nt + 1) * S3 : nullptr;
+        if (SLICED && n_first > 0) {
+            // the state the tile's last slice left (from L2: this SM may hold older lines)
+            if (tid == 0) abort_flag = slice_wait(a.ticket + 1 + sl_tile, sl) ? 0 : 1;
+            __syncthreads();
+            if (abort_flag) {
+                if (tid == 0) atomicExch(a.err, DEV_TIMEOUT_MMA);
+                break;
             }
-            g += (uint32_t)J;
-            if (ok) {
-                umma_commit(done);
-            } else {
-                abort_flag = 1;
-                atomicExch(a.err, DEV_TIMEOUT_TMA);
+            const float* st = a.state + sl_tile * (int64_t)fu_state(NM, ND) * rows + tid;
+#pragma unroll
+            for (int i = 0; i < NM; ++i) {
+                del[i] = __ldcg(st + i * rows);
+                w[i] = __ldcg(st + (NM + i) * rows);
             }
-        }
-        __syncthreads();
-        bool ok = (abort_flag == 0);
-        if (ok && !mbar_wait(done, cp & 1u)) {
-            ok = false;
-            atomicExch(a.err, DEV_TIMEOUT_MMA);
-        }
-        ++cp;
-        if (!__syncthreads_and(ok)) {
-            failed = true;
-            break;
-        }
-        tc_fence_after();
-        }
-
-        if constexpr (SMOOTH) {
-            if (n0 < 0) {
-                // f(0): the last column of the contraction over the rows up to 0
+            theta = __ldcg(st + 2 * NM * rows);
+            racc = __ldcg(st + (2 * NM + 1) * rows);
 #pragma unroll
-                for (int q = 0; q < ND; ++q)
-                    if (q < d) f0[q] = tmem_ld1(lane_addr + (uint32_t)(q * CW + CW - 1));
-                tmem_ld_wait();
-                continue;
-            }
-        }
-        const int steps = SLICED ? ((n_last - n0) < TC ? (n_last - n0) : TC) : ((a.Nt - n0) < TC ? (a.Nt - n0) : TC);
-        // ---- disturbance paths of this chunk into TMEM (each warp its own lanes) ----
-        if constexpr (!SMOOTH)
-            disturbance_chunk<ND, ND, true>(lane_addr, TC, steps, n0, d, -1, x0, p.ou_a, p.ou_s, p.ito, p.dt, a.em,
-                                            (uint32_t)(a.em.k0 + srow));
-
-        // ---- FP32 pipes: integrate this chunk ----
-        for (int s = 0; s < steps; ++s) {
-            if constexpr (SMOOTH) {
-                // the forcing at t_n + dt/2 and t_{n+1}; the stage values of the
-                // disturbances' random ODE feed the swing stages
-                float fh[ND], f1[ND], xst[4][ND];
-#pragma unroll
-                for (int q = 0; q < ND; ++q) {
-                    fh[q] = 0.f;
-                    f1[q] = 0.f;
-                }
-#pragma unroll
-                for (int q = 0; q < ND; ++q)
-                    if (q < d) {
-                        fh[q] = tmem_ld1(lane_addr + (uint32_t)(q * CW + 2 * s));
-                        f1[q] = tmem_ld1(lane_addr + (uint32_t)(q * CW + 2 * s + 1));
-                    }
-                tmem_ld_wait();
-                smooth_stages<NM, ND>(p, n0 + s, x0, f0, fh, f1, xst);
-#pragma unroll
-                for (int q = 0; q < ND; ++q) f0[q] = f1[q];
-                swing_step_staged<NM, ND>(p, del, w, theta, xst);
-            } else {
-                float x1[ND];
-#pragma unroll
-                for (int q = 0; q < ND; ++q) x1[q] = 0.f;
-#pragma unroll
-                for (int q = 0; q < ND; ++q)
-                    if (q < d) x1[q] = tmem_ld1(lane_addr + (uint32_t)(q * TC + s));
-                tmem_ld_wait();
-                // the event slot: 0 before the event's grid step, 1 from it
-#pragma unroll
-                for (int q = 0; q < ND; ++q)
-                    if (q == p.ev_slot) {
-                        x0[q] = (n0 + s >= p.ev_step) ? 1.f : 0.f;
-                        x1[q] = x0[q];
-                    }
-                swing_step<NM, ND, (NM <= 10)>(p, del, w, theta, x0, x1);
-#pragma unroll
-                for (int q = 0; q < ND; ++q) x0[q] = x1[q];
-            }
-            if (a.rrf) {
-                const float cs = coi_speed<NM, ND>(p, w);
-                racc = fmaf(cs, cs, racc);
-            }
-
-            const int tn = n0 + s + 1;  // grid index of the new state
+            for (int q = 0; q < ND; ++q) x0[q] = __ldcg(st + (2 * NM + 2 + q) * rows);
+        } else {
             if (traj) {
-                float* o = traj + (int64_t)tn * trow;
 #pragma unroll
                 for (int i = 0; i < NM; ++i)
                     if (i < n) {
-                        o[i] = (theta + del[i]) + p.dst[i];
-                        o[n + i] = w[i];
+                        traj[i] = p.dst[i];
+                        traj[n + i] = 0.f;
                     }
             }
-            // ---- moments: transpose the warp's states and sum per state ----
-            // (row r holds lane r's sample: angles in columns 0..NM-1, speeds in
-            // NM..2NM-1; rows past the tile's last sample hold whatever those
-            // lanes integrated, and column_sums reads only the first na_warp rows)
-            float* myrow = wbuf + lane * WROW;
+            // time 0: every sample sits at the (rounded) shift, so both sums are zero.  (The
+            // pointer is formed here in the unsliced form and before the branch in the sliced
+            // one: the other way round the kernels of 10 machines and 4 disturbances spill 176
+            // and 224 bytes instead of 64 and 12, and 2^20 samples take 427 ms instead of 387.)
+            if constexpr (!SLICED) part_tile = a.part ? a.part + tile * (a.Nt + 1) * S3 : nullptr;
+            if (part_tile)
+                for (int v = tid; v < S3; v += rows) part_tile[v] = 0.f;
+        }
+
+        float f0[ND];  // the smooth form's forcing at the chunk's first grid time
 #pragma unroll
-            for (int i = 0; i < NM; ++i) {
-                myrow[i] = theta + del[i];
-                myrow[NM + i] = w[i];
-            }
-            __syncwarp();
-            const int ms = s % FU_MS;
-            if (lane < S) {
-                // the warp's reference value, sum about it and squared deviations, per
-                // state (lane j: state j, its column of the transpose buffer)
-                const int mcol = lane < n ? lane : NM + lane - n;
-                const int64_t left = a.count - (srow - lane);
-                const int na_warp = left <= 0 ? 0 : (left >= 32 ? 32 : (int)left);
-                float rf, dv, m2;
-                column_sums(wbuf + mcol, WROW, na_warp, &rf, &dv, &m2);
-                float* slot = msum + (ms * warps + warp) * MSLOT;
-                slot[lane] = rf;
-                slot[S + lane] = dv;
-                slot[2 * S + lane] = m2;
-            }
-            __syncwarp();
-            if (ms == FU_MS - 1 || s == steps - 1) {
-                asm volatile("bar.sync 1, %0;" ::"r"(rows) : "memory");
-                const int nst = ms + 1;
-                const int tn0 = tn - ms;
-                // samples of this tile (the last tile may be partly empty)
-                const int64_t left = a.count - row0;
-                const int n_tile = left <= 0 ? 0 : (left >= rows ? rows : (int)left);
-                for (int e = tid; e < nst * S; e += rows) {
-                    const int sl = e / S, j = e - sl * S;  // step slot, state
-                    const float* m = msum + sl * warps * MSLOT + j;
-                    // the tile's triple: reference (warp 0's), sum about it, squared deviations
-                    float c, dv, m2;
-                    combine_groups(m, m + S, m + 2 * S, MSLOT, left, warps, &c, &dv, &m2);
-                    if (part_tile) {
-                        float* o = part_tile + (int64_t)(tn0 + sl) * S3;
-                        o[j] = c;
-                        o[S + j] = dv;
-                        o[2 * S + j] = m2;
-                    } else if (n_tile > 0) {
-                        // the tile's S1 and S2 (= M2 + S1^2 / n) about the shift, in FP64
-                        const int64_t row = (int64_t)(tn0 + sl) * S;
-                        const double s1 = fma((double)n_tile, (double)c, (double)dv);
-                        atomicAdd(a.S1 + row + j, s1);
-                        atomicAdd(a.S2 + row + j, (double)m2 + s1 * s1 / (double)n_tile);
+        for (int q = 0; q < ND; ++q) f0[q] = 0.f;
+        for (int n0 = SMOOTH ? -TC : n_first; n0 < (SLICED ? n_last : a.Nt); n0 += TC) {
+            // ---- tensor cores: dW of this chunk into TMEM ----
+            if (!em) {
+                tc_fence_before();
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncthreads();
+                if (tid == 0) {
+                    tc_fence_after();
+                    // item j: disturbance wj, K block kb; loads run up to ns - 1 items ahead
+                    // of the MMAs (a stage is refilled once its MMAs completed)
+                    auto load_item = [&](int j) {
+                        const int wj = j / a.nkb, kb = j - wj * a.nkb;
+                        return ring_load(r, g + (uint32_t)j, &mAh, &mAl, &mBh, &mBl, wj * a.Ks + kb * TC_BK, (int)row0,
+                                         kb * TC_BK, SMOOTH ? 2 * n0 + 1 : n0);
+                    };
+                    bool ok = true;
+                    int issued = 0;
+                    for (; issued < J && issued + 1 < (int)r.ns && ok; ++issued) ok = load_item(issued);
+                    for (int j = 0; j < J && ok; ++j) {
+                        if (issued < J) {
+                            ok = load_item(issued);
+                            ++issued;
+                            if (!ok) break;
+                        }
+                        const int wj = j / a.nkb, kb = j - wj * a.nkb;
+                        ok = ring_mma(r, g + (uint32_t)j, tmem + (uint32_t)(wj * CW), idesc, kb == 0);
+                    }
+                    g += (uint32_t)J;
+                    if (ok) {
+                        umma_commit(done);
+                    } else {
+                        abort_flag = 1;
+                        atomicExch(a.err, DEV_TIMEOUT_TMA);
                     }
                 }
-                asm volatile("bar.sync 1, %0;" ::"r"(rows) : "memory");
+                __syncthreads();
+                bool ok = (abort_flag == 0);
+                if (ok && !mbar_wait(done, cp & 1u)) {
+                    ok = false;
+                    atomicExch(a.err, DEV_TIMEOUT_MMA);
+                }
+                ++cp;
+                if (!__syncthreads_and(ok)) {
+                    failed = true;
+                    break;
+                }
+                tc_fence_after();
+            }
+
+            if constexpr (SMOOTH) {
+                if (n0 < 0) {
+                    // f(0): the last column of the contraction over the rows up to 0
+#pragma unroll
+                    for (int q = 0; q < ND; ++q)
+                        if (q < d) f0[q] = tmem_ld1(lane_addr + (uint32_t)(q * CW + CW - 1));
+                    tmem_ld_wait();
+                    continue;
+                }
+            }
+            const int steps =
+                SLICED ? ((n_last - n0) < TC ? (n_last - n0) : TC) : ((a.Nt - n0) < TC ? (a.Nt - n0) : TC);
+            // ---- disturbance paths of this chunk into TMEM (each warp its own lanes) ----
+            if constexpr (!SMOOTH)
+                disturbance_chunk<ND, ND, true>(lane_addr, TC, steps, n0, d, -1, x0, p.ou_a, p.ou_s, p.ito, p.dt, a.em,
+                                                (uint32_t)(a.em.k0 + srow));
+
+            // ---- FP32 pipes: integrate this chunk ----
+            for (int s = 0; s < steps; ++s) {
+                if constexpr (SMOOTH) {
+                    // the forcing at t_n + dt/2 and t_{n+1}; the stage values of the
+                    // disturbances' random ODE feed the swing stages
+                    float fh[ND], f1[ND], xst[4][ND];
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) {
+                        fh[q] = 0.f;
+                        f1[q] = 0.f;
+                    }
+#pragma unroll
+                    for (int q = 0; q < ND; ++q)
+                        if (q < d) {
+                            fh[q] = tmem_ld1(lane_addr + (uint32_t)(q * CW + 2 * s));
+                            f1[q] = tmem_ld1(lane_addr + (uint32_t)(q * CW + 2 * s + 1));
+                        }
+                    tmem_ld_wait();
+                    smooth_stages<NM, ND>(p, n0 + s, x0, f0, fh, f1, xst);
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) f0[q] = f1[q];
+                    swing_step_staged<NM, ND>(p, del, w, theta, xst);
+                } else {
+                    float x1[ND];
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) x1[q] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < ND; ++q)
+                        if (q < d) x1[q] = tmem_ld1(lane_addr + (uint32_t)(q * TC + s));
+                    tmem_ld_wait();
+                    // the event slot: 0 before the event's grid step, 1 from it
+#pragma unroll
+                    for (int q = 0; q < ND; ++q)
+                        if (q == p.ev_slot) {
+                            x0[q] = (n0 + s >= p.ev_step) ? 1.f : 0.f;
+                            x1[q] = x0[q];
+                        }
+                    swing_step<NM, ND, (NM <= 10)>(p, del, w, theta, x0, x1);
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) x0[q] = x1[q];
+                }
+                if (a.rrf) {
+                    const float cs = coi_speed<NM, ND>(p, w);
+                    racc = fmaf(cs, cs, racc);
+                }
+
+                const int tn = n0 + s + 1;  // grid index of the new state
+                if (traj) {
+                    float* o = traj + (int64_t)tn * trow;
+#pragma unroll
+                    for (int i = 0; i < NM; ++i)
+                        if (i < n) {
+                            o[i] = (theta + del[i]) + p.dst[i];
+                            o[n + i] = w[i];
+                        }
+                }
+                // ---- moments: transpose the warp's states and sum per state ----
+                // (row r holds lane r's sample: angles in columns 0..NM-1, speeds in
+                // NM..2NM-1; rows past the tile's last sample hold whatever those
+                // lanes integrated, and column_sums reads only the first na_warp rows)
+                float* myrow = wbuf + lane * WROW;
+#pragma unroll
+                for (int i = 0; i < NM; ++i) {
+                    myrow[i] = theta + del[i];
+                    myrow[NM + i] = w[i];
+                }
+                __syncwarp();
+                const int ms = s % FU_MS;
+                if (lane < S) {
+                    // the warp's reference value, sum about it and squared deviations, per
+                    // state (lane j: state j, its column of the transpose buffer)
+                    const int mcol = lane < n ? lane : NM + lane - n;
+                    const int64_t left = a.count - (srow - lane);
+                    const int na_warp = left <= 0 ? 0 : (left >= 32 ? 32 : (int)left);
+                    float rf, dv, m2;
+                    column_sums(wbuf + mcol, WROW, na_warp, &rf, &dv, &m2);
+                    float* slot = msum + (ms * warps + warp) * MSLOT;
+                    slot[lane] = rf;
+                    slot[S + lane] = dv;
+                    slot[2 * S + lane] = m2;
+                }
+                __syncwarp();
+                if (ms == FU_MS - 1 || s == steps - 1) {
+                    asm volatile("bar.sync 1, %0;" ::"r"(rows) : "memory");
+                    const int nst = ms + 1;
+                    const int tn0 = tn - ms;
+                    // samples of this tile (the last tile may be partly empty)
+                    const int64_t left = a.count - row0;
+                    const int n_tile = left <= 0 ? 0 : (left >= rows ? rows : (int)left);
+                    for (int e = tid; e < nst * S; e += rows) {
+                        const int sl = e / S, j = e - sl * S;  // step slot, state
+                        const float* m = msum + sl * warps * MSLOT + j;
+                        // the tile's triple: reference (warp 0's), sum about it, squared deviations
+                        float c, dv, m2;
+                        combine_groups(m, m + S, m + 2 * S, MSLOT, left, warps, &c, &dv, &m2);
+                        if (part_tile) {
+                            float* o = part_tile + (int64_t)(tn0 + sl) * S3;
+                            o[j] = c;
+                            o[S + j] = dv;
+                            o[2 * S + j] = m2;
+                        } else if (n_tile > 0) {
+                            // the tile's S1 and S2 (= M2 + S1^2 / n) about the shift, in FP64
+                            const int64_t row = (int64_t)(tn0 + sl) * S;
+                            const double s1 = fma((double)n_tile, (double)c, (double)dv);
+                            atomicAdd(a.S1 + row + j, s1);
+                            atomicAdd(a.S2 + row + j, (double)m2 + s1 * s1 / (double)n_tile);
+                        }
+                    }
+                    asm volatile("bar.sync 1, %0;" ::"r"(rows) : "memory");
+                }
             }
         }
-    }
-    if (SLICED && n_last < a.Nt && !failed) {
-        // the tile goes on in a later item, on whichever CTA takes it
-        float* st = a.state + sl_tile * (int64_t)fu_state(NM, ND) * rows + tid;
+        if (SLICED && n_last < a.Nt && !failed) {
+            // the tile goes on in a later item, on whichever CTA takes it
+            float* st = a.state + sl_tile * (int64_t)fu_state(NM, ND) * rows + tid;
 #pragma unroll
-        for (int i = 0; i < NM; ++i) {
-            st[i * rows] = del[i];
-            st[(NM + i) * rows] = w[i];
-        }
-        st[2 * NM * rows] = theta;
-        st[(2 * NM + 1) * rows] = racc;
+            for (int i = 0; i < NM; ++i) {
+                st[i * rows] = del[i];
+                st[(NM + i) * rows] = w[i];
+            }
+            st[2 * NM * rows] = theta;
+            st[(2 * NM + 1) * rows] = racc;
 #pragma unroll
-        for (int q = 0; q < ND; ++q) st[(2 * NM + 2 + q) * rows] = x0[q];
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) atomicExch(a.ticket + 1 + sl_tile, sl + 1u);
-        continue;
-    }
-    if (a.rrf) rrf_accumulate(active ? sqrtf(racc / (float)a.Nt) : 0.f, a.rrf);
-    if (!em && tile < a.keep_tiles) {
-        // the tile's design rows back to normal L2 priority
-        const int64_t left = a.count - row0;
-        const int64_t bytes = (left < rows ? left : rows) * a.zeta_row_bytes;
-        for (int64_t o = (int64_t)tid * 128; o < bytes; o += (int64_t)rows * 128) {
-            l2_priority_normal(a.zeta_hi + row0 * a.zeta_row_bytes + o);
-            if (a.split) l2_priority_normal(a.zeta_lo + row0 * a.zeta_row_bytes + o);
+            for (int q = 0; q < ND; ++q) st[(2 * NM + 2 + q) * rows] = x0[q];
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) atomicExch(a.ticket + 1 + sl_tile, sl + 1u);
+            continue;
         }
-    }
-    if (!SLICED || failed) break;
+        if (a.rrf) rrf_accumulate(active ? sqrtf(racc / (float)a.Nt) : 0.f, a.rrf);
+        if (!em && tile < a.keep_tiles) {
+            // the tile's design rows back to normal L2 priority
+            const int64_t left = a.count - row0;
+            const int64_t bytes = (left < rows ? left : rows) * a.zeta_row_bytes;
+            for (int64_t o = (int64_t)tid * 128; o < bytes; o += (int64_t)rows * 128) {
+                l2_priority_normal(a.zeta_hi + row0 * a.zeta_row_bytes + o);
+                if (a.split) l2_priority_normal(a.zeta_lo + row0 * a.zeta_row_bytes + o);
+            }
+        }
+        if (!SLICED || failed) break;
     }
     tc_fence_before();
     __syncthreads();
